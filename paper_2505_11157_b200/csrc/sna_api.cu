@@ -403,9 +403,9 @@ sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float*
     if (!q || !k || !v || !out) { set_error("q, k, v and out must not be NULL"); return SNA_ERR_INVALID_ARG; }
     if (!all_aligned(q, k, v, out) || (reinterpret_cast<uintptr_t>(lse) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     cudaError_t e;
-    if (lse != nullptr && sna::dense2_global_supported(plan->dev, C)) {
+    if (sna::dense2_global_supported(plan->dev, C)) {
         // every window is a whole ring (a global plan, or a cutoff that reaches every point): the dense kernel alone
-        // produces the final out and lse
+        // produces the final out and, if asked for, lse (64x128, N = 4, without lse: 5.44 ms on the generic kernel, 0.25 ms here)
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
     } else if (plan->is_global) {
         e = sna::launch_forward_generic(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);

@@ -66,8 +66,8 @@ cudaError_t launch_forward_mma(const DevPlan& p, const float* q, const float* k,
 // Dense (tcgen05) kernels (sna_kernels_dense2.cu: TMA loads, warp-specialised, operands and accumulators in TMEM) for
 // the windows in the plan's dense lists: whole input rings, and wide banded windows as masked blocks.  The forward kernel
 // writes the partial result (normalised out, lse) of the output latitudes in p.dense_rows and launch_forward_mma_band
-// continues from it with the narrower windows; both need lse != null.  dense2_path_supported tells whether the pair may
-// be used for this problem.
+// continues from it with the narrower windows; both need lse != null then (alone, for a problem of whole rings only, the
+// dense kernel does not).  dense2_path_supported tells whether the pair may be used for this problem.
 cudaError_t dense2_prepare_device();   // once per device: opt in to the kernels' shared-memory sizes
 bool dense2_path_supported(const DevPlan& p, int C);
 cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t stream);

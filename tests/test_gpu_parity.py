@@ -276,6 +276,22 @@ def test_global_plan_against_oracle(shape, reuse):
         assert not dk.reshape(wl.N, nlat_in, -1)[:, 0].any() and not dv.reshape(wl.N, nlat_in, -1)[:, 0].any()
 
 
+@pytest.mark.parametrize("nlat, nlon", [(6, 32), (9, 128), (5, 129), (12, 80)])
+def test_global_forward_without_lse(nlat, nlon):
+    """The dense forward kernel alone serves a global plan with and without an lse buffer: same values, bit for bit."""
+    wl = small_workload("global_no_lse", nlat, nlon, nlat, nlon, EQ, EQ, math.pi, 1, 2, 32, 61)
+    q, k, v, _ = make_inputs(wl)
+    ref = orc.forward(_geometry(wl), q, k, v)
+    with sna.Plan(nlat, nlon, nlat, nlon, EQ, EQ, global_attention=True) as plan:
+        qd, kd, vd = _dev(q, k, v)
+        out = plan.forward(qd, kd, vd)
+        with_lse, _ = plan.forward(qd, kd, vd, return_lse=True)
+        torch.cuda.synchronize()
+        sna.sna_plan_check(plan.handle)
+    assert torch.equal(out, with_lse)
+    assert nerr(out.cpu().numpy().reshape(ref.shape), ref) <= FWD_TOL
+
+
 def test_a_bounded_wait_that_runs_out_is_reported_once_and_the_plan_stays_usable():
     """The failure path of the bounded waits, without faulting or hanging anything: a probe kernel waits 1000 polls
     on a barrier nobody arrives on, gives up, records it; the check reports it once; compute calls still work."""
