@@ -42,6 +42,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 struct sna_plan {
     sna::HostPlan host;
     sna::DevPlan dev{};
+    std::vector<int32_t> band_lengths[4];      // of the four band streams (DevBand::lengths)
     int device = 0;
     std::vector<int> zero_rings;       // input rings of quadrature weight zero (no kernel of a global plan visits them)
     bool is_global = false;            // created by sna_plan_create_global: no column streams, dense kernels only
@@ -79,6 +80,9 @@ bool all_aligned(P... ptrs) { return (aligned16(ptrs) && ...); }
 
 size_t stats_elems(const sna_plan_t* plan, int B, int H) {
     return (size_t)B * H * plan->host.nlat_out * plan->host.nlon_out;
+}
+bool tf32_supported(const sna_plan_t* plan, int C) {
+    return (C == 16 || C == 32 || C == 64) && plan->host.nlon_out >= 32 && sna::band_path_supported(plan->dev, C);
 }
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -146,9 +150,8 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     std::vector<float> log2_omega(hp.nlat_in);
     for (int h = 0; h < hp.nlat_in; ++h) log2_omega[h] = (float)std::log2(hp.omega[h]);
 
-    sna::Stream fwd_stream, t_stream, fwdb_stream, tb_stream;
+    sna::BandStream bands[4];          // forward and transposed, each with all windows and without the dense kernels' ones
     sna::DenseLists dense, t_dense;
-    std::vector<int32_t> grp_order, t_grp_order, grpb_order, tb_grp_order;
 #ifdef SNA_PROF
     const int32_t zero_status[512] = {};   // room for the per-role profile of a -DSNA_PROF build
 #else
@@ -165,54 +168,20 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
         // rows with the longest lists first: the dense kernels run one block per SM, so the long tiles must not start last
         std::stable_sort(dense.rows.begin(), dense.rows.end(), [&](int a, int b) { return dense.ptr[a + 1] - dense.ptr[a] > dense.ptr[b + 1] - dense.ptr[b]; });
         std::stable_sort(t_dense.rows.begin(), t_dense.rows.end(), [&](int a, int b) { return t_dense.ptr[a + 1] - t_dense.ptr[a] > t_dense.ptr[b + 1] - t_dense.ptr[b]; });
-        if (global) {
-            // every window is a whole ring: the dense kernels do all the work, so the column streams (which would list
-            // every pair of the dense problem) are not built; they stay empty and the band kernels are never launched
-            const size_t g_out = (hp.nlat_out + sna::TILE_LAT - 1) / sna::TILE_LAT, g_in = (hp.nlat_in + sna::TILE_LAT - 1) / sna::TILE_LAT;
-            fwd_stream.chunk_ptr.assign(g_out + 1, 0);
-            fwdb_stream.chunk_ptr.assign(g_out + 1, 0);
-            t_stream.chunk_ptr.assign(g_in + 1, 0);
-            tb_stream.chunk_ptr.assign(g_in + 1, 0);
-            t_consecutive = true;
-            grp_order.resize(g_out);
-            std::iota(grp_order.begin(), grp_order.end(), 0);
-            grpb_order = grp_order;
-        } else {
-        sna::build_forward_stream(hp, fwd_stream);
-        t_consecutive = sna::build_transposed_stream(hp, t_stream);
-        sna::build_forward_stream(hp, fwdb_stream, dense_min_width);
-        grpb_order.resize(fwdb_stream.chunk_ptr.size() - 1);
-        std::iota(grpb_order.begin(), grpb_order.end(), 0);
-        std::stable_sort(grpb_order.begin(), grpb_order.end(), [&](int a, int b) {
-            return fwdb_stream.chunk_ptr[a + 1] - fwdb_stream.chunk_ptr[a] > fwdb_stream.chunk_ptr[b + 1] - fwdb_stream.chunk_ptr[b];
-        });
-        // heavy-first orders of the ring groups (by stream length; for the transposed stream summed over residues)
-        grp_order.resize(fwd_stream.chunk_ptr.size() - 1);
-        std::iota(grp_order.begin(), grp_order.end(), 0);
-        std::stable_sort(grp_order.begin(), grp_order.end(), [&](int a, int b) {
-            return fwd_stream.chunk_ptr[a + 1] - fwd_stream.chunk_ptr[a] > fwd_stream.chunk_ptr[b + 1] - fwd_stream.chunk_ptr[b];
-        });
-        sna::build_transposed_stream(hp, tb_stream, dense_min_width);
+        // (a global plan's windows are all whole rings: the dense kernels do all the work and no band stream, which would
+        // list every pair of the dense problem, is built)
+        if (!global) {
+            sna::build_forward_band(hp, bands[0]);
+            sna::build_forward_band(hp, bands[1], dense_min_width);
+            t_consecutive = sna::build_transposed_band(hp, bands[2]);
+            sna::build_transposed_band(hp, bands[3], dense_min_width);
         }
-        const int rows_per_group = t_consecutive ? 1 : hp.ps;
-        tb_grp_order.resize((tb_stream.chunk_ptr.size() - 1) / rows_per_group);
-        std::iota(tb_grp_order.begin(), tb_grp_order.end(), 0);
-        std::stable_sort(tb_grp_order.begin(), tb_grp_order.end(), [&](int a, int b) {
-            return tb_stream.chunk_ptr[(a + 1) * rows_per_group] - tb_stream.chunk_ptr[a * rows_per_group] >
-                   tb_stream.chunk_ptr[(b + 1) * rows_per_group] - tb_stream.chunk_ptr[b * rows_per_group];
-        });
-        t_grp_order.resize((t_stream.chunk_ptr.size() - 1) / rows_per_group);
-        std::iota(t_grp_order.begin(), t_grp_order.end(), 0);
-        std::stable_sort(t_grp_order.begin(), t_grp_order.end(), [&](int a, int b) {
-            return t_stream.chunk_ptr[(a + 1) * rows_per_group] - t_stream.chunk_ptr[a * rows_per_group] >
-                   t_stream.chunk_ptr[(b + 1) * rows_per_group] - t_stream.chunk_ptr[b * rows_per_group];
-        });
     } catch (const std::bad_alloc&) {
         delete plan;
-        set_error("out of host memory while building the column streams");
+        set_error("out of host memory while building the band streams");
         return SNA_ERR_ALLOC;
     }
-    static_assert(sizeof(sna::StreamEntry) == 16, "stream entries are read as int4");
+    static_assert(sizeof(sna::BandColumn) == 16, "read as int4");
 
     // pack everything into one device allocation (each array 256-byte aligned)
     struct Piece { const void* src; size_t bytes; size_t offset; };
@@ -220,16 +189,17 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
         {hp.row_ptr.data(), hp.row_ptr.size() * 4, 0}, {win_lat.data(), win_lat.size() * 4, 0}, {win_m.data(), win_m.size() * 4, 0},
         {row_order.data(), row_order.size() * 4, 0}, {hp.t_row_ptr.data(), hp.t_row_ptr.size() * 4, 0}, {t_lat.data(), t_lat.size() * 4, 0},
         {t_m.data(), t_m.size() * 4, 0}, {t_row_order.data(), t_row_order.size() * 4, 0}, {log2_omega.data(), log2_omega.size() * 4, 0},
-        {fwd_stream.entries.data(), fwd_stream.entries.size() * 16, 0}, {fwd_stream.chunk_ptr.data(), fwd_stream.chunk_ptr.size() * 4, 0},
-        {t_stream.entries.data(), t_stream.entries.size() * 16, 0}, {t_stream.chunk_ptr.data(), t_stream.chunk_ptr.size() * 4, 0},
-        {grp_order.data(), grp_order.size() * 4, 0}, {t_grp_order.data(), t_grp_order.size() * 4, 0},
-        {fwdb_stream.entries.data(), fwdb_stream.entries.size() * 16, 0}, {fwdb_stream.chunk_ptr.data(), fwdb_stream.chunk_ptr.size() * 4, 0},
-        {grpb_order.data(), grpb_order.size() * 4, 0}, {dense.ptr.data(), dense.ptr.size() * 4, 0},
-        {dense.lat.data(), dense.lat.size() * 4, 0}, {dense.rows.data(), dense.rows.size() * 4, 0}, {zero_status, sizeof(zero_status), 0},
-        {tb_stream.entries.data(), tb_stream.entries.size() * 16, 0}, {tb_stream.chunk_ptr.data(), tb_stream.chunk_ptr.size() * 4, 0},
-        {tb_grp_order.data(), tb_grp_order.size() * 4, 0}, {t_dense.ptr.data(), t_dense.ptr.size() * 4, 0},
-        {t_dense.lat.data(), t_dense.lat.size() * 4, 0}, {t_dense.rows.data(), t_dense.rows.size() * 4, 0},
-        {dense.m.data(), dense.m.size() * 4, 0}, {t_dense.m.data(), t_dense.m.size() * 4, 0}};
+        {dense.ptr.data(), dense.ptr.size() * 4, 0}, {dense.lat.data(), dense.lat.size() * 4, 0}, {dense.m.data(), dense.m.size() * 4, 0},
+        {dense.rows.data(), dense.rows.size() * 4, 0}, {t_dense.ptr.data(), t_dense.ptr.size() * 4, 0}, {t_dense.lat.data(), t_dense.lat.size() * 4, 0},
+        {t_dense.m.data(), t_dense.m.size() * 4, 0}, {t_dense.rows.data(), t_dense.rows.size() * 4, 0}, {zero_status, sizeof(zero_status), 0}};
+    const size_t first_band_piece = pieces.size();
+    constexpr size_t BAND_PIECES = 4;
+    for (const sna::BandStream& b : bands) {
+        pieces.push_back({b.chunk_ptr.data(), b.chunk_ptr.size() * 4, 0});
+        pieces.push_back({b.columns.data(), b.columns.size() * sizeof(sna::BandColumn), 0});
+        pieces.push_back({b.masks.data(), b.masks.size() * 4, 0});
+        pieces.push_back({b.order.data(), b.order.size() * 4, 0});
+    }
     size_t total = 0;
     for (Piece& p : pieces) { p.offset = total; total += round256(p.bytes); }
     cudaError_t e = cudaGetDevice(&plan->device);
@@ -241,29 +211,35 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
         e = cudaMemcpy((char*)plan->dev_blob + p.offset, p.src, p.bytes, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) { cudaFree(plan->dev_blob); delete plan; return cuda_fail(e, "cudaMemcpy of plan tables"); }
     }
-    auto at = [&](int i) { return (const int32_t*)((char*)plan->dev_blob + pieces[i].offset); };
+    auto at = [&](size_t i) { return (const int32_t*)((char*)plan->dev_blob + pieces[i].offset); };
     sna::DevPlan& d = plan->dev;
     d.nlat_in = hp.nlat_in; d.nlon_in = hp.nlon_in; d.nlat_out = hp.nlat_out; d.nlon_out = hp.nlon_out; d.ps = hp.ps;
     d.row_ptr = at(0); d.win_lat = at(1); d.win_m = at(2); d.row_order = at(3);
     d.t_row_ptr = at(4); d.t_win_lat = at(5); d.t_win_m = at(6); d.t_row_order = at(7);
     d.log2_omega = (const float*)at(8);
-    d.fwd_stream = (const int4*)at(9); d.fwd_chunk_ptr = at(10);
-    d.t_stream = (const int4*)at(11); d.t_chunk_ptr = at(12);
-    d.grp_order = at(13); d.t_grp_order = at(14);
-    d.t_consecutive = t_consecutive ? 1 : 0;
-    d.fwdb_stream = (const int4*)at(15); d.fwdb_chunk_ptr = at(16); d.grpb_order = at(17);
-    d.dense_ptr = at(18); d.dense_lat = at(19); d.dense_rows = at(20);
+    d.dense_ptr = at(9); d.dense_lat = at(10); d.dense_m = at(11); d.dense_rows = at(12);
+    d.t_dense_ptr = at(13); d.t_dense_lat = at(14); d.t_dense_m = at(15); d.t_dense_rows = at(16);
+    d.dev_status = (int*)((char*)plan->dev_blob + pieces[17].offset);
     d.n_dense_rows = (int)dense.rows.size();
+    d.n_t_dense_rows = (int)t_dense.rows.size();
+    d.dense_blocks = dense.blocks;
+    d.dense_longest = dense.longest;
     d.dense_fraction = hp.nnz > 0 ? (float)((double)dense.pairs / (double)hp.nnz) : 0.f;
     d.is_global = global ? 1 : 0;
-    d.dev_status = (int*)((char*)plan->dev_blob + pieces[21].offset);
-    d.tb_stream = (const int4*)at(22); d.tb_chunk_ptr = at(23); d.tb_grp_order = at(24);
-    d.t_dense_ptr = at(25); d.t_dense_lat = at(26); d.t_dense_rows = at(27);
-    d.n_t_dense_rows = (int)t_dense.rows.size();
-    d.dense_m = at(28); d.t_dense_m = at(29);
+    d.t_consecutive = t_consecutive ? 1 : 0;
+    sna::DevBand* dev_bands[4] = {&d.fwd, &d.fwdb, &d.t, &d.tb};
+    for (size_t i = 0; i < 4; ++i) {
+        const size_t f = first_band_piece + BAND_PIECES * i;
+        plan->band_lengths[i] = std::move(bands[i].lengths);
+        *dev_bands[i] = global ? sna::DevBand{} : sna::DevBand{at(f), (const int4*)at(f + 1), (const uint32_t*)at(f + 2), at(f + 3),
+                                                               plan->band_lengths[i].data(), (int)bands[i].order.size(),
+                                                               (long long)bands[i].chunk_ptr.back()};
+    }
+    e = cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, plan->device);
+    if (e != cudaSuccess) { sna_plan_destroy(plan); return cuda_fail(e, "cudaDeviceGetAttribute"); }
     // opt in to the kernels' dynamic shared-memory sizes on this device (once here instead of on every launch)
     e = sna::dense2_prepare_device();
-    if (e == cudaSuccess) e = sna::mma_prepare_device();
+    if (e == cudaSuccess) e = sna::band_prepare_device();
     if (e != cudaSuccess) { sna_plan_destroy(plan); return cuda_fail(e, "cudaFuncSetAttribute"); }
     *plan_out = plan;
     return SNA_OK;
@@ -393,7 +369,7 @@ size_t sna_workspace_bytes(const sna_plan_t* plan, int B, int H, int C) {
 int sna_forward_kernel_count(const sna_plan_t* plan, int C, int with_lse) {
     if (plan == nullptr || plan->dev_blob == nullptr || !supported_C(C)) return 0;
     if (plan->is_global || sna::dense2_global_supported(plan->dev, C)) return 1;
-    return (with_lse && sna::dense2_path_supported(plan->dev, C)) ? 2 : 1;
+    return (with_lse && sna::dense2_path_chosen(plan->dev, C, 1 << 20)) ? 2 : 1;
 }
 
 sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
@@ -409,12 +385,12 @@ sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float*
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
     } else if (plan->is_global) {
         e = sna::launch_forward_generic(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (lse != nullptr && sna::dense2_path_supported(plan->dev, C)) {
+    } else if (lse != nullptr && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its partial result travels in out / lse), the rest on the band kernel
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_forward_mma_band(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (sna::mma_path_supported(plan->dev, C)) {
-        e = sna::launch_forward_mma(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, true, false, (cudaStream_t)cuda_stream);
+    } else if (sna::band_path_supported(plan->dev, C)) {
+        e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, false, false, (cudaStream_t)cuda_stream);
     } else {
         e = sna::launch_forward_generic(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
     }
@@ -441,12 +417,12 @@ sna_status_t sna_backward_dq(const sna_plan_t* plan, const float* q, const float
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
     } else if (plan->is_global) {
         e = sna::launch_backward_dq_generic(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (out != nullptr && out != dq && plan->dev.dense_fraction >= 0.10f && sna::dense2_path_supported(plan->dev, C)) {
+    } else if (out != nullptr && out != dq && plan->dev.dense_fraction >= 0.10f && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dq is written first), the rest is added by the band kernel
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, nullptr, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_backward_dq_mma_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (out != nullptr && sna::mma_path_supported(plan->dev, C)) {
-        e = sna::launch_backward_dq_mma(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, true, false, (cudaStream_t)cuda_stream);
+    } else if (out != nullptr && sna::band_path_supported(plan->dev, C)) {
+        e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, false, false, (cudaStream_t)cuda_stream);
     } else {
         e = sna::launch_backward_dq_generic(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
     }
@@ -475,12 +451,12 @@ sna_status_t sna_backward_dkdv(const sna_plan_t* plan, const float* q, const flo
         e = dense
                 ? sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream)
                 : sna::launch_backward_dkdv_generic(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_supported(plan->dev, C)) {
+    } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dk, dv is written first), the band kernel adds the rest
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_backward_dkdv_mma_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (sna::mma_path_supported(plan->dev, C)) {
-        e = sna::launch_backward_dkdv_mma(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, true, false, (cudaStream_t)cuda_stream);
+    } else if (sna::band_path_supported(plan->dev, C)) {
+        e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, false, false, (cudaStream_t)cuda_stream);
     } else {
         e = sna::launch_backward_dkdv_generic(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
     }
@@ -518,11 +494,11 @@ sna_status_t sna_backward_ex(const sna_plan_t* plan, const float* q, const float
             if (e != cudaSuccess) return cuda_fail(e, "statistics launch");
             lse = ws_lse;
         }
-    } else if (sna::mma_path_supported(plan->dev, C)) {
+    } else if (sna::band_path_supported(plan->dev, C)) {
         if (lse == nullptr || out == nullptr) {
             // recompute the forward pass: lse into the workspace, out into the dq buffer, which the dq stage
             // reads row by row before it overwrites the same rows with dq
-            e = sna::launch_forward_mma(plan->dev, q, k, v, dq, ws_lse, N, C, stream);
+            e = sna::launch_forward_band(plan->dev, q, k, v, dq, ws_lse, N, C, false, false, stream);
             if (e != cudaSuccess) return cuda_fail(e, "statistics launch");
             lse = ws_lse;
             out = dq;
@@ -656,8 +632,8 @@ sna_status_t sna_forward_tf32(const sna_plan_t* plan, const float* q, const floa
     if (st != SNA_OK) return st;
     if (!q || !k || !v || !out) { set_error("q, k, v and out must not be NULL"); return SNA_ERR_INVALID_ARG; }
     if (!all_aligned(q, k, v, out) || (reinterpret_cast<uintptr_t>(lse) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
-    if (!sna::mma_path_supported(plan->dev, C)) { set_error("the reduced-precision variant needs C in {16, 32, 64} and nlon_out >= 32"); return SNA_ERR_UNSUPPORTED; }
-    cudaError_t e = sna::launch_forward_mma_lp(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
+    if (!tf32_supported(plan, C)) { set_error("the reduced-precision variant needs C in {16, 32, 64} and nlon_out >= 32"); return SNA_ERR_UNSUPPORTED; }
+    cudaError_t e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, false, true, (cudaStream_t)cuda_stream);
     if (e != cudaSuccess) return cuda_fail(e, "forward launch");
     return SNA_OK;
 }
@@ -671,20 +647,20 @@ sna_status_t sna_backward_tf32(const sna_plan_t* plan, const float* q, const flo
     if (!all_aligned(q, k, v, dout, dq, dk, dv, out) || (reinterpret_cast<uintptr_t>(lse) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & 255u)) { set_error("workspace must be non-NULL and 256-byte aligned"); return SNA_ERR_INVALID_ARG; }
     if (workspace_bytes < sna_workspace_bytes(plan, B, H, C)) { set_error("workspace too small: %zu < %zu bytes", workspace_bytes, sna_workspace_bytes(plan, B, H, C)); return SNA_ERR_WORKSPACE; }
-    if (!sna::mma_path_supported(plan->dev, C)) { set_error("the reduced-precision variant needs C in {16, 32, 64} and nlon_out >= 32"); return SNA_ERR_UNSUPPORTED; }
+    if (!tf32_supported(plan, C)) { set_error("the reduced-precision variant needs C in {16, 32, 64} and nlon_out >= 32"); return SNA_ERR_UNSUPPORTED; }
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const int N = B * H;
     float* ws_lse = (float*)workspace;
     float* ws_D = ws_lse + stats_elems(plan, B, H);
     cudaError_t e;
     if (lse == nullptr || out == nullptr) {   // recompute the forward pass: lse into the workspace, out into the dq buffer
-        e = sna::launch_forward_mma_lp(plan->dev, q, k, v, dq, ws_lse, N, C, stream);
+        e = sna::launch_forward_band(plan->dev, q, k, v, dq, ws_lse, N, C, false, true, stream);
         if (e != cudaSuccess) return cuda_fail(e, "statistics launch");
         lse = ws_lse;
         out = dq;
     }
-    e = sna::launch_backward_dq_mma_lp(plan->dev, q, k, v, dout, out, lse, dq, ws_D, N, C, stream);
-    if (e == cudaSuccess) e = sna::launch_backward_dkdv_mma_lp(plan->dev, q, k, v, dout, lse, ws_D, dk, dv, N, C, stream);
+    e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, ws_D, N, C, false, true, stream);
+    if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, ws_D, dk, dv, N, C, false, true, stream);
     if (e != cudaSuccess) return cuda_fail(e, "backward launch");
     return SNA_OK;
 }

@@ -1388,9 +1388,16 @@ cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t 
     return cudaGetLastError();
 }
 
-bool dense2_path_supported(const DevPlan& p, int C) {
-    return C == C2 && p.dense_ptr != nullptr && p.n_dense_rows > 0 && p.fwdb_stream != nullptr && mma_path_supported(p, C) &&
-           encode_fn2() != nullptr;
+bool dense2_path_chosen(const DevPlan& p, int C, int N) {
+    if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
+    // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time; below that much work per
+    // SM the band kernels alone, which share long streams between warps, are faster.  Measured (fwd / dq / dkdv us, with : without
+    // the dense kernels; work in longest lists per SM): 128x256, cutoff 4 rings, N = 1 (0.1) 57/62/80 : 32/36/40, N = 4 (0.4)
+    // 99/114/150 : 89/110/124, N = 8 (0.8) 166/191/239 : 170/202/233, N = 16 (1.6) 310/356/447 : 329/389/456; 256x512 -> 128x256
+    // N = 8 (0.9) 370/408/539 : 387/464/551; 361x720 N = 1 (0.6) 271/287/375 : 258/299/351, N = 2 (1.2) 486/521/672 : 488/577/686.
+    // The second bound is the fixed cost of another kernel: 32x64, N = 32 (0.9 lists of 3 blocks) 49/52/55 : 36/41/39.
+    const long long work = (long long)((p.nlon_out + M2 - 1) / M2) * N * p.dense_blocks;
+    return work * 10 >= p.num_sms * 8LL * p.dense_longest && work >= p.num_sms * 6LL;
 }
 
 bool dense2_global_supported(const DevPlan& p, int C) {

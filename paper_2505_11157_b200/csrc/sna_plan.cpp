@@ -239,51 +239,10 @@ namespace {
 inline int floor_div(int a, int b) { int q = a / b; return ((a % b != 0) && ((a < 0) != (b < 0))) ? q - 1 : q; }
 inline int ceil_div(int a, int b) { return -floor_div(-a, b); }
 
-// One partner ring as seen from the rings of a group: per group ring either absent, a band of offsets, or whole.
-struct GroupRange {
-    bool present = false, whole = false;
-    int lo = 0, hi = -1;
-};
-
-// Appends the columns of one partner ring / residue for a ring group.
-void append_group_columns(std::vector<StreamEntry>& v, int32_t base, float bias, const GroupRange (&rg)[TILE_LAT], int whole_count) {
-    uint32_t whole_rows = 0, band_rows_any = 0;
-    for (int k = 0; k < TILE_LAT; ++k) {
-        if (rg[k].present && rg[k].whole) whole_rows |= ((1u << TILE_LON) - 1u) << (k * TILE_LON);
-        if (rg[k].present && !rg[k].whole && rg[k].hi >= rg[k].lo) band_rows_any |= 1u << k;
-    }
-    if (whole_rows) {   // absolute partner index: every partner of the ring, for the rings that take it whole
-        for (int u = 0; u < whole_count; ++u)
-            v.push_back(StreamEntry{(int32_t)(base | (int32_t)0x80000000), (int32_t)((u & 0xffff) | (whole_rows << 16)), bias, 0});
-    }
-    if (!band_rows_any) return;
-    int lo = INT32_MAX, hi = INT32_MIN;
-    for (int k = 0; k < TILE_LAT; ++k)
-        if (band_rows_any & (1u << k)) { lo = std::min(lo, rg[k].lo); hi = std::max(hi, rg[k].hi); }
-    for (int x = 0; x < TILE_LON - 1 + (hi - lo + 1); ++x) {
-        const int e_rel = lo + x;
-        uint32_t mask = 0;
-        for (int k = 0; k < TILE_LAT; ++k) {
-            if (!(band_rows_any & (1u << k))) continue;
-            for (int i = 0; i < TILE_LON; ++i)
-                if (e_rel - i >= rg[k].lo && e_rel - i <= rg[k].hi) mask |= 1u << (k * TILE_LON + i);
-        }
-        if (mask) v.push_back(StreamEntry{base, (int32_t)(((uint32_t)e_rel & 0xffffu) | (mask << 16)), bias, 0});
-    }
-}
-
-void pad_row(std::vector<StreamEntry>& v, size_t row_start) {
-    while ((v.size() - row_start) % 16 != 0) {
-        StreamEntry pad = v.size() > row_start ? v.back() : StreamEntry{0, 0, 0.f, 0};
-        pad.e_mask &= 0xffff;   // row mask 0: the column is ignored
-        v.push_back(pad);
-    }
-}
-
 // Merges the window lists of the rings of a group (each sorted by partner ring) and calls
 // emit(partner_ring, m[TILE_LAT]) with m = -2 for "not in this ring's list".
 template <typename Emit>
-void merge_group(const std::vector<int32_t>& ptr, const std::vector<RingWindow>& win, int first_ring, int nrings, Emit&& emit) {
+void merge_group(const std::vector<int32_t>& ptr, const std::vector<RingWindow>& win, int first_ring, int nrings, int dense_min_width, Emit&& emit) {
     int pos[TILE_LAT], end[TILE_LAT];
     for (int k = 0; k < TILE_LAT; ++k) {
         const int ring = first_ring + k;
@@ -296,9 +255,85 @@ void merge_group(const std::vector<int32_t>& ptr, const std::vector<RingWindow>&
             if (pos[k] < end[k]) lat = std::min(lat, win[pos[k]].lat);
         if (lat == INT32_MAX) break;
         int m[TILE_LAT];
-        for (int k = 0; k < TILE_LAT; ++k) m[k] = (pos[k] < end[k] && win[pos[k]].lat == lat) ? win[pos[k]++].m : -2;
+        for (int k = 0; k < TILE_LAT; ++k) {
+            m[k] = (pos[k] < end[k] && win[pos[k]].lat == lat) ? win[pos[k]++].m : -2;
+            if (m[k] != -2 && served_by_dense(RingWindow{lat, m[k]}, dense_min_width)) m[k] = -2;
+        }
         emit(lat, m);
     }
+}
+
+// Collects the columns of one stream row and packs them into chunks.
+class BandBuilder {
+public:
+    // All `count` points of a partner ring, for the group rings that take it whole (m = -1).
+    void add_whole(int32_t base, float bias, const int (&m)[TILE_LAT], int count) {
+        uint32_t mask = 0;
+        for (int k = 0; k < TILE_LAT; ++k)
+            if (m[k] == -1) mask |= ((1u << TILE_LON) - 1u) << (k * TILE_LON);
+        if (mask) for (int u = 0; u < count; ++u) add((int32_t)(base | (int32_t)0x80000000), u, bias, mask);
+    }
+    // A partner ring for the group rings with a band (m >= 0): band_range(m, i, lo, hi) gives the partner offsets [lo, hi] that
+    // tile longitude i uses.
+    template <typename Range>
+    void add_band(int32_t base, float bias, const int (&m)[TILE_LAT], Range&& band_range) {
+        int rlo[TILE_LAT][TILE_LON], rhi[TILE_LAT][TILE_LON], lo = INT32_MAX, hi = INT32_MIN;
+        for (int k = 0; k < TILE_LAT; ++k)
+            for (int i = 0; i < TILE_LON; ++i) {
+                rlo[k][i] = 0; rhi[k][i] = -1;          // empty
+                if (m[k] < 0) continue;
+                band_range(m[k], i, rlo[k][i], rhi[k][i]);
+                if (rhi[k][i] >= rlo[k][i]) { lo = std::min(lo, rlo[k][i]); hi = std::max(hi, rhi[k][i]); }
+            }
+        for (int e = lo; e <= hi; ++e) {
+            uint32_t mask = 0;
+            for (int k = 0; k < TILE_LAT; ++k)
+                for (int i = 0; i < TILE_LON; ++i)
+                    if (e >= rlo[k][i] && e <= rhi[k][i]) mask |= 1u << (k * TILE_LON + i);
+            if (mask) add(base, e, bias, mask);
+        }
+    }
+    void finish(BandStream& S) {
+        if (S.chunk_ptr.empty()) S.chunk_ptr.push_back(0);
+        for (size_t c = 0; c < cols_.size(); c += BAND_CHUNK) {
+            uint32_t mask[BAND_CHUNK], all = 0xffffu;
+            for (size_t j = 0; j < BAND_CHUNK; ++j) {          // padding repeats the last column with an empty mask
+                const bool exists = c + j < cols_.size();
+                S.columns.push_back(exists ? cols_[c + j] : cols_.back());
+                mask[j] = exists ? masks_[c + j] : 0u;
+                all &= mask[j];
+            }
+            for (int lane = 0; lane < 32; ++lane) {
+                uint32_t bits = all == 0xffffu ? BAND_ALL : 0u;
+                for (int j = 0; j < 2; ++j)
+                    for (int r = 0; r < 2; ++r)
+                        for (int k = 0; k < 2; ++k)
+                            bits |= (mask[8 * j + 2 * (lane & 3) + k] >> (8 * r + lane / 4) & 1u) << (4 * j + 2 * r + k);
+                S.masks.push_back(bits);
+            }
+        }
+        S.chunk_ptr.push_back((int32_t)(S.columns.size() / BAND_CHUNK));
+    }
+
+private:
+    void add(int32_t base, int32_t e, float bias, uint32_t mask) {
+        cols_.push_back(BandColumn{base, e, bias, 0});
+        masks_.push_back(mask);
+    }
+    std::vector<BandColumn> cols_;
+    std::vector<uint32_t> masks_;
+};
+
+void complete(BandStream& S, int rows_per_group) {
+    // the kernels read three chunks ahead
+    const BandColumn last = S.columns.empty() ? BandColumn{0, 0, 0.f, 0} : S.columns.back();
+    S.columns.insert(S.columns.end(), 3 * BAND_CHUNK, last);
+    S.masks.insert(S.masks.end(), 3 * 32, 0u);
+    S.order.resize((S.chunk_ptr.size() - 1) / rows_per_group);
+    for (size_t i = 0; i < S.order.size(); ++i) S.order[i] = (int32_t)i;
+    auto length = [&](int g) { return S.chunk_ptr[(size_t)(g + 1) * rows_per_group] - S.chunk_ptr[(size_t)g * rows_per_group]; };
+    std::stable_sort(S.order.begin(), S.order.end(), [&](int a, int b) { return length(a) > length(b); });
+    for (int g : S.order) S.lengths.push_back(length(g) / rows_per_group);
 }
 
 }  // namespace
@@ -307,14 +342,20 @@ void build_dense_lists(const HostPlan& P, DenseLists& D, int dense_min_width) {
     D = DenseLists();
     D.ptr.assign(P.nlat_out + 1, 0);
     for (int h = 0; h < P.nlat_out; ++h) {
+        int64_t blocks = 0;
         for (int e = P.row_ptr[h]; e < P.row_ptr[h + 1]; ++e) {
             if (!served_by_dense(P.windows[e], dense_min_width)) continue;
             D.lat.push_back(P.windows[e].lat);
             D.m.push_back(P.windows[e].m);
             D.pairs += P.window_count(P.windows[e]);
+            // the columns between the first row's window and the last row's
+            const int64_t span = P.windows[e].m < 0 ? P.nlon_in : std::min<int64_t>(2 * P.windows[e].m + 1 + 127LL * P.ps, P.nlon_in);
+            blocks += (span + 127) / 128;
         }
         D.ptr[h + 1] = (int32_t)D.lat.size();
         if (D.ptr[h + 1] > D.ptr[h]) D.rows.push_back(h);
+        D.blocks += blocks;
+        D.longest = std::max(D.longest, blocks);
     }
 }
 
@@ -333,91 +374,45 @@ void build_transposed_dense_lists(const HostPlan& P, DenseLists& D, int dense_mi
     }
 }
 
-void build_forward_stream(const HostPlan& P, Stream& S, int dense_min_width) {
-    const int groups = (P.nlat_out + TILE_LAT - 1) / TILE_LAT;
-    S.chunk_ptr.assign(groups + 1, 0);
-    S.entries.clear();
-    for (int gi = 0; gi < groups; ++gi) {
-        const size_t start = S.entries.size();
-        merge_group(P.row_ptr, P.windows, gi * TILE_LAT, P.nlat_out, [&](int lat, const int (&m)[TILE_LAT]) {
+void build_forward_band(const HostPlan& P, BandStream& S, int dense_min_width) {
+    S = BandStream();
+    for (int first = 0; first < P.nlat_out; first += TILE_LAT) {
+        BandBuilder b;
+        merge_group(P.row_ptr, P.windows, first, P.nlat_out, dense_min_width, [&](int lat, const int (&m)[TILE_LAT]) {
             const float bias = (float)std::log2(P.omega[lat]);
             for (int r = 0; r < P.ps; ++r) {
-                GroupRange rg[TILE_LAT];
-                for (int k = 0; k < TILE_LAT; ++k) {
-                    if (m[k] == -2) continue;
-                    if (served_by_dense(RingWindow{lat, m[k]}, dense_min_width)) continue;
-                    rg[k].present = true;
-                    if (m[k] < 0) rg[k].whole = true;
-                    else { rg[k].lo = ceil_div(-m[k] - r, P.ps); rg[k].hi = floor_div(m[k] - r, P.ps); }
-                }
-                append_group_columns(S.entries, lat * P.nlon_in + r, bias, rg, P.nlon_out);
+                b.add_whole(lat * P.nlon_in + r, bias, m, P.nlon_out);
+                b.add_band(lat * P.nlon_in + r, bias, m, [&](int mk, int i, int& lo, int& hi) {
+                    lo = i + ceil_div(-mk - r, P.ps);
+                    hi = i + floor_div(mk - r, P.ps);
+                });
             }
         });
-        pad_row(S.entries, start);
-        S.chunk_ptr[gi + 1] = (int32_t)(S.entries.size() / 16);
+        b.finish(S);
     }
+    complete(S, 1);
 }
 
-bool build_transposed_stream(const HostPlan& P, Stream& S, int dense_min_width) {
-    const int groups = (P.nlat_in + TILE_LAT - 1) / TILE_LAT;
-    S.entries.clear();
-    if (TILE_LON % P.ps == 0) {
-        // Consecutive layout.  Tile row i of ring k is input column c0 + i; output point (h, w) is its partner iff
-        // (c0 + i) - w*ps in [-m, m]  <=>  w - c0/ps in [ceil((i - m)/ps), floor((i + m)/ps)].
-        S.chunk_ptr.assign((size_t)groups + 1, 0);
-        for (int gi = 0; gi < groups; ++gi) {
-            const size_t start = S.entries.size();
-            merge_group(P.t_row_ptr, P.t_windows, gi * TILE_LAT, P.nlat_in, [&](int lat, const int (&m)[TILE_LAT]) {
-                const int32_t base = lat * P.nlon_out;
-                uint32_t whole_rows = 0;
-                int lo = INT32_MAX, hi = INT32_MIN;
-                for (int k = 0; k < TILE_LAT; ++k) {
-                    if (m[k] == -2) continue;
-                    if (served_by_dense(RingWindow{lat, m[k]}, dense_min_width)) continue;
-                    if (m[k] < 0) { whole_rows |= ((1u << TILE_LON) - 1u) << (k * TILE_LON); continue; }
-                    lo = std::min(lo, ceil_div(-m[k], P.ps));
-                    hi = std::max(hi, floor_div(TILE_LON - 1 + m[k], P.ps));
-                }
-                if (whole_rows)
-                    for (int u = 0; u < P.nlon_out; ++u)
-                        S.entries.push_back(StreamEntry{(int32_t)(base | (int32_t)0x80000000), (int32_t)((u & 0xffff) | (whole_rows << 16)), 0.f, 0});
-                for (int e_rel = lo; e_rel <= hi; ++e_rel) {
-                    uint32_t mask = 0;
-                    for (int k = 0; k < TILE_LAT; ++k) {
-                        if (m[k] < 0 || served_by_dense(RingWindow{lat, m[k]}, dense_min_width)) continue;   // absent, whole (above) or dense
-                        for (int i = 0; i < TILE_LON; ++i)
-                            if (e_rel >= ceil_div(i - m[k], P.ps) && e_rel <= floor_div(i + m[k], P.ps)) mask |= 1u << (k * TILE_LON + i);
-                    }
-                    if (mask) S.entries.push_back(StreamEntry{base, (int32_t)(((uint32_t)e_rel & 0xffffu) | (mask << 16)), 0.f, 0});
-                }
+bool build_transposed_band(const HostPlan& P, BandStream& S, int dense_min_width) {
+    S = BandStream();
+    const bool consecutive = TILE_LON % P.ps == 0;
+    for (int first = 0; first < P.nlat_in; first += TILE_LAT)
+        for (int r = 0; r < (consecutive ? 1 : P.ps); ++r) {
+            BandBuilder b;
+            merge_group(P.t_row_ptr, P.t_windows, first, P.nlat_in, dense_min_width, [&](int lat, const int (&m)[TILE_LAT]) {
+                // Output point w is a partner of input column c iff c - w*ps lies in [-m, m].  Consecutive: c = c0 + i, so
+                // w - c0/ps in [ceil((i - m)/ps), floor((i + m)/ps)].  By residue: c = ps*(u0+i) + r, so w - u0 in
+                // [i + ceil((r - m)/ps), i + floor((r + m)/ps)].
+                b.add_whole(lat * P.nlon_out, 0.f, m, P.nlon_out);
+                b.add_band(lat * P.nlon_out, 0.f, m, [&](int mk, int i, int& lo, int& hi) {
+                    lo = consecutive ? ceil_div(i - mk, P.ps) : i + ceil_div(r - mk, P.ps);
+                    hi = consecutive ? floor_div(i + mk, P.ps) : i + floor_div(r + mk, P.ps);
+                });
             });
-            pad_row(S.entries, start);
-            S.chunk_ptr[(size_t)gi + 1] = (int32_t)(S.entries.size() / 16);
+            b.finish(S);
         }
-        return true;
-    }
-    // By residue.  Row (group, r): tile rows are input columns c = ps*u + r.  Output point (h, w) is a partner of
-    // column u of input ring h' iff c - w*ps in [-m, m]  <=>  w - u in [ceil((r - m)/ps), floor((r + m)/ps)].
-    S.chunk_ptr.assign((size_t)groups * P.ps + 1, 0);
-    for (int gi = 0; gi < groups; ++gi) {
-        for (int r = 0; r < P.ps; ++r) {
-            const size_t start = S.entries.size();
-            merge_group(P.t_row_ptr, P.t_windows, gi * TILE_LAT, P.nlat_in, [&](int lat, const int (&m)[TILE_LAT]) {
-                GroupRange rg[TILE_LAT];
-                for (int k = 0; k < TILE_LAT; ++k) {
-                    if (m[k] == -2) continue;
-                    if (served_by_dense(RingWindow{lat, m[k]}, dense_min_width)) continue;
-                    rg[k].present = true;
-                    if (m[k] < 0) rg[k].whole = true;
-                    else { rg[k].lo = ceil_div(r - m[k], P.ps); rg[k].hi = floor_div(r + m[k], P.ps); }
-                }
-                append_group_columns(S.entries, lat * P.nlon_out, 0.f, rg, P.nlon_out);
-            });
-            pad_row(S.entries, start);
-            S.chunk_ptr[(size_t)gi * P.ps + r + 1] = (int32_t)(S.entries.size() / 16);
-        }
-    }
-    return false;
+    complete(S, consecutive ? 1 : P.ps);
+    return consecutive;
 }
 
 }  // namespace sna

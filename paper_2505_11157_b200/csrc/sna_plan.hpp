@@ -39,35 +39,48 @@ struct HostPlan {
 // weight zero.
 bool drop_zero_weight_rings(const HostPlan& full, HostPlan& out);
 
-// Column streams for the tensor-core kernels.  A warp owns a tile of 16 points: TILE_LON = 8 consecutive
-// longitudes on each of TILE_LAT = 2 adjacent rings (a "ring group"); tile row i is ring i / 8 of the group,
-// longitude first + i % 8.  Two adjacent rings see almost the same partner points, and 8-wide rows waste fewer
-// columns on the slanted band than 16-wide rows would.  The warp walks a stream of partner points ("columns"),
-// 16 per step.  For a window with offsets e in [e_lo, e_hi] (in units of ps input columns for the forward
-// table, of output columns for the transposed one) a row at longitude first + i uses partner first + e_rel iff
-// e_lo <= e_rel - i <= e_hi: that is the row's bit in the column's 16-bit mask.  The stream of a ring group is
-// the concatenation, over partner rings and residues, of the columns at least one row uses, padded to a
-// multiple of 16 with mask-0 columns; it is the same for every tile of the group, so it is built once on the host.
+// Band streams for the mma.sync kernels.  A warp owns a tile of 16 points = 8 consecutive longitudes on each of 2 adjacent rings (a
+// "ring group"); tile row i is ring i / 8 of the group, longitude first + i % 8.  It walks the group's stream of partner points
+// ("columns"), 16 at a time (a chunk).  Adjacent rings see almost the same partner points, and 8-wide rows waste fewer columns
+// on the slanted band than 16-wide rows would.
+// A window with offsets [lo, hi] (in units of ps input columns for the forward table, of output columns for the transposed
+// one) makes the row at longitude first + i use the partner at first + e iff lo <= e - i <= hi: that is the row's bit in the
+// column's mask.  The stream of a ring group is the concatenation, over partner rings and residues, of the columns at least one
+// row uses; it is the same for every longitude, so it is built once on the host.
 constexpr int TILE_LON = 8;
 constexpr int TILE_LAT = 2;
+constexpr int BAND_CHUNK = 16;
 
-struct StreamEntry {
-    int32_t base;      // flat row index of the partner ring plus the residue r; bit 31 set = e is absolute
-    int32_t e_mask;    // low 16 bits: e_rel (signed) or the absolute partner index; high 16 bits: row mask
+struct BandColumn {
+    int32_t base;      // flat index of the partner ring's first point plus the residue r; bit 31 set = e is absolute
+    int32_t e;         // partner index relative to the tile's first point (or absolute)
     float bias;        // forward: log2 of the partner ring's quadrature weight; transposed: unused (0)
-    int32_t aux;       // unused
+    int32_t unused;
+};
+// Per chunk and lane of the warp, the mask of the 8 scores that the lane holds: lane 4 g + t, bit 4 j + 2 r + c is tile row
+// g + 8 r, column 8 j + 2 t + c; and, the same for all lanes, whether every row uses every column.
+constexpr uint32_t BAND_ALL = 1u << 16;
+struct BandStream {
+    std::vector<int32_t> chunk_ptr;     // [rows+1] first chunk of each stream row
+    std::vector<BandColumn> columns;    // BAND_CHUNK per chunk
+    std::vector<uint32_t> masks;        // 32 per chunk
+    std::vector<int32_t> order;         // ring groups, longest stream first
+    std::vector<int32_t> lengths;       // chunks per stream row of order[i]
 };
 
-struct Stream {
-    std::vector<int32_t> chunk_ptr;     // [rows+1] first 16-column chunk of each stream row
-    std::vector<StreamEntry> entries;   // 16 * chunk_ptr.back()
-};
-
-// Forward stream: one row per group of output latitudes (ceil(nlat_out / TILE_LAT) rows); partners are input
-// points, flat index base + u*ps.
-// With dense_min_width > 0 the columns of the windows that served_by_dense() accepts are left out: those are served
-// by the dense kernels (see DenseLists), and the stream only carries the narrower windows.
-void build_forward_stream(const HostPlan& plan, Stream& out, int dense_min_width = 0);
+// Forward stream: one row per group of TILE_LAT output latitudes; partners are input points, flat index base + u*ps.
+// With dense_min_width > 0 the windows that served_by_dense() accepts are left out: those are served by the dense
+// kernels (see DenseLists), and the stream only carries the narrower windows.
+void build_forward_band(const HostPlan& plan, BandStream& out, int dense_min_width = 0);
+// Transposed stream for dk/dv; tile rows are input points, partners are output points (h, w).  Two layouts:
+//  - consecutive (when ps divides 8): one stream row per group of input latitudes; tile rows are 8 consecutive input
+//    columns c = c0 + i%8 (c0 a multiple of 8) and the partner index is c0/ps + e.  Neighbouring
+//    input columns share most of their partners, so this needs ~ps times fewer stream columns per input column
+//    than splitting by residue.
+//  - by residue (any other ps): one stream row per (group, residue r); tile rows are c = ps*(u0+i%8) + r and
+//    the partner index is u0 + e.
+// Returns true for the consecutive layout.
+bool build_transposed_band(const HostPlan& plan, BandStream& out, int dense_min_width = 0);
 
 // Which windows the dense (tcgen05) kernels take: whole rings, and banded windows of at least dense_min_width input
 // columns (they run as masked blocks there).  dense_min_width = nlon_in + 1 selects the whole rings only.
@@ -83,21 +96,13 @@ struct DenseLists {
     std::vector<int32_t> m;      // window half widths in input columns, -1 = whole ring
     std::vector<int32_t> rows;   // output latitudes that have at least one such window
     int64_t pairs = 0;           // table entries covered, per output longitude / input column
+    int64_t blocks = 0;          // 128-column blocks that a tile of 128 points walks, over all rows
+    int64_t longest = 0;         // ... of the row with most
 };
 void build_dense_lists(const HostPlan& plan, DenseLists& out, int dense_min_width);
 // The transposed lists for the dense dk/dv kernel: input ring h' is attended to through such a window by the output
 // rings lat[ptr[h']] .. lat[ptr[h'+1]-1]; rows = input latitudes with at least one such output ring.
 void build_transposed_dense_lists(const HostPlan& plan, DenseLists& out, int dense_min_width);
-// Transposed stream for dk/dv; partners are output points (h, w).  Two layouts:
-//  - consecutive (when ps divides 8): one stream row per group of input latitudes; tile rows are 8 consecutive
-//    input columns c = c0 + i%8 (c0 a multiple of 8) and the partner index is c0/ps + e_rel.  Neighbouring
-//    input columns share most of their partners, so this needs ~ps times fewer stream columns per input column
-//    than splitting by residue.
-//  - by residue (any other ps): one stream row per (group, residue r); tile rows are c = ps*(u0+i%8) + r and
-//    the partner index is u0 + e_rel.
-// Returns true for the consecutive layout.
-bool build_transposed_stream(const HostPlan& plan, Stream& out, int dense_min_width = 0);
-
 // Builds the plan.  On failure returns a status and fills `why`.
 PlanStatus build_plan(int nlat_in, int nlon_in, int nlat_out, int nlon_out, int grid_in, int grid_out,
                       double theta_cutoff, HostPlan& plan, std::string& why);

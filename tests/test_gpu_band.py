@@ -1,0 +1,93 @@
+"""Band kernels at the edges of their tiles and value ranges, against the fp64 CPU oracle.
+
+Tolerance: every operand of a product is held to 22 significant bits, so a score of magnitude s (log2 domain) carries an error of
+about 2^-21 * sum|q k|, which is |s| * sqrt(C) at most; with unit-variance inputs (|s| <= 5, C <= 64) that is 2e-5 for the worst
+weight and, as errors are independent, below 2e-6 in the 2-norm over an output.  5e-6 is used; measured 4e-7 to 1.3e-6.
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import sna_oracle as orc
+from paper_2505_11157_b200 import sna
+from paper_2505_11157_b200.synthetic import make_inputs, small_workload
+
+pytestmark = pytest.mark.gpu
+
+TOL, TOL_REDUCED = 5e-6, 3e-3        # reduced precision: 2^-11 per operand, 2^10 times the above
+
+
+def rel(x, ref):
+    return float(np.linalg.norm(x.detach().cpu().numpy().reshape(ref.shape).astype(np.float64) - ref) / np.linalg.norm(ref))
+
+
+def check(wl, q, k, v, dout, tol=TOL, precision="fp32", recompute=False):
+    g = orc.geometry(wl.nlat_in, wl.nlon_in, wl.nlat_out, wl.nlon_out, wl.grid_in, wl.grid_out, wl.theta_cutoff)
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (q, k, v, dout)]
+    with sna.Plan(wl.nlat_in, wl.nlon_in, wl.nlat_out, wl.nlon_out, wl.grid_in, wl.grid_out, wl.theta_cutoff) as plan:
+        out, lse = plan.forward(*dev[:3], return_lse=True, precision=precision)
+        state = {} if recompute else {"out": out, "lse": lse}
+        grads = plan.backward(*dev, precision=precision, **state)
+        torch.cuda.synchronize()
+        sna.sna_plan_check(plan.handle)
+    ref, ref_lse = orc.forward(g, q, k, v, return_lse=True)
+    assert rel(out, ref) <= tol
+    assert np.max(np.abs(lse.cpu().numpy().reshape(ref_lse.shape) - ref_lse)) <= 20 * tol
+    for name, x, r in zip(("dq", "dk", "dv"), grads, orc.backward(g, q, k, v, dout)):
+        assert rel(x, r) <= tol, name
+
+
+@pytest.mark.parametrize("C", [4, 12, 16, 20, 28, 32, 36, 52, 60, 64])
+@pytest.mark.parametrize("shape", [(9, 17, 9, 17, 0.7), (12, 34, 7, 17, 0.6), (13, 96, 7, 32, 0.5)], ids=["odd", "down2", "down3"])
+def test_head_widths_and_ragged_tiles(C, shape):
+    """Partial pieces of a row, rings that end inside a tile, a last ring without a partner, strides 1 to 3."""
+    wl = small_workload("edge", *shape[:4], 0, 0, shape[4], 1, 2, C, 70 + C)
+    check(wl, *make_inputs(wl), recompute=C % 8 == 4)
+
+
+@pytest.mark.parametrize("slices", [1, 5, 300])
+def test_shared_and_private_streams(slices):
+    """Few slices: the warps of a block share a tile's stream; many: each warp walks its own."""
+    wl = small_workload("streams", 24, 48, 24, 48, 0, 1, 0.4, 1, slices, 16, 71)
+    check(wl, *make_inputs(wl))
+
+
+@pytest.mark.parametrize("slices", [1, 24])
+def test_dense_kernels_above_a_size(slices):
+    """C = 32: whole rings on the dense kernels for many slices, everything on the band kernels for few."""
+    wl = small_workload("dense_rule", 40, 160, 40, 160, 0, 0, 0.25, 1, slices, 32, 72)
+    check(wl, *make_inputs(wl))
+
+
+@pytest.mark.parametrize("precision, tol", [("fp32", TOL), ("tf32", TOL_REDUCED)])
+@pytest.mark.parametrize("C", [16, 32, 64])
+@pytest.mark.parametrize("which", ["k", "v", "dout", "all_tiny"])
+def test_value_ranges(which, C, precision, tol):
+    """Rows that grow by 2^24 along a stream overflow the scale taken from its first chunk: the tile is computed again.  Rows that
+    are zero at first, and inputs far below 1, must find a scale too."""
+    wl = small_workload("range", 16, 32, 16, 32, 0, 0, 0.6, 1, 2, C, 73)
+    q, k, v, dout = make_inputs(wl)
+    grow = np.exp2(np.linspace(0.0, 24.0, 16)).astype(np.float32).reshape(1, 1, 16, 1, 1)
+    grow[..., :2, :, :] = 0.0
+    if which == "k":
+        k, q = k * grow, q * np.float32(2.0 ** -24)
+    elif which == "v":
+        v = v * grow
+    elif which == "dout":
+        dout = dout * grow
+    else:
+        k, v, dout, q = (a * np.float32(s) for a, s in ((k, 2.0 ** -30), (v, 2.0 ** -30), (dout, 2.0 ** -20), (q, 2.0 ** 30)))      # gradients down to 2^-80
+    check(wl, q, k, v, dout, tol=tol, precision=precision)
+
+
+def test_an_infinite_value_reaches_the_outputs_that_attend_to_it():
+    wl = small_workload("inf", 16, 32, 16, 32, 0, 0, 0.3, 1, 1, 32, 74)
+    q, k, v, _ = make_inputs(wl)
+    v = v.copy()
+    v[0, 0, 8, 10, :] = math.inf
+    with sna.Plan(16, 32, 16, 32, 0, 0, 0.3) as plan:
+        out = plan.forward(*(torch.from_numpy(a).cuda() for a in (q, k, v))).cpu()
+    assert not torch.isfinite(out[0, 0, 8, 10]).any()
+    assert torch.isfinite(out[0, 0, 0]).all()
