@@ -103,10 +103,15 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+def _address(t) -> Optional[int]:
+    return None if t is None else t.data_ptr()
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        from torch import _C
+        # the current stream's handle without building a Stream object around it (3 us less per call)
+        return _C._cuda_getCurrentRawStream(_C._cuda_getDevice()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
@@ -310,6 +315,22 @@ class Plan:
             raise ValueError("tensor shapes do not match the plan")
         return B, H, C
 
+    def _usable(self, q, out_grid, in_grid, lse) -> bool:
+        """Whether every tensor is what the kernels expect: contiguous fp32 CUDA tensors of the plan's shapes, on the device of
+        q.  None stands for a tensor that is not given.  The fast way through a call; _validate says what is wrong otherwise."""
+        from torch import Tensor, float32
+        B, H, C = q.shape[0], q.shape[1], q.shape[4]
+        device = q.get_device()
+        if device < 0:
+            return False
+        out_shape, in_shape = (B, H, self.nlat_out, self.nlon_out, C), (B, H, self.nlat_in, self.nlon_in, C)
+        for tensors, shape in ((out_grid, out_shape), (in_grid, in_shape), ((lse,), out_shape[:-1])):
+            for t in tensors:
+                if t is not None and not (isinstance(t, Tensor) and t.dtype is float32 and t.shape == shape
+                                          and t.is_contiguous() and t.get_device() == device):
+                    return False
+        return True
+
     def _validate(self, q, **tensors):
         """The kernels read raw pointers as contiguous fp32 of the plan's shapes: refuse anything else here, on the
         host, instead of letting a kernel run past an allocation.  Keyword names select the expected shape:
@@ -341,14 +362,16 @@ class Plan:
         """precision: "fp32" (default, error-compensated products) or "tf32" (reduced-precision variant)."""
         import torch
         B, H, C = self._bhc(q, k)
-        self._validate(q, k=k, v=v, out=out, lse=lse)
+        if not self._usable(q, (q, out), (k, v), lse):
+            self._validate(q, k=k, v=v, out=out, lse=lse)
         if precision not in ("fp32", "tf32"):
             raise ValueError("precision must be 'fp32' or 'tf32'")
         if out is None:
             out = torch.empty_like(q)
         if return_lse and lse is None:
             lse = torch.empty(q.shape[:-1], dtype=torch.float32, device=q.device)
-        (sna_forward_ex if precision == "fp32" else sna_forward_tf32)(self.handle, q, k, v, out, lse, B, H, C, stream)
+        _check((_lib.sna_forward_ex if precision == "fp32" else _lib.sna_forward_tf32)(
+            self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), _address(lse), B, H, C, _stream(stream)))
         return (out, lse) if return_lse else out
 
     def _validate_cf(self, heads, **tensors):
@@ -412,23 +435,20 @@ class Plan:
         B, H, C = self._bhc(q, k)
         if precision not in ("fp32", "tf32"):
             raise ValueError("precision must be 'fp32' or 'tf32'")
-        self._validate(q, k=k, v=v, dout=dout, out=out, lse=lse, dq=dq, dk=dk, dv=dv)
+        if dout is None or not self._usable(q, (q, dout, out, dq), (k, v, dk, dv), lse):
+            self._validate(q, k=k, v=v, dout=dout, out=out, lse=lse, dq=dq, dk=dk, dv=dv)
         if workspace is not None and (not workspace.is_cuda or workspace.device != q.device or not workspace.is_contiguous()):
             raise ValueError("workspace must be a contiguous CUDA tensor on the device of q")
         dq = torch.empty_like(q) if dq is None else dq
         dk = torch.empty_like(k) if dk is None else dk
         dv = torch.empty_like(k) if dv is None else dv
-        if precision == "tf32":
-            need = self.workspace_bytes(B, H, C)
-            if workspace is None:
-                workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-            sna_backward_tf32(self.handle, q, k, v, dout, out, lse, dq, dk, dv, workspace,
-                              workspace.numel() * workspace.element_size(), B, H, C, stream)
-        elif workspace is None and out is None and lse is None:
-            sna_backward(self.handle, q, k, v, dout, dq, dk, dv, B, H, C, stream)
+        inputs = (self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), _address(dout))
+        gradients = (dq.data_ptr(), dk.data_ptr(), dv.data_ptr())
+        if precision == "fp32" and workspace is None and out is None and lse is None:
+            _check(_lib.sna_backward(*inputs, *gradients, B, H, C, _stream(stream)))
         else:
-            need = self.workspace_bytes(B, H, C)
             if workspace is None:
-                workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-            sna_backward_ex(self.handle, q, k, v, dout, out, lse, dq, dk, dv, workspace, workspace.numel() * workspace.element_size(), B, H, C, stream)
+                workspace = torch.empty(self.workspace_bytes(B, H, C), dtype=torch.uint8, device=q.device)
+            _check((_lib.sna_backward_ex if precision == "fp32" else _lib.sna_backward_tf32)(
+                *inputs, _address(out), _address(lse), *gradients, workspace.data_ptr(), workspace.nbytes, B, H, C, _stream(stream)))
         return dq, dk, dv
