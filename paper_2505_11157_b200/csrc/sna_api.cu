@@ -45,7 +45,7 @@ struct sna_plan {
     std::vector<int32_t> band_lengths[4];      // of the four band streams (DevBand::lengths)
     int device = 0;
     std::vector<int> zero_rings;       // input rings of quadrature weight zero (no kernel of a global plan visits them)
-    bool is_global = false;            // created by sna_plan_create_global: no column streams, dense kernels only
+    bool is_global = false;            // created by sna_plan_create_global: every window is a whole ring
     void* dev_blob = nullptr;          // one allocation holding every device table
     mutable std::mutex ws_mutex;
     mutable void* ws = nullptr;        // workspace grown on demand by sna_backward
@@ -82,7 +82,7 @@ size_t stats_elems(const sna_plan_t* plan, int B, int H) {
     return (size_t)B * H * plan->host.nlat_out * plan->host.nlon_out;
 }
 bool tf32_supported(const sna_plan_t* plan, int C) {
-    return (C == 16 || C == 32 || C == 64) && plan->host.nlon_out >= 32 && sna::band_path_supported(plan->dev, C);
+    return (C == 16 || C == 32 || C == 64) && plan->host.nlon_out >= 32 && !plan->is_global && sna::band_path_supported(plan->dev, C);
 }
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -168,9 +168,10 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
         // rows with the longest lists first: the dense kernels run one block per SM, so the long tiles must not start last
         std::stable_sort(dense.rows.begin(), dense.rows.end(), [&](int a, int b) { return dense.ptr[a + 1] - dense.ptr[a] > dense.ptr[b + 1] - dense.ptr[b]; });
         std::stable_sort(t_dense.rows.begin(), t_dense.rows.end(), [&](int a, int b) { return t_dense.ptr[a + 1] - t_dense.ptr[a] > t_dense.ptr[b + 1] - t_dense.ptr[b]; });
-        // (a global plan's windows are all whole rings: the dense kernels do all the work and no band stream, which would
-        // list every pair of the dense problem, is built)
-        if (!global) {
+        if (global) {
+            sna::build_global_bands(hp, bands[0], bands[2]);
+            t_consecutive = true;
+        } else {
             sna::build_forward_band(hp, bands[0]);
             sna::build_forward_band(hp, bands[1], dense_min_width);
             t_consecutive = sna::build_transposed_band(hp, bands[2]);
@@ -231,9 +232,11 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     for (size_t i = 0; i < 4; ++i) {
         const size_t f = first_band_piece + BAND_PIECES * i;
         plan->band_lengths[i] = std::move(bands[i].lengths);
-        *dev_bands[i] = global ? sna::DevBand{} : sna::DevBand{at(f), (const int4*)at(f + 1), (const uint32_t*)at(f + 2), at(f + 3),
-                                                               plan->band_lengths[i].data(), (int)bands[i].order.size(),
-                                                               (long long)bands[i].chunk_ptr.back()};
+        const sna::BandStream& b = bands[i];
+        if (b.chunk_ptr.empty()) continue;
+        const int groups = (int)b.order.size();
+        *dev_bands[i] = sna::DevBand{at(f), (const int4*)at(f + 1), (const uint32_t*)at(f + 2), at(f + 3), plan->band_lengths[i].data(),
+                                     groups, b.one_row, (long long)b.chunk_ptr.back() * (b.one_row ? groups : 1)};
     }
     e = cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, plan->device);
     if (e != cudaSuccess) { sna_plan_destroy(plan); return cuda_fail(e, "cudaDeviceGetAttribute"); }
@@ -379,12 +382,10 @@ sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float*
     if (!q || !k || !v || !out) { set_error("q, k, v and out must not be NULL"); return SNA_ERR_INVALID_ARG; }
     if (!all_aligned(q, k, v, out) || (reinterpret_cast<uintptr_t>(lse) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     cudaError_t e;
-    if (sna::dense2_global_supported(plan->dev, C)) {
+    if (sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::FORWARD)) {
         // every window is a whole ring (a global plan, or a cutoff that reaches every point): the dense kernel alone
         // produces the final out and, if asked for, lse (64x128, N = 4, without lse: 5.44 ms on the generic kernel, 0.25 ms here)
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (plan->is_global) {
-        e = sna::launch_forward_generic(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
     } else if (lse != nullptr && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its partial result travels in out / lse), the rest on the band kernel
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
@@ -413,10 +414,8 @@ sna_status_t sna_backward_dq(const sna_plan_t* plan, const float* q, const float
     cudaError_t e;
     // The dense dq kernel takes the whole-ring and wide windows when they are at least a tenth of the work (measured on the
     // benchmark configurations: -8 % on the dq stage at a 22 % share, -6 % at 13 %).
-    if (out != nullptr && out != dq && sna::dense2_global_supported(plan->dev, C)) {
+    if (out != nullptr && out != dq && sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::DQ)) {
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (plan->is_global) {
-        e = sna::launch_backward_dq_generic(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
     } else if (out != nullptr && out != dq && plan->dev.dense_fraction >= 0.10f && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dq is written first), the rest is added by the band kernel
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, nullptr, B * H, C, (cudaStream_t)cuda_stream);
@@ -438,19 +437,16 @@ sna_status_t sna_backward_dkdv(const sna_plan_t* plan, const float* q, const flo
     if (!q || !k || !v || !dout || !lse || !D || !dk || !dv) { set_error("q, k, v, dout, lse, D, dk and dv must not be NULL"); return SNA_ERR_INVALID_ARG; }
     if (!all_aligned(q, k, v, dout, dk, dv) || ((reinterpret_cast<uintptr_t>(lse) | reinterpret_cast<uintptr_t>(D)) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     cudaError_t e;
-    if (plan->is_global || sna::dense2_global_supported(plan->dev, C)) {
+    if (sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::DKDV)) {
         // the dense kernel writes only the rings some window refers to; rings of weight zero get their (zero) gradient here
-        const bool dense = sna::dense2_global_supported(plan->dev, C);
         const size_t ring_bytes = (size_t)plan->host.nlon_in * C * sizeof(float), pitch = ring_bytes * plan->host.nlat_in;
-        for (size_t i = 0; dense && i < plan->zero_rings.size(); ++i) {
+        for (size_t i = 0; i < plan->zero_rings.size(); ++i) {
             const size_t off = ring_bytes * plan->zero_rings[i];
             e = cudaMemset2DAsync((char*)dk + off, pitch, 0, ring_bytes, (size_t)B * H, (cudaStream_t)cuda_stream);
             if (e == cudaSuccess) e = cudaMemset2DAsync((char*)dv + off, pitch, 0, ring_bytes, (size_t)B * H, (cudaStream_t)cuda_stream);
             if (e != cudaSuccess) return cuda_fail(e, "clearing the gradients of zero-weight rings");
         }
-        e = dense
-                ? sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream)
-                : sna::launch_backward_dkdv_generic(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
+        e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
     } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dk, dv is written first), the band kernel adds the rest
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
@@ -478,13 +474,14 @@ sna_status_t sna_backward_ex(const sna_plan_t* plan, const float* q, const float
     float* ws_lse = (float*)workspace;
     float* ws_D = ws_lse + stats_elems(plan, B, H);
     cudaError_t e;
-    if (plan->is_global) {
+    const bool dense_alone = sna::dense2_global_chosen(plan->dev, C, N, sna::Pass::FORWARD);
+    if (plan->is_global && (dense_alone || !sna::band_path_supported(plan->dev, C))) {
         if (lse == nullptr || out == nullptr) {
             // recompute the forward pass.  The dense dq kernel may not read out from the dq buffer, so out goes into
             // the dk buffer (written only after the dq stage) when that is large enough; otherwise only the
             // statistics are recomputed and the generic dq kernel runs.
             const bool fits = (long long)plan->host.nlat_in * plan->host.nlon_in >= (long long)plan->host.nlat_out * plan->host.nlon_out;
-            if (fits && sna::dense2_global_supported(plan->dev, C)) {
+            if (fits && dense_alone) {
                 e = sna::launch_forward_dense2(plan->dev, q, k, v, dk, ws_lse, N, C, stream);
                 out = dk;
             } else {

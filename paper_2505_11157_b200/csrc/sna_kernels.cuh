@@ -13,6 +13,7 @@ struct DevBand {
     const int32_t* order;           // ring groups, longest stream first
     const int32_t* lengths;         // in host memory: chunks per stream row of order[i]
     int groups;
+    int one_row;                    // 1: every group walks row 0 (global attention)
     long long chunks;               // of all stream rows
 };
 
@@ -32,7 +33,7 @@ struct DevPlan {
     const int32_t* t_row_order; // input latitudes, most work first
     const float* log2_omega;    // [nlat_in] log2 of the per-point quadrature weight
     // band streams of the mma.sync kernels (see sna_plan.hpp): forward and transposed, each with all windows and with the ones
-    // the dense kernels serve left out; null if not built
+    // the dense kernels serve left out (null for a global plan)
     DevBand fwd, fwdb, t, tb;
     // the dense kernels' lists
     const int32_t* dense_ptr;       // [nlat_out+1] the dense kernels' windows per output latitude
@@ -50,7 +51,7 @@ struct DevPlan {
     float dense_fraction;           // share of the table's entries that the dense kernels' windows cover
     int* dev_status;                // set to non-zero by a kernel whose bounded wait ran out
     int t_consecutive;              // 1: transposed tiles are 8 consecutive input columns; 0: split by residue mod ps
-    int is_global;                  // 1: every window is a whole ring and no column stream exists (dense kernels or generic kernels only)
+    int is_global;                  // 1: every window is a whole ring; the band streams have one row
 };
 
 // Band kernels (sna_kernels_band.cu: mma.sync; C <= 64); same contracts as the generic launchers.
@@ -77,6 +78,8 @@ cudaError_t dense2_prepare_device();   // once per device: opt in to the kernels
 bool dense2_path_chosen(const DevPlan& p, int C, int N);
 cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t stream);
 bool dense2_global_supported(const DevPlan& p, int C);   // every window is a whole ring and the dense kernels can do all the work
+enum class Pass { FORWARD, DQ, DKDV };
+bool dense2_global_chosen(const DevPlan& p, int C, int N, Pass pass);   // ... and are faster than the band kernels
 cudaError_t launch_forward_dense2(const DevPlan& p, const float* q, const float* k, const float* v, float* out, float* lse,
                                   int N, int C, cudaStream_t stream);
 // The same split for the dq stage: the dense kernel writes its part of dq (out and dq must be different buffers) and,

@@ -541,6 +541,7 @@ struct Task {
         return true;
     }
     __device__ __forceinline__ void chunks(const BandView& v, int row, int& first, int& count) const {
+        if (v.s.one_row) row = 0;
         first = v.s.chunk_ptr[row];
         count = v.s.chunk_ptr[row + 1] - first;
         if (shared) {
@@ -1048,7 +1049,8 @@ cudaError_t dispatch(int C, bool lp, F&& f) {
 // of a small launch.  Whole streams, us without : with sharing: 32x64, N = 1, C = 16, forward 17.0 : 9.0; 256x512 -> 128x256,
 // N = 4, C = 32, forward 316 : 226; 128x256, N = 4, dk/dv 127.6 : 126.8.  A limit of 0.25 or 0.5 costs large launches
 // 2 to 4 % (each sharer repeats the prologue), 2 leaves the down-sampling case at 308.
-constexpr double SHARE_ABOVE = 1, SHARE_MIN = 8;
+// Equally long streams (global attention) leave a last wave of blocks that is nearly empty, up to four waves or so.
+constexpr double SHARE_ABOVE = 1, SHARE_EQUAL_ABOVE = 0.25, SHARE_MIN = 8;
 
 int ceil_div_host(int a, int b) { return (a + b - 1) / b; }
 
@@ -1063,7 +1065,8 @@ bool make_view(const DevPlan& p, bool transposed, bool band, int N, int blocks_p
     if (total > 0x7fffffffLL) return false;
     // Share the streams that alone would take long in comparison with the whole launch.
     const double fair = (double)v.s.chunks * (transposed && !p.t_consecutive ? v.tiles / p.ps : v.tiles) * N / ((double)p.num_sms * blocks_per_sm * WARPS);
-    const double longest = fair * SHARE_ABOVE > SHARE_MIN ? fair * SHARE_ABOVE : SHARE_MIN;
+    const double above = v.s.one_row ? SHARE_EQUAL_ABOVE : SHARE_ABOVE;
+    const double longest = fair * above > SHARE_MIN ? fair * above : SHARE_MIN;
     int heavy = 0;
     while (heavy < v.s.groups && v.s.lengths[heavy] >= longest) ++heavy;
     v.shared = (int)(heavy * per_group);
@@ -1085,7 +1088,7 @@ cudaError_t band_prepare_device() {
 }
 
 bool band_path_supported(const DevPlan& p, int C) {
-    return p.fwd.columns != nullptr && !p.is_global && C >= 4 && C <= 64 && C % 4 == 0 && p.nlon_out >= 16 &&
+    return p.fwd.columns != nullptr && C >= 4 && C <= 64 && C % 4 == 0 && p.nlon_out >= 16 &&
            (long long)p.nlat_in * p.nlon_in * C < (1LL << 32) && (long long)p.nlat_out * p.nlon_out * C < (1LL << 32);
 }
 

@@ -1389,7 +1389,7 @@ cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t 
 }
 
 bool dense2_path_chosen(const DevPlan& p, int C, int N) {
-    if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
+    if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || p.dense_fraction >= 0.999f || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
     // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time; below that much work per
     // SM the band kernels alone, which share long streams between warps, are faster.  Measured (fwd / dq / dkdv us, with : without
     // the dense kernels; work in longest lists per SM): 128x256, cutoff 4 rings, N = 1 (0.1) 57/62/80 : 32/36/40, N = 4 (0.4)
@@ -1403,6 +1403,27 @@ bool dense2_path_chosen(const DevPlan& p, int C, int N) {
 bool dense2_global_supported(const DevPlan& p, int C) {
     return C == C2 && (p.is_global || p.dense_fraction >= 0.999f) && p.n_dense_rows > 0 && p.n_t_dense_rows > 0 && encode_fn2() != nullptr &&
            (long long)p.nlat_in * p.nlon_in * C < (1LL << 32) && (long long)p.nlat_out * p.nlon_out * C < (1LL << 32);
+}
+
+bool dense2_global_chosen(const DevPlan& p, int C, int N, Pass pass) {
+    if (!dense2_global_supported(p, C)) return false;
+    if (!band_path_supported(p, C)) return true;
+    // Both sides are a number of equal units of work of known duration (us).  Dense: each block walks all rings of the other grid in
+    // units of `unit` columns, one block per SM at a time; rings that are no multiple of the unit leave it partly empty, and the
+    // forward kernel masks then.  Band: 256 pairs per unit over the whole GPU.  Measured dense : band, fwd / dq / dkdv:
+    // 24x48 N = 4 73/38/57 : 21/23/23, 32x64 N = 16 339/170/277 : 149/165/196, 51x102 N = 4 263/224/402 : 242/287/342,
+    // 64x128 N = 1 131/132/255 : 154/182/230, N = 4 251/262/504 : 511/609/732, 90x180 N = 1 859/573/1047 : 502/597/739.
+    const bool whole = p.nlon_in % M2 == 0 && p.nlon_out % M2 == 0;
+    const int unit = pass == Pass::FORWARD ? 128 : pass == Pass::DQ ? 64 : 32;
+    const double dense_unit = pass == Pass::FORWARD ? (whole ? 2.0 : 2.7) : pass == Pass::DQ ? 1.05 : 1.0;
+    const double band_unit = pass == Pass::FORWARD ? 0.50e-3 : pass == Pass::DQ ? 0.61e-3 : 0.745e-3;
+    const bool gather = pass == Pass::DKDV;      // tiles of input points, columns of output points
+    const int rows = gather ? p.nlat_in : p.nlat_out, row_len = gather ? p.nlon_in : p.nlon_out;
+    const int rings = gather ? p.nlat_out : p.nlat_in, ring_len = gather ? p.nlon_out : p.nlon_in;
+    const long long blocks = (long long)rows * ((row_len + M2 - 1) / M2) * N, waves = (blocks + p.num_sms - 1) / p.num_sms;
+    const double dense = (double)waves * rings * ((ring_len + unit - 1) / unit) * dense_unit;
+    const double band = (double)rows * row_len * rings * ring_len / 256 * N * band_unit;
+    return dense <= band;
 }
 
 cudaError_t launch_backward_dq_dense2(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,

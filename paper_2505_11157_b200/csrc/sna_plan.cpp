@@ -324,11 +324,15 @@ private:
     std::vector<uint32_t> masks_;
 };
 
-void complete(BandStream& S, int rows_per_group) {
-    // the kernels read three chunks ahead
+// the kernels read three chunks ahead
+void pad(BandStream& S) {
     const BandColumn last = S.columns.empty() ? BandColumn{0, 0, 0.f, 0} : S.columns.back();
     S.columns.insert(S.columns.end(), 3 * BAND_CHUNK, last);
     S.masks.insert(S.masks.end(), 3 * 32, 0u);
+}
+
+void complete(BandStream& S, int rows_per_group) {
+    pad(S);
     S.order.resize((S.chunk_ptr.size() - 1) / rows_per_group);
     for (size_t i = 0; i < S.order.size(); ++i) S.order[i] = (int32_t)i;
     auto length = [&](int g) { return S.chunk_ptr[(size_t)(g + 1) * rows_per_group] - S.chunk_ptr[(size_t)g * rows_per_group]; };
@@ -372,6 +376,25 @@ void build_transposed_dense_lists(const HostPlan& P, DenseLists& D, int dense_mi
         D.ptr[hp + 1] = (int32_t)D.lat.size();
         if (D.ptr[hp + 1] > D.ptr[hp]) D.rows.push_back(hp);
     }
+}
+
+void build_global_bands(const HostPlan& P, BandStream& forward, BandStream& transposed) {
+    const int whole[TILE_LAT] = {-1, -1};
+    auto one_row = [](BandBuilder& b, BandStream& S, int rings) {
+        S = BandStream();
+        b.finish(S);
+        pad(S);
+        S.one_row = true;
+        S.order.assign(ceil_div(rings, TILE_LAT), 0);
+        for (size_t i = 0; i < S.order.size(); ++i) S.order[i] = (int32_t)i;
+        S.lengths.assign(S.order.size(), S.chunk_ptr[1]);
+    };
+    BandBuilder f, t;
+    for (int lat = 0; lat < P.nlat_in; ++lat)
+        for (int r = 0; r < P.ps && P.omega[lat] > 0.0; ++r) f.add_whole(lat * P.nlon_in + r, (float)std::log2(P.omega[lat]), whole, P.nlon_out);
+    for (int lat = 0; lat < P.nlat_out; ++lat) t.add_whole(lat * P.nlon_out, 0.f, whole, P.nlon_out);
+    one_row(f, forward, P.nlat_out);
+    one_row(t, transposed, P.nlat_in);
 }
 
 void build_forward_band(const HostPlan& P, BandStream& S, int dense_min_width) {

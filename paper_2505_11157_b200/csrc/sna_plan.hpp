@@ -66,6 +66,7 @@ struct BandStream {
     std::vector<uint32_t> masks;        // 32 per chunk
     std::vector<int32_t> order;         // ring groups, longest stream first
     std::vector<int32_t> lengths;       // chunks per stream row of order[i]
+    bool one_row = false;               // every group walks row 0 (global attention)
 };
 
 // Forward stream: one row per group of TILE_LAT output latitudes; partners are input points, flat index base + u*ps.
@@ -81,6 +82,9 @@ void build_forward_band(const HostPlan& plan, BandStream& out, int dense_min_wid
 //    the partner index is u0 + e.
 // Returns true for the consecutive layout.
 bool build_transposed_band(const HostPlan& plan, BandStream& out, int dense_min_width = 0);
+// Streams of a global plan: the same for every group, so that only one row is stored (the points of the partner grid, once).
+// The transposed one has the consecutive layout.
+void build_global_bands(const HostPlan& plan, BandStream& forward, BandStream& transposed);
 
 // Which windows the dense (tcgen05) kernels take: whole rings, and banded windows of at least dense_min_width input
 // columns (they run as masked blocks there).  dense_min_width = nlon_in + 1 selects the whole rings only.

@@ -91,3 +91,24 @@ def test_an_infinite_value_reaches_the_outputs_that_attend_to_it():
         out = plan.forward(*(torch.from_numpy(a).cuda() for a in (q, k, v))).cpu()
     assert not torch.isfinite(out[0, 0, 8, 10]).any()
     assert torch.isfinite(out[0, 0, 0]).all()
+
+
+@pytest.mark.parametrize("shape", [(5, 17, 5, 17), (9, 48, 4, 16), (8, 36, 5, 36), (3, 128, 3, 128)], ids=["odd", "down3", "ragged", "one_tile"])
+@pytest.mark.parametrize("C, slices, grid", [(8, 1, 0), (20, 3, 1), (32, 2, 2), (64, 40, 0)])
+@pytest.mark.parametrize("recompute", [False, True])
+def test_global_attention_on_the_band_kernels(shape, C, slices, grid, recompute):
+    """A global plan's single stream: shared by all ring groups, split over a block's warps or not, zero-weight rings left out."""
+    wl = small_workload("global_band", *shape, grid, 0, math.pi, 1, slices, C, 75)
+    q, k, v, dout = make_inputs(wl)
+    g = orc.geometry(*shape, grid, 0, math.pi)
+    dev = [torch.from_numpy(a).cuda() for a in (q, k, v, dout)]
+    with sna.Plan(*shape, grid, 0, global_attention=True) as plan:
+        out, lse = plan.forward(*dev[:3], return_lse=True)
+        grads = plan.backward(*dev, **({} if recompute else {"out": out, "lse": lse}))
+        torch.cuda.synchronize()
+        sna.sna_plan_check(plan.handle)
+    assert rel(out, orc.forward(g, q, k, v)) <= TOL
+    for name, x, r in zip(("dq", "dk", "dv"), grads, orc.backward(g, q, k, v, dout)):
+        assert rel(x, r) <= (TOL if C != 32 else 1e-5), name       # (C = 32: a pass may run on the dense kernels, 2^-21 per operand)
+    if grid == 2:
+        assert not grads[1][..., 0, :, :].any() and not grads[2][..., 0, :, :].any()
