@@ -207,11 +207,18 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     if (e != cudaSuccess) { delete plan; return cuda_fail(e, "cudaGetDevice"); }
     e = cudaMalloc(&plan->dev_blob, total);
     if (e != cudaSuccess) { delete plan; set_error("cudaMalloc of %zu bytes: %s", total, cudaGetErrorString(e)); return SNA_ERR_ALLOC; }
-    for (const Piece& p : pieces) {
-        if (p.bytes == 0) continue;
-        e = cudaMemcpy((char*)plan->dev_blob + p.offset, p.src, p.bytes, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { cudaFree(plan->dev_blob); delete plan; return cuda_fail(e, "cudaMemcpy of plan tables"); }
+    try {
+        std::vector<char> blob(total);       // one copy instead of one per piece
+        for (const Piece& p : pieces)
+            if (p.bytes != 0) std::memcpy(blob.data() + p.offset, p.src, p.bytes);
+        e = cudaMemcpy(plan->dev_blob, blob.data(), total, cudaMemcpyHostToDevice);
+    } catch (const std::bad_alloc&) {
+        cudaFree(plan->dev_blob);
+        delete plan;
+        set_error("out of host memory while uploading the plan");
+        return SNA_ERR_ALLOC;
     }
+    if (e != cudaSuccess) { cudaFree(plan->dev_blob); delete plan; return cuda_fail(e, "cudaMemcpy of plan tables"); }
     auto at = [&](size_t i) { return (const int32_t*)((char*)plan->dev_blob + pieces[i].offset); };
     sna::DevPlan& d = plan->dev;
     d.nlat_in = hp.nlat_in; d.nlon_in = hp.nlon_in; d.nlat_out = hp.nlat_out; d.nlon_out = hp.nlon_out; d.ps = hp.ps;

@@ -64,12 +64,14 @@ void legendre_gauss(int n, std::vector<double>& x, std::vector<double>& w) {
 void clenshaw_curtis(int nlat, std::vector<double>& w) {
     const int n = nlat - 1;
     w.resize(nlat);
+    std::vector<long double> cosine(2 * n);              // of i pi / n: all that the sums need
+    for (int i = 0; i < 2 * n; ++i) cosine[i] = cosl(PI_L * (long double)i / (long double)n);
     for (int h = 0; h <= n; ++h) {
         long double acc = 1.0L;
         for (int k = 1; k <= n / 2; ++k) {
             long long arg = (2LL * k * h) % (2LL * n);           // cos(2 k pi h / n) with an exactly reduced argument
             long double bk = (2 * k == n) ? 1.0L : 2.0L;
-            acc -= bk * cosl(PI_L * (long double)arg / (long double)n) / (4.0L * k * k - 1.0L);
+            acc -= bk * cosine[arg] / (4.0L * k * k - 1.0L);
         }
         long double ch = (h == 0 || h == n) ? 1.0L : 2.0L;
         w[h] = (double)(ch * acc / n);
@@ -145,6 +147,8 @@ PlanStatus build_plan(int nlat_in, int nlon_in, int nlat_out, int nlon_out, int 
     P.row_ptr.assign(nlat_out + 1, 0);
     P.row_nnz.assign(nlat_out, 0);
     std::vector<std::vector<RingWindow>> by_input(nlat_in);
+    std::vector<double> sin_in(nlat_in), cos_in(nlat_in);
+    for (int hp = 0; hp < nlat_in; ++hp) { sin_in[hp] = std::sin(P.theta_in[hp]); cos_in[hp] = std::cos(P.theta_in[hp]); }
     for (int h = 0; h < nlat_out; ++h) {
         const double so = std::sin(P.theta_out[h]), co = std::cos(P.theta_out[h]);
         for (int hp = 0; hp < nlat_in; ++hp) {
@@ -152,7 +156,9 @@ PlanStatus build_plan(int nlat_in, int nlon_in, int nlat_out, int nlon_out, int 
             if (everything) {
                 m = -1;
             } else {
-                const double si = std::sin(P.theta_in[hp]), ci = std::cos(P.theta_in[hp]);
+                // the nearest point is as far as the colatitudes differ: no need to evaluate rings that are clearly outside
+                if (std::fabs(P.theta_out[h] - P.theta_in[hp]) > theta_cutoff + 1e-3) continue;
+                const double si = sin_in[hp], ci = cos_in[hp];
                 if (!member(geodesic(so, co, si, ci, 0.0))) continue;   // nearest point of the ring is outside
                 const double denom = so * si;
                 int guess;
@@ -277,42 +283,49 @@ public:
     // tile longitude i uses.
     template <typename Range>
     void add_band(int32_t base, float bias, const int (&m)[TILE_LAT], Range&& band_range) {
-        int rlo[TILE_LAT][TILE_LON], rhi[TILE_LAT][TILE_LON], lo = INT32_MAX, hi = INT32_MIN;
-        for (int k = 0; k < TILE_LAT; ++k)
-            for (int i = 0; i < TILE_LON; ++i) {
-                rlo[k][i] = 0; rhi[k][i] = -1;          // empty
-                if (m[k] < 0) continue;
-                band_range(m[k], i, rlo[k][i], rhi[k][i]);
-                if (rhi[k][i] >= rlo[k][i]) { lo = std::min(lo, rlo[k][i]); hi = std::max(hi, rhi[k][i]); }
-            }
+        int rlo[TILE_LAT * TILE_LON], rhi[TILE_LAT * TILE_LON], lo = INT32_MAX, hi = INT32_MIN;
+        for (int row = 0; row < TILE_LAT * TILE_LON; ++row) {
+            rlo[row] = 0; rhi[row] = -1;          // empty
+            if (m[row / TILE_LON] < 0) continue;
+            band_range(m[row / TILE_LON], row % TILE_LON, rlo[row], rhi[row]);
+            if (rhi[row] >= rlo[row]) { lo = std::min(lo, rlo[row]); hi = std::max(hi, rhi[row]); }
+        }
+        if (hi < lo) return;
+        // where each row's range begins and ends; the running exclusive-or is the mask
+        toggle_.assign((size_t)(hi - lo) + 2, 0u);
+        for (int row = 0; row < TILE_LAT * TILE_LON; ++row)
+            if (rhi[row] >= rlo[row]) { toggle_[rlo[row] - lo] ^= 1u << row; toggle_[rhi[row] + 1 - lo] ^= 1u << row; }
+        uint32_t mask = 0;
         for (int e = lo; e <= hi; ++e) {
-            uint32_t mask = 0;
-            for (int k = 0; k < TILE_LAT; ++k)
-                for (int i = 0; i < TILE_LON; ++i)
-                    if (e >= rlo[k][i] && e <= rhi[k][i]) mask |= 1u << (k * TILE_LON + i);
+            mask ^= toggle_[e - lo];
             if (mask) add(base, e, bias, mask);
         }
     }
+    // Appends the columns to the stream as a row, and starts anew.
     void finish(BandStream& S) {
         if (S.chunk_ptr.empty()) S.chunk_ptr.push_back(0);
-        for (size_t c = 0; c < cols_.size(); c += BAND_CHUNK) {
-            uint32_t mask[BAND_CHUNK], all = 0xffffu;
-            for (size_t j = 0; j < BAND_CHUNK; ++j) {          // padding repeats the last column with an empty mask
-                const bool exists = c + j < cols_.size();
-                S.columns.push_back(exists ? cols_[c + j] : cols_.back());
-                mask[j] = exists ? masks_[c + j] : 0u;
-                all &= mask[j];
+        // padding repeats the last column with an empty mask
+        while (cols_.size() % BAND_CHUNK != 0) { cols_.push_back(BandColumn(cols_.back())); masks_.push_back(0u); }
+        S.columns.insert(S.columns.end(), cols_.begin(), cols_.end());
+        for (size_t c = 0; c < masks_.size(); c += BAND_CHUNK) {
+            const uint32_t* mask = masks_.data() + c;
+            uint32_t all = 0xffffu;
+            for (size_t j = 0; j < BAND_CHUNK; ++j) all &= mask[j];
+            uint32_t lanes[32];
+            for (int t = 0; t < 4; ++t) {
+                // the four columns of lanes 4 g + t, each as two bytes of rows: an 8 x 8 bit matrix whose columns are the lanes' masks
+                const uint64_t rows = (mask[2 * t] & 0xffu) | (uint64_t)(mask[2 * t + 1] & 0xffu) << 8 | (uint64_t)(mask[2 * t] >> 8) << 16 |
+                                      (uint64_t)(mask[2 * t + 1] >> 8) << 24 | (uint64_t)(mask[8 + 2 * t] & 0xffu) << 32 |
+                                      (uint64_t)(mask[9 + 2 * t] & 0xffu) << 40 | (uint64_t)(mask[8 + 2 * t] >> 8) << 48 |
+                                      (uint64_t)(mask[9 + 2 * t] >> 8) << 56;
+                const uint64_t bytes = transpose_bits(rows);
+                for (int g = 0; g < 8; ++g) lanes[4 * g + t] = (uint32_t)(bytes >> 8 * g & 0xffu) | (all == 0xffffu ? BAND_ALL : 0u);
             }
-            for (int lane = 0; lane < 32; ++lane) {
-                uint32_t bits = all == 0xffffu ? BAND_ALL : 0u;
-                for (int j = 0; j < 2; ++j)
-                    for (int r = 0; r < 2; ++r)
-                        for (int k = 0; k < 2; ++k)
-                            bits |= (mask[8 * j + 2 * (lane & 3) + k] >> (8 * r + lane / 4) & 1u) << (4 * j + 2 * r + k);
-                S.masks.push_back(bits);
-            }
+            S.masks.insert(S.masks.end(), lanes, lanes + 32);
         }
         S.chunk_ptr.push_back((int32_t)(S.columns.size() / BAND_CHUNK));
+        cols_.clear();
+        masks_.clear();
     }
 
 private:
@@ -320,8 +333,17 @@ private:
         cols_.push_back(BandColumn{base, e, bias, 0});
         masks_.push_back(mask);
     }
+    // byte i, bit j -> byte j, bit i (three rounds of swapping blocks, as one does by hand)
+    static uint64_t transpose_bits(uint64_t x) {
+        auto swap = [&](uint64_t where, int by) { const uint64_t d = (x ^ (x >> by)) & where; x ^= d ^ (d << by); };
+        swap(0x00aa00aa00aa00aaull, 7);
+        swap(0x0000cccc0000ccccull, 14);
+        swap(0x00000000f0f0f0f0ull, 28);
+        return x;
+    }
     std::vector<BandColumn> cols_;
     std::vector<uint32_t> masks_;
+    std::vector<uint32_t> toggle_;
 };
 
 // the kernels read three chunks ahead
@@ -399,8 +421,8 @@ void build_global_bands(const HostPlan& P, BandStream& forward, BandStream& tran
 
 void build_forward_band(const HostPlan& P, BandStream& S, int dense_min_width) {
     S = BandStream();
+    BandBuilder b;
     for (int first = 0; first < P.nlat_out; first += TILE_LAT) {
-        BandBuilder b;
         merge_group(P.row_ptr, P.windows, first, P.nlat_out, dense_min_width, [&](int lat, const int (&m)[TILE_LAT]) {
             const float bias = (float)std::log2(P.omega[lat]);
             for (int r = 0; r < P.ps; ++r) {
@@ -419,9 +441,9 @@ void build_forward_band(const HostPlan& P, BandStream& S, int dense_min_width) {
 bool build_transposed_band(const HostPlan& P, BandStream& S, int dense_min_width) {
     S = BandStream();
     const bool consecutive = TILE_LON % P.ps == 0;
+    BandBuilder b;
     for (int first = 0; first < P.nlat_in; first += TILE_LAT)
         for (int r = 0; r < (consecutive ? 1 : P.ps); ++r) {
-            BandBuilder b;
             merge_group(P.t_row_ptr, P.t_windows, first, P.nlat_in, dense_min_width, [&](int lat, const int (&m)[TILE_LAT]) {
                 // Output point w is a partner of input column c iff c - w*ps lies in [-m, m].  Consecutive: c = c0 + i, so
                 // w - c0/ps in [ceil((i - m)/ps), floor((i + m)/ps)].  By residue: c = ps*(u0+i) + r, so w - u0 in
