@@ -251,6 +251,7 @@ class Plan:
         self.grid_in, self.grid_out, self.theta_cutoff = grid_in, grid_out, float(theta_cutoff)
         self.host_only = host_only
         self.handle = None
+        self.native = None      # the autograd function's owner of the handle, once there is one
         if global_attention:
             self.handle = sna_plan_create_global(nlat_in, nlon_in, nlat_out, nlon_out, grid_in, grid_out)
         else:
@@ -260,11 +261,15 @@ class Plan:
     def close(self):
         if self.handle is not None:
             handle, self.handle = self.handle, None
-            sna_plan_destroy(handle)
+            if self.native is not None:
+                _check(self.native.close())
+            else:
+                sna_plan_destroy(handle)
 
     def __del__(self):
         try:
-            self.close()
+            if self.native is None:      # (otherwise with the last graph that uses the plan)
+                self.close()
         except Exception:
             pass
 
