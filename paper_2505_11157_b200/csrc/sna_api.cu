@@ -502,10 +502,19 @@ sna_status_t sna_backward_ex(const sna_plan_t* plan, const float* q, const float
         if (lse == nullptr || out == nullptr) {
             // recompute the forward pass: lse into the workspace, out into the dq buffer, which the dq stage
             // reads row by row before it overwrites the same rows with dq
-            e = sna::launch_forward_band(plan->dev, q, k, v, dq, ws_lse, N, C, false, false, stream);
+            // (into the dk buffer, which is written only after that stage, if the dense kernels help: they may not read out from
+            // the buffer that they write dq to.  256x512 -> 128x256, N = 4: 733 -> 677 us)
+            const bool fits = (long long)plan->host.nlat_in * plan->host.nlon_in >= (long long)plan->host.nlat_out * plan->host.nlon_out;
+            if (fits && sna::dense2_path_chosen(plan->dev, C, N)) {
+                e = sna::launch_forward_dense2(plan->dev, q, k, v, dk, ws_lse, N, C, stream);
+                if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, dk, ws_lse, N, C, true, false, stream);
+                out = dk;
+            } else {
+                e = sna::launch_forward_band(plan->dev, q, k, v, dq, ws_lse, N, C, false, false, stream);
+                out = dq;
+            }
             if (e != cudaSuccess) return cuda_fail(e, "statistics launch");
             lse = ws_lse;
-            out = dq;
         }
     } else if (lse == nullptr) {   // recompute the softmax statistics
         e = sna::launch_forward_generic(plan->dev, q, k, v, nullptr, ws_lse, N, C, stream);

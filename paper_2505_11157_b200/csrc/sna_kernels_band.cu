@@ -524,7 +524,13 @@ struct BandView {
     int tiles, N;                 // longitude tiles per ring group, slices
     int shared;                   // the first tasks, one per block: its warps share the tile's stream
     int total;                    // tasks
+    // whether one of the two rings from h0 on has windows on the dense kernels
+    __device__ __forceinline__ bool has_dense(int h0, int nlat) const { return dense_ptr[min(h0 + 2, nlat)] > dense_ptr[h0]; }
 };
+// The band kernel is launched to start when the dense kernel before it leaves SMs idle (programmatic dependent launch).  Tiles with
+// windows on the dense kernel wait here until that has finished and its results are visible; the others need nothing from it.
+// There is always one that waits, so the band kernel never finishes first.
+__device__ __forceinline__ void wait_for_dense() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A warp's task: longitude tile, slice and ring group (heavy-first order), and its part of the tile's stream.
 struct Task {
     int tile, n, group, warp;
@@ -659,6 +665,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
         l0 = l1 = bad = 0;
         const bool seeded = view.dense_ptr != nullptr && (!task.shared || task.warp == 0);
         if (seeded) {
+            if (view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
             // continue from the dense kernel's partial result of this row (normalised out and lse), one weight of value 2^lse
             const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
             if (view.dense_ptr[at.ha + 1] > view.dense_ptr[at.ha]) {
@@ -884,7 +891,8 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
         x.add(acc, task, 0);
         f0 = f1 = 1.f;
     }
-    // the dense kernel has already written its part of dq for rows that have windows there: add it
+    // the dense kernel has written its part of dq for rows that have windows there: add it
+    if (view.dense_ptr != nullptr && view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
     const bool add0 = view.dense_ptr != nullptr && view.dense_ptr[at.ha + 1] > view.dense_ptr[at.ha];
     const bool add1 = view.dense_ptr != nullptr && view.dense_ptr[at.hb + 1] > view.dense_ptr[at.hb];
 #pragma unroll
@@ -1002,6 +1010,7 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
         x.add(gv, task, CP / 2);
         fk = fv = 1.f;
     }
+    if (view.dense_ptr != nullptr && view.has_dense(group * TILE_LAT, p.nlat_in)) wait_for_dense();
     const bool add0 = view.dense_ptr != nullptr && view.dense_ptr[at.ha + 1] > view.dense_ptr[at.ha];
     const bool add1 = view.dense_ptr != nullptr && view.dense_ptr[at.hb + 1] > view.dense_ptr[at.hb];
 #pragma unroll
@@ -1075,6 +1084,21 @@ bool make_view(const DevPlan& p, bool transposed, bool band, int N, int blocks_p
     return true;
 }
 
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), unsigned grid, size_t smem, bool after_dense, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config{};
+    config.gridDim = grid;
+    config.blockDim = THREADS;
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &overlap;
+    config.numAttrs = after_dense ? 1 : 0;
+    return cudaLaunchKernelEx(&config, kernel, P(args)...);
+}
+
 }  // namespace
 
 cudaError_t band_prepare_device() {
@@ -1099,9 +1123,7 @@ cudaError_t launch_forward_band(const DevPlan& p, const float* q, const float* k
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::FWD, view, grid)) return cudaErrorInvalidValue;
-        forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value>
-            <<<grid, THREADS, smem_bytes<CP>(), stream>>>(p, view, q, k, v, out, lse, C, LOG2E / sqrtf((float)C));
-        return cudaGetLastError();
+        return launch(forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, out, lse, C, LOG2E / sqrtf((float)C));
     });
 }
 
@@ -1113,9 +1135,7 @@ cudaError_t launch_backward_dq_band(const DevPlan& p, const float* q, const floa
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::DQ, view, grid)) return cudaErrorInvalidValue;
-        backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value>
-            <<<grid, THREADS, smem_bytes<CP>(), stream>>>(p, view, q, k, v, dout, out, lse, dq, Dws, C, 1.0f / sqrtf((float)C));
-        return cudaGetLastError();
+        return launch(backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, out, lse, dq, Dws, C, 1.0f / sqrtf((float)C));
     });
 }
 
@@ -1127,9 +1147,7 @@ cudaError_t launch_backward_dkdv_band(const DevPlan& p, const float* q, const fl
         BandView view;
         unsigned grid;
         if (!make_view(p, true, after_dense, N, Blocks<CP, decltype(low)::value>::DKDV, view, grid)) return cudaErrorInvalidValue;
-        backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value>
-            <<<grid, THREADS, smem_bytes<CP>(), stream>>>(p, view, q, k, v, dout, lse, Dws, dk, dv, C, 1.0f / sqrtf((float)C));
-        return cudaGetLastError();
+        return launch(backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, lse, Dws, dk, dv, C, 1.0f / sqrtf((float)C));
     });
 }
 

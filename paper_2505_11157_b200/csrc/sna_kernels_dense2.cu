@@ -80,6 +80,8 @@ enum { B_KFULL = 0, B_KCONV = 2, B_KFREE = 4, B_VFULL = 6, B_VRAWFREE = 8, B_VCO
 // phase; an issuer commits to a buffer's DONE / STFULL barrier again only for a block whose operands-ready phase needs the
 // element-wise threads to have seen the previous use of that buffer complete.
 
+// Lets a band kernel that was launched to follow this one (its programmatic dependent) take the SMs that the last blocks leave idle.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float ex2f(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float trunc19f(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
@@ -282,6 +284,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
     __shared__ uint32_t tmem_base_s;
     __shared__ int fail_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) allow_dependents();
     const int tile = blockIdx.x % tiles_per_row;
     const int rest = blockIdx.x / tiles_per_row;
     const int n = rest % N;
@@ -687,6 +690,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
     __shared__ uint32_t tmem_base_s;
     __shared__ int fail_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) allow_dependents();
     const int tile = blockIdx.x % tiles_per_row;
     const int rest = blockIdx.x / tiles_per_row;
     const int n = rest % N;
@@ -1020,6 +1024,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
     __shared__ uint32_t tmem_base_s;
     __shared__ int fail_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) allow_dependents();
     const int tile = blockIdx.x % tiles_per_row;
     const int rest = blockIdx.x / tiles_per_row;
     const int n = rest % N;
@@ -1390,14 +1395,15 @@ cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t 
 
 bool dense2_path_chosen(const DevPlan& p, int C, int N) {
     if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || p.dense_fraction >= 0.999f || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
-    // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time; below that much work per
-    // SM the band kernels alone, which share long streams between warps, are faster.  Measured (fwd / dq / dkdv us, with : without
-    // the dense kernels; work in longest lists per SM): 128x256, cutoff 4 rings, N = 1 (0.1) 57/62/80 : 32/36/40, N = 4 (0.4)
-    // 99/114/150 : 89/110/124, N = 8 (0.8) 166/191/239 : 170/202/233, N = 16 (1.6) 310/356/447 : 329/389/456; 256x512 -> 128x256
-    // N = 8 (0.9) 370/408/539 : 387/464/551; 361x720 N = 1 (0.6) 271/287/375 : 258/299/351, N = 2 (1.2) 486/521/672 : 488/577/686.
+    // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time, in which the band kernel fills
+    // only the SMs that it leaves idle; with too little work per SM the band kernels alone, which share long streams between warps,
+    // are faster.  Measured (fwd / dq / dkdv us, with : without the dense kernels; work in longest lists per SM): 128x256, cutoff 4
+    // rings, N = 1 (0.1) 57/62/80 : 32/36/40, N = 4 (0.39) 97/113/150 : 88/108/123, N = 8 (0.8) 161/184/224 : 168/200/233, N = 16
+    // 307/353/439 : 329/389/456; 10 rings, N = 2 (0.47) 159/172/216 : 147/176/213; 256x512 -> 128x256 N = 4 (0.44) 196/212/272 :
+    // 208/246/280; 361x720 N = 1 (0.6) 237/253/321 : 254/298/352.
     // The second bound is the fixed cost of another kernel: 32x64, N = 32 (0.9 lists of 3 blocks) 49/52/55 : 36/41/39.
     const long long work = (long long)((p.nlon_out + M2 - 1) / M2) * N * p.dense_blocks;
-    return work * 10 >= p.num_sms * 8LL * p.dense_longest && work >= p.num_sms * 6LL;
+    return work * 10 >= p.num_sms * 4LL * p.dense_longest && work >= p.num_sms * 6LL;
 }
 
 bool dense2_global_supported(const DevPlan& p, int C) {

@@ -353,12 +353,23 @@ void pad(BandStream& S) {
     S.masks.insert(S.masks.end(), 3 * 32, 0u);
 }
 
-void complete(BandStream& S, int rows_per_group) {
+// ptr, win, dense_min_width: as given to merge_group
+void complete(BandStream& S, int rows_per_group, const std::vector<int32_t>& ptr, const std::vector<RingWindow>& win, int dense_min_width) {
     pad(S);
     S.order.resize((S.chunk_ptr.size() - 1) / rows_per_group);
     for (size_t i = 0; i < S.order.size(); ++i) S.order[i] = (int32_t)i;
     auto length = [&](int g) { return S.chunk_ptr[(size_t)(g + 1) * rows_per_group] - S.chunk_ptr[(size_t)g * rows_per_group]; };
     std::stable_sort(S.order.begin(), S.order.end(), [&](int a, int b) { return length(a) > length(b); });
+    // Groups with windows on the dense kernels depend on their results: not among the first, which may start before those are there.
+    std::vector<int32_t> independent, dependent;
+    for (int g : S.order) {
+        bool dense = false;
+        const size_t end = std::min<size_t>((size_t)(g + 1) * TILE_LAT, ptr.size() - 1);
+        for (int i = ptr[(size_t)g * TILE_LAT]; i < ptr[end]; ++i) dense = dense || served_by_dense(win[i], dense_min_width);
+        (dense ? dependent : independent).push_back(g);
+    }
+    S.order = independent;
+    S.order.insert(S.order.begin() + independent.size() / 4, dependent.begin(), dependent.end());
     for (int g : S.order) S.lengths.push_back(length(g) / rows_per_group);
 }
 
@@ -435,7 +446,7 @@ void build_forward_band(const HostPlan& P, BandStream& S, int dense_min_width) {
         });
         b.finish(S);
     }
-    complete(S, 1);
+    complete(S, 1, P.row_ptr, P.windows, dense_min_width);
 }
 
 bool build_transposed_band(const HostPlan& P, BandStream& S, int dense_min_width) {
@@ -456,7 +467,7 @@ bool build_transposed_band(const HostPlan& P, BandStream& S, int dense_min_width
             });
             b.finish(S);
         }
-    complete(S, consecutive ? 1 : P.ps);
+    complete(S, consecutive ? 1 : P.ps, P.t_row_ptr, P.t_windows, dense_min_width);
     return consecutive;
 }
 

@@ -64,7 +64,7 @@ struct BandStream {
     std::vector<int32_t> chunk_ptr;     // [rows+1] first chunk of each stream row
     std::vector<BandColumn> columns;    // BAND_CHUNK per chunk
     std::vector<uint32_t> masks;        // 32 per chunk
-    std::vector<int32_t> order;         // ring groups, longest stream first
+    std::vector<int32_t> order;         // ring groups, longest stream first (but see complete())
     std::vector<int32_t> lengths;       // chunks per stream row of order[i]
     bool one_row = false;               // every group walks row 0 (global attention)
 };
