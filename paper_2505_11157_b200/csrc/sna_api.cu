@@ -78,6 +78,8 @@ sna_status_t check_problem(const sna_plan_t* plan, int B, int H, int C) {
 template <typename... P>
 bool all_aligned(P... ptrs) { return (aligned16(ptrs) && ...); }
 
+long long points_in(const sna_plan_t* plan) { return (long long)plan->host.nlat_in * plan->host.nlon_in; }
+long long points_out(const sna_plan_t* plan) { return (long long)plan->host.nlat_out * plan->host.nlon_out; }
 size_t stats_elems(const sna_plan_t* plan, int B, int H) {
     return (size_t)B * H * plan->host.nlat_out * plan->host.nlon_out;
 }
@@ -382,8 +384,9 @@ int sna_forward_kernel_count(const sna_plan_t* plan, int C, int with_lse) {
     return (with_lse && sna::dense2_path_chosen(plan->dev, C, 1 << 20)) ? 2 : 1;
 }
 
-sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
-                            float* lse, int B, int H, int C, void* cuda_stream) {
+// out_cf: if not null, the output is wanted there too, channels first (the band kernels write it themselves)
+static sna_status_t forward_into(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
+                            float* lse, int B, int H, int C, void* cuda_stream, float* out_cf) {
     sna_status_t st = check_problem(plan, B, H, C);
     if (st != SNA_OK) return st;
     if (!q || !k || !v || !out) { set_error("q, k, v and out must not be NULL"); return SNA_ERR_INVALID_ARG; }
@@ -396,14 +399,23 @@ sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float*
     } else if (lse != nullptr && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its partial result travels in out / lse), the rest on the band kernel
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, true, false, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, true, false, (cudaStream_t)cuda_stream, out_cf);
+        out_cf = nullptr;
     } else if (sna::band_path_supported(plan->dev, C)) {
-        e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, false, false, (cudaStream_t)cuda_stream);
+        e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, false, false, (cudaStream_t)cuda_stream, out_cf);
+        out_cf = nullptr;
     } else {
         e = sna::launch_forward_generic(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "forward launch");
+    if (out_cf != nullptr) e = sna::launch_cl_to_cf(out, out_cf, B * H, C, points_out(plan), (cudaStream_t)cuda_stream);
+    if (e != cudaSuccess) return cuda_fail(e, "layout launch");
     return SNA_OK;
+}
+
+sna_status_t sna_forward_ex(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
+                            float* lse, int B, int H, int C, void* cuda_stream) {
+    return forward_into(plan, q, k, v, out, lse, B, H, C, cuda_stream, nullptr);
 }
 
 sna_status_t sna_forward(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
@@ -411,9 +423,10 @@ sna_status_t sna_forward(const sna_plan_t* plan, const float* q, const float* k,
     return sna_forward_ex(plan, q, k, v, out, nullptr, B, H, C, cuda_stream);
 }
 
-sna_status_t sna_backward_dq(const sna_plan_t* plan, const float* q, const float* k, const float* v,
+// *_cf: if not null, the gradients are wanted there, channels first, and the channels-last buffers are scratch
+static sna_status_t backward_dq_into(const sna_plan_t* plan, const float* q, const float* k, const float* v,
                              const float* dout, const float* out, const float* lse, float* dq, float* D,
-                             int B, int H, int C, void* cuda_stream) {
+                             int B, int H, int C, void* cuda_stream, float* dq_cf) {
     sna_status_t st = check_problem(plan, B, H, C);
     if (st != SNA_OK) return st;
     if (!q || !k || !v || !dout || !lse || !dq || !D) { set_error("q, k, v, dout, lse, dq and D must not be NULL"); return SNA_ERR_INVALID_ARG; }
@@ -426,19 +439,29 @@ sna_status_t sna_backward_dq(const sna_plan_t* plan, const float* q, const float
     } else if (out != nullptr && out != dq && plan->dev.dense_fraction >= 0.10f && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dq is written first), the rest is added by the band kernel
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, nullptr, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, true, false, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, true, false, (cudaStream_t)cuda_stream, dq_cf);
+        dq_cf = nullptr;
     } else if (out != nullptr && sna::band_path_supported(plan->dev, C)) {
-        e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, false, false, (cudaStream_t)cuda_stream);
+        e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, false, false, (cudaStream_t)cuda_stream, dq_cf);
+        dq_cf = nullptr;
     } else {
         e = sna::launch_backward_dq_generic(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "backward dq launch");
+    if (dq_cf != nullptr) e = sna::launch_cl_to_cf(dq, dq_cf, B * H, C, points_out(plan), (cudaStream_t)cuda_stream);
+    if (e != cudaSuccess) return cuda_fail(e, "layout launch");
     return SNA_OK;
 }
 
-sna_status_t sna_backward_dkdv(const sna_plan_t* plan, const float* q, const float* k, const float* v,
+sna_status_t sna_backward_dq(const sna_plan_t* plan, const float* q, const float* k, const float* v,
+                             const float* dout, const float* out, const float* lse, float* dq, float* D,
+                             int B, int H, int C, void* cuda_stream) {
+    return backward_dq_into(plan, q, k, v, dout, out, lse, dq, D, B, H, C, cuda_stream, nullptr);
+}
+
+static sna_status_t backward_dkdv_into(const sna_plan_t* plan, const float* q, const float* k, const float* v,
                                const float* dout, const float* lse, const float* D, float* dk, float* dv,
-                               int B, int H, int C, void* cuda_stream) {
+                               int B, int H, int C, void* cuda_stream, float* dk_cf, float* dv_cf) {
     sna_status_t st = check_problem(plan, B, H, C);
     if (st != SNA_OK) return st;
     if (!q || !k || !v || !dout || !lse || !D || !dk || !dv) { set_error("q, k, v, dout, lse, D, dk and dv must not be NULL"); return SNA_ERR_INVALID_ARG; }
@@ -457,14 +480,27 @@ sna_status_t sna_backward_dkdv(const sna_plan_t* plan, const float* q, const flo
     } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_chosen(plan->dev, C, B * H)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dk, dv is written first), the band kernel adds the rest
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
-        if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, true, false, (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, true, false, (cudaStream_t)cuda_stream, dk_cf, dv_cf);
+        dk_cf = nullptr;
     } else if (sna::band_path_supported(plan->dev, C)) {
-        e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, false, false, (cudaStream_t)cuda_stream);
+        e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, false, false, (cudaStream_t)cuda_stream, dk_cf, dv_cf);
+        dk_cf = nullptr;
     } else {
         e = sna::launch_backward_dkdv_generic(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "backward dk/dv launch");
+    if (dk_cf != nullptr) {
+        e = sna::launch_cl_to_cf(dk, dk_cf, B * H, C, points_in(plan), (cudaStream_t)cuda_stream);
+        if (e == cudaSuccess) e = sna::launch_cl_to_cf(dv, dv_cf, B * H, C, points_in(plan), (cudaStream_t)cuda_stream);
+        if (e != cudaSuccess) return cuda_fail(e, "layout launch");
+    }
     return SNA_OK;
+}
+
+sna_status_t sna_backward_dkdv(const sna_plan_t* plan, const float* q, const float* k, const float* v,
+                               const float* dout, const float* lse, const float* D, float* dk, float* dv,
+                               int B, int H, int C, void* cuda_stream) {
+    return backward_dkdv_into(plan, q, k, v, dout, lse, D, dk, dv, B, H, C, cuda_stream, nullptr, nullptr);
 }
 
 sna_status_t sna_backward_ex(const sna_plan_t* plan, const float* q, const float* k, const float* v,
@@ -595,11 +631,7 @@ sna_status_t sna_forward_cf(const sna_plan_t* plan, const float* q_cf, const flo
     if (e == cudaSuccess) e = sna::launch_cf_to_cl(k_cf, s.k, B * H, C, p_in, stream);
     if (e == cudaSuccess) e = sna::launch_cf_to_cl(v_cf, s.v, B * H, C, p_in, stream);
     if (e != cudaSuccess) return cuda_fail(e, "layout launch");
-    st = sna_forward_ex(plan, s.q, s.k, s.v, s.out, s.lse, B, H, C, cuda_stream);
-    if (st != SNA_OK) return st;
-    e = sna::launch_cl_to_cf(s.out, out_cf, B * H, C, p_out, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "layout launch");
-    return SNA_OK;
+    return forward_into(plan, s.q, s.k, s.v, s.out, s.lse, B, H, C, cuda_stream, out_cf);
 }
 
 sna_status_t sna_backward_cf(const sna_plan_t* plan, const float* dout_cf, const void* state, size_t state_bytes,
@@ -626,17 +658,12 @@ sna_status_t sna_backward_cf(const sna_plan_t* plan, const float* dout_cf, const
     float* dq = (float*)p;   p += round256(out_elems(plan, B, H, C) * sizeof(float));
     float* dk = (float*)p;   p += round256(in_elems(plan, B, H, C) * sizeof(float));
     float* dv = (float*)p;   p += round256(in_elems(plan, B, H, C) * sizeof(float));
-    void* ws = p;
-    const long long p_in = (long long)plan->host.nlat_in * plan->host.nlon_in, p_out = (long long)plan->host.nlat_out * plan->host.nlon_out;
-    cudaError_t e = sna::launch_cf_to_cl(dout_cf, dout, B * H, C, p_out, stream);
+    cudaError_t e = sna::launch_cf_to_cl(dout_cf, dout, B * H, C, points_out(plan), stream);
     if (e != cudaSuccess) return cuda_fail(e, "layout launch");
-    st = sna_backward_ex(plan, s.q, s.k, s.v, dout, s.out, s.lse, dq, dk, dv, ws, sna_workspace_bytes(plan, B, H, C), B, H, C, cuda_stream);
+    float* D = (float*)p;
+    st = backward_dq_into(plan, s.q, s.k, s.v, dout, s.out, s.lse, dq, D, B, H, C, cuda_stream, dq_cf);
     if (st != SNA_OK) return st;
-    e = sna::launch_cl_to_cf(dq, dq_cf, B * H, C, p_out, stream);
-    if (e == cudaSuccess) e = sna::launch_cl_to_cf(dk, dk_cf, B * H, C, p_in, stream);
-    if (e == cudaSuccess) e = sna::launch_cl_to_cf(dv, dv_cf, B * H, C, p_in, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "layout launch");
-    return SNA_OK;
+    return backward_dkdv_into(plan, s.q, s.k, s.v, dout, s.lse, D, dk, dv, B, H, C, cuda_stream, dk_cf, dv_cf);
 }
 
 sna_status_t sna_forward_tf32(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,

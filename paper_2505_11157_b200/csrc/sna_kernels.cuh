@@ -57,18 +57,19 @@ struct DevPlan {
 // Band kernels (sna_kernels_band.cu: mma.sync; C <= 64); same contracts as the generic launchers.
 // after_dense: the dense kernels have served their windows (see below) and left partial results in the output buffers; the
 // band kernels walk the remaining windows and continue from those.  lp: reduced-precision variant (C = 16, 32, 64), every
-// product is one FP16 MMA (operands rounded to 11 significant bits).
+// product is one FP16 MMA (operands rounded to 11 significant bits).  *_cf: if not null, the results go there in channels-first
+// planes ([slices][C][points]; forward: there too); the channels-last buffers still carry the dense kernels' partial results.
 cudaError_t band_prepare_device();   // once per device: opt in to the kernels' shared-memory sizes
 bool band_path_supported(const DevPlan& p, int C);
 cudaError_t launch_forward_band(const DevPlan& p, const float* q, const float* k, const float* v, float* out, float* lse,
-                                int N, int C, bool after_dense, bool lp, cudaStream_t stream);
+                                int N, int C, bool after_dense, bool lp, cudaStream_t stream, float* out_cf = nullptr);
 // out is required (D_i = dout_i . out_i); out and dq may be the same buffer unless after_dense.
 cudaError_t launch_backward_dq_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                     const float* out, const float* lse, float* dq, float* Dws, int N, int C, bool after_dense, bool lp,
-                                    cudaStream_t stream);
+                                    cudaStream_t stream, float* dq_cf = nullptr);
 cudaError_t launch_backward_dkdv_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                       const float* lse, const float* Dws, float* dk, float* dv, int N, int C, bool after_dense, bool lp,
-                                      cudaStream_t stream);
+                                      cudaStream_t stream, float* dk_cf = nullptr, float* dv_cf = nullptr);
 // Dense (tcgen05) kernels (sna_kernels_dense2.cu: TMA loads, warp-specialised, operands and accumulators in TMEM) for
 // the windows in the plan's dense lists: whole input rings, and wide banded windows as masked blocks.  The forward kernel
 // writes the partial result (normalised out, lse) of the output latitudes in p.dense_rows and the band kernel

@@ -515,6 +515,15 @@ __device__ __forceinline__ void store_quad(float* p, int m, int C, int t, const 
     const int c = Own<CP>::channel(t, 4 * m);
     if (c < C) *reinterpret_cast<float4*>(p + c) = x;
 }
+// The same four channels in channels-first planes of P points: eight threads fill 32 bytes of each plane.  cf: the tensor; pt: the
+// point, counted over all slices; n: its slice.
+template <int CP>
+__device__ __forceinline__ void store_quad_cf(float* cf, size_t pt, int n, size_t P, int m, int C, int t, const float4& x) {
+    const int c = Own<CP>::channel(t, 4 * m);
+    if (c >= C) return;
+    float* p = cf + (size_t)n * (C - 1) * P + pt + c * P;
+    p[0] = x.x; p[P] = x.y; p[2 * P] = x.z; p[3 * P] = x.w;
+}
 __device__ __forceinline__ float4 operator+(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // The stream a launch walks.
@@ -634,7 +643,7 @@ struct Blocks {
 template <int CP, bool LP, bool PAD>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::FWD)
 forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
-                    float* out, float* lse, int C_, float scale_log2) {
+                    float* out, float* lse, float* out_cf, int C_, float scale_log2) {
     const int C = PAD ? C_ : CP;
     constexpr int NT = CP / 8;
     using S = Stage<CP>;
@@ -781,6 +790,11 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
         if (!task.writes(m)) continue;
         if (at.ok0) store_quad<CP>(out + at.pt0 * C, m, C, t, quad(o, m, 0, inv0));
         if (at.ok1) store_quad<CP>(out + at.pt1 * C, m, C, t, quad(o, m, 1, inv1));
+        if (out_cf != nullptr) {
+            const size_t P = (size_t)p.nlat_out * p.nlon_out;
+            if (at.ok0) store_quad_cf<CP>(out_cf, at.pt0, n, P, m, C, t, quad(o, m, 0, inv0));
+            if (at.ok1) store_quad_cf<CP>(out_cf, at.pt1, n, P, m, C, t, quad(o, m, 1, inv1));
+        }
     }
     if (lse != nullptr && t == 0 && task.writes(0)) {
         if (at.ok0) lse[at.pt0] = ((m0 + W_SET) + log2f(ls0 * W_UNIT)) * LN2;
@@ -797,7 +811,7 @@ template <int CP, bool LP, bool PAD>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DQ)
 backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                         const float* __restrict__ dout, const float* out, const float* __restrict__ lse,
-                        float* dq, float* __restrict__ Dws, int C_, float scale) {
+                        float* dq, float* __restrict__ Dws, float* dq_cf, int C_, float scale) {
     const int C = PAD ? C_ : CP;
     constexpr int NT = CP / 8;
     using S = Stage<CP>;
@@ -901,8 +915,14 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
         float4 r0 = quad(acc, m, 0, f0), r1 = quad(acc, m, 1, f1);
         if (add0) r0 = r0 + load_quad<CP>(dq + at.pt0 * C, m, C, t);
         if (add1) r1 = r1 + load_quad<CP>(dq + at.pt1 * C, m, C, t);
-        if (at.ok0) store_quad<CP>(dq + at.pt0 * C, m, C, t, r0);
-        if (at.ok1) store_quad<CP>(dq + at.pt1 * C, m, C, t, r1);
+        if (dq_cf == nullptr) {
+            if (at.ok0) store_quad<CP>(dq + at.pt0 * C, m, C, t, r0);
+            if (at.ok1) store_quad<CP>(dq + at.pt1 * C, m, C, t, r1);
+        } else {
+            const size_t P = (size_t)p.nlat_out * p.nlon_out;
+            if (at.ok0) store_quad_cf<CP>(dq_cf, at.pt0, n, P, m, C, t, r0);
+            if (at.ok1) store_quad_cf<CP>(dq_cf, at.pt1, n, P, m, C, t, r1);
+        }
     }
 }
 
@@ -917,7 +937,7 @@ template <int CP, bool LP, bool PAD>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DKDV)
 backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                           const float* __restrict__ dout, const float* __restrict__ lse, const float* __restrict__ Dws,
-                          float* dk, float* dv, int C_, float scale) {
+                          float* dk, float* dv, float* dk_cf, float* dv_cf, int C_, float scale) {
     const int C = PAD ? C_ : CP;
     constexpr int NT = CP / 8;
     using S = Stage<CP>;
@@ -1025,8 +1045,14 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
             k1 = k1 + load_quad<CP>(dk + at.pt1 * C, m, C, t);
             v1 = v1 + load_quad<CP>(dv + at.pt1 * C, m, C, t);
         }
-        if (at.ok0) { store_quad<CP>(dk + at.pt0 * C, m, C, t, k0); store_quad<CP>(dv + at.pt0 * C, m, C, t, v0); }
-        if (at.ok1) { store_quad<CP>(dk + at.pt1 * C, m, C, t, k1); store_quad<CP>(dv + at.pt1 * C, m, C, t, v1); }
+        if (dk_cf == nullptr) {
+            if (at.ok0) { store_quad<CP>(dk + at.pt0 * C, m, C, t, k0); store_quad<CP>(dv + at.pt0 * C, m, C, t, v0); }
+            if (at.ok1) { store_quad<CP>(dk + at.pt1 * C, m, C, t, k1); store_quad<CP>(dv + at.pt1 * C, m, C, t, v1); }
+        } else {
+            const size_t P = (size_t)p.nlat_in * p.nlon_in;
+            if (at.ok0) { store_quad_cf<CP>(dk_cf, at.pt0, n, P, m, C, t, k0); store_quad_cf<CP>(dv_cf, at.pt0, n, P, m, C, t, v0); }
+            if (at.ok1) { store_quad_cf<CP>(dk_cf, at.pt1, n, P, m, C, t, k1); store_quad_cf<CP>(dv_cf, at.pt1, n, P, m, C, t, v1); }
+        }
     }
 }
 
@@ -1117,37 +1143,37 @@ bool band_path_supported(const DevPlan& p, int C) {
 }
 
 cudaError_t launch_forward_band(const DevPlan& p, const float* q, const float* k, const float* v, float* out, float* lse,
-                                int N, int C, bool after_dense, bool lp, cudaStream_t stream) {
+                                int N, int C, bool after_dense, bool lp, cudaStream_t stream, float* out_cf) {
     return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::FWD, view, grid)) return cudaErrorInvalidValue;
-        return launch(forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, out, lse, C, LOG2E / sqrtf((float)C));
+        return launch(forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, out, lse, out_cf, C, LOG2E / sqrtf((float)C));
     });
 }
 
 cudaError_t launch_backward_dq_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                     const float* out, const float* lse, float* dq, float* Dws, int N, int C, bool after_dense, bool lp,
-                                    cudaStream_t stream) {
+                                    cudaStream_t stream, float* dq_cf) {
     return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::DQ, view, grid)) return cudaErrorInvalidValue;
-        return launch(backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, out, lse, dq, Dws, C, 1.0f / sqrtf((float)C));
+        return launch(backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, out, lse, dq, Dws, dq_cf, C, 1.0f / sqrtf((float)C));
     });
 }
 
 cudaError_t launch_backward_dkdv_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                       const float* lse, const float* Dws, float* dk, float* dv, int N, int C, bool after_dense, bool lp,
-                                      cudaStream_t stream) {
+                                      cudaStream_t stream, float* dk_cf, float* dv_cf) {
     return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, true, after_dense, N, Blocks<CP, decltype(low)::value>::DKDV, view, grid)) return cudaErrorInvalidValue;
-        return launch(backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, lse, Dws, dk, dv, C, 1.0f / sqrtf((float)C));
+        return launch(backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, lse, Dws, dk, dv, dk_cf, dv_cf, C, 1.0f / sqrtf((float)C));
     });
 }
 
