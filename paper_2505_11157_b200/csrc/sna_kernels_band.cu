@@ -640,7 +640,7 @@ struct Blocks {
     static constexpr int FWD = CP == 64 ? 3 : CP == 32 && !LP ? 4 : 5, DQ = CP == 64 ? 2 : CP == 32 || !LP ? 4 : 5, DKDV = CP == 64 ? 2 : CP == 32 && !LP ? 3 : 4;
 };
 
-template <int CP, bool LP, bool PAD>
+template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::FWD)
 forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                     float* out, float* lse, float* out_cf, int C_, float scale_log2) {
@@ -790,7 +790,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
         if (!task.writes(m)) continue;
         if (at.ok0) store_quad<CP>(out + at.pt0 * C, m, C, t, quad(o, m, 0, inv0));
         if (at.ok1) store_quad<CP>(out + at.pt1 * C, m, C, t, quad(o, m, 1, inv1));
-        if (out_cf != nullptr) {
+        if constexpr (CF) {
             const size_t P = (size_t)p.nlat_out * p.nlon_out;
             if (at.ok0) store_quad_cf<CP>(out_cf, at.pt0, n, P, m, C, t, quad(o, m, 0, inv0));
             if (at.ok1) store_quad_cf<CP>(out_cf, at.pt1, n, P, m, C, t, quad(o, m, 1, inv1));
@@ -807,7 +807,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
 // `out` and `dq` may be the same buffer: a warp reads its own 16 rows of `out` before it writes them as dq.
 // The row scale of dout is left out of t, D and ds until the end, so that ds is of the order of v for every row.
 // ---------------------------------------------------------------------------------------------------------
-template <int CP, bool LP, bool PAD>
+template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DQ)
 backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                         const float* __restrict__ dout, const float* out, const float* __restrict__ lse,
@@ -915,7 +915,7 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
         float4 r0 = quad(acc, m, 0, f0), r1 = quad(acc, m, 1, f1);
         if (add0) r0 = r0 + load_quad<CP>(dq + at.pt0 * C, m, C, t);
         if (add1) r1 = r1 + load_quad<CP>(dq + at.pt1 * C, m, C, t);
-        if (dq_cf == nullptr) {
+        if constexpr (!CF) {
             if (at.ok0) store_quad<CP>(dq + at.pt0 * C, m, C, t, r0);
             if (at.ok1) store_quad<CP>(dq + at.pt1 * C, m, C, t, r1);
         } else {
@@ -933,7 +933,7 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
 // ---------------------------------------------------------------------------------------------------------
 constexpr float P_SHIFT = 10.f;      // weights p <= 1 are held times 2^10
 
-template <int CP, bool LP, bool PAD>
+template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DKDV)
 backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
                           const float* __restrict__ dout, const float* __restrict__ lse, const float* __restrict__ Dws,
@@ -1045,7 +1045,7 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
             k1 = k1 + load_quad<CP>(dk + at.pt1 * C, m, C, t);
             v1 = v1 + load_quad<CP>(dv + at.pt1 * C, m, C, t);
         }
-        if (dk_cf == nullptr) {
+        if constexpr (!CF) {
             if (at.ok0) { store_quad<CP>(dk + at.pt0 * C, m, C, t, k0); store_quad<CP>(dv + at.pt0 * C, m, C, t, v0); }
             if (at.ok1) { store_quad<CP>(dk + at.pt1 * C, m, C, t, k1); store_quad<CP>(dv + at.pt1 * C, m, C, t, v1); }
         } else {
@@ -1056,22 +1056,25 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
     }
 }
 
-template <int CP, bool LP, bool PAD>
+template <int CP, bool LP, bool PAD, bool CF>
 cudaError_t prepare_instantiation() {
     const int bytes = (int)smem_bytes<CP>();
-    cudaError_t e = cudaFuncSetAttribute(forward_band_kernel<CP, LP, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_dq_band_kernel<CP, LP, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_dkdv_band_kernel<CP, LP, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(forward_band_kernel<CP, LP, PAD, CF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_dq_band_kernel<CP, LP, PAD, CF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_dkdv_band_kernel<CP, LP, PAD, CF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     return e;
 }
 
-// Calls f(channels of the instantiation, reduced precision, padded) with constants.
+// Calls f(channels of the instantiation, reduced precision, padded, channels-first results) with constants.
 template <typename F>
-cudaError_t dispatch(int C, bool lp, F&& f) {
+cudaError_t dispatch(int C, bool lp, bool cf, F&& f) {
+    constexpr std::false_type no;
+    constexpr std::true_type yes;
     auto with = [&](auto cp) {
-        constexpr int CP = decltype(cp)::value;
-        if (C == CP) return lp ? f(cp, std::true_type(), std::false_type()) : f(cp, std::false_type(), std::false_type());
-        return lp ? cudaErrorInvalidValue : f(cp, std::false_type(), std::true_type());
+        const bool pad = C != decltype(cp)::value;
+        if (lp) return pad || cf ? cudaErrorInvalidValue : f(cp, yes, no, no);
+        if (pad) return cf ? f(cp, no, yes, yes) : f(cp, no, yes, no);
+        return cf ? f(cp, no, no, yes) : f(cp, no, no, no);
     };
     if (C <= 16) return with(std::integral_constant<int, 16>());
     if (C <= 32) return with(std::integral_constant<int, 32>());
@@ -1132,8 +1135,9 @@ cudaError_t band_prepare_device() {
     const std::pair<int, bool> wide[] = {{48, false}, {64, false}, {64, true}};       // narrower rows need less than the default 48 KB
     static_assert(smem_bytes<32>() <= 48 * 1024, "list of the instantiations to prepare");
     for (const auto& [C, lp] : wide)
-        if (e == cudaSuccess)
-            e = dispatch(C, lp, [](auto cp, auto low, auto pad) { return prepare_instantiation<decltype(cp)::value, decltype(low)::value, decltype(pad)::value>(); });
+        for (bool cf : {false, true})
+            if (e == cudaSuccess && !(lp && cf))
+                e = dispatch(C, lp, cf, [](auto cp, auto low, auto pad, auto cf) { return prepare_instantiation<decltype(cp)::value, decltype(low)::value, decltype(pad)::value, decltype(cf)::value>(); });
     return e;
 }
 
@@ -1144,36 +1148,36 @@ bool band_path_supported(const DevPlan& p, int C) {
 
 cudaError_t launch_forward_band(const DevPlan& p, const float* q, const float* k, const float* v, float* out, float* lse,
                                 int N, int C, bool after_dense, bool lp, cudaStream_t stream, float* out_cf) {
-    return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
+    return dispatch(C, lp, out_cf != nullptr, [&](auto cp, auto low, auto pad, auto cf) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::FWD, view, grid)) return cudaErrorInvalidValue;
-        return launch(forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, out, lse, out_cf, C, LOG2E / sqrtf((float)C));
+        return launch(forward_band_kernel<CP, decltype(low)::value, decltype(pad)::value, decltype(cf)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, out, lse, out_cf, C, LOG2E / sqrtf((float)C));
     });
 }
 
 cudaError_t launch_backward_dq_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                     const float* out, const float* lse, float* dq, float* Dws, int N, int C, bool after_dense, bool lp,
                                     cudaStream_t stream, float* dq_cf) {
-    return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
+    return dispatch(C, lp, dq_cf != nullptr, [&](auto cp, auto low, auto pad, auto cf) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, false, after_dense, N, Blocks<CP, decltype(low)::value>::DQ, view, grid)) return cudaErrorInvalidValue;
-        return launch(backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, out, lse, dq, Dws, dq_cf, C, 1.0f / sqrtf((float)C));
+        return launch(backward_dq_band_kernel<CP, decltype(low)::value, decltype(pad)::value, decltype(cf)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, out, lse, dq, Dws, dq_cf, C, 1.0f / sqrtf((float)C));
     });
 }
 
 cudaError_t launch_backward_dkdv_band(const DevPlan& p, const float* q, const float* k, const float* v, const float* dout,
                                       const float* lse, const float* Dws, float* dk, float* dv, int N, int C, bool after_dense, bool lp,
                                       cudaStream_t stream, float* dk_cf, float* dv_cf) {
-    return dispatch(C, lp, [&](auto cp, auto low, auto pad) {
+    return dispatch(C, lp, dk_cf != nullptr, [&](auto cp, auto low, auto pad, auto cf) {
         constexpr int CP = decltype(cp)::value;
         BandView view;
         unsigned grid;
         if (!make_view(p, true, after_dense, N, Blocks<CP, decltype(low)::value>::DKDV, view, grid)) return cudaErrorInvalidValue;
-        return launch(backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, lse, Dws, dk, dv, dk_cf, dv_cf, C, 1.0f / sqrtf((float)C));
+        return launch(backward_dkdv_band_kernel<CP, decltype(low)::value, decltype(pad)::value, decltype(cf)::value>, grid, smem_bytes<CP>(), after_dense, stream, p, view, q, k, v, dout, lse, Dws, dk, dv, dk_cf, dv_cf, C, 1.0f / sqrtf((float)C));
     });
 }
 

@@ -194,7 +194,7 @@ def sna_backward_dkdv(plan, q, k, v, dout, lse, D, dk, dv, B, H, C, stream=None)
 
 
 def sna_forward_tf32(plan, q, k, v, out, lse, B, H, C, stream=None):
-    """Reduced-precision forward pass (one TF32 product per contraction; normalised error below 5e-3)."""
+    """Reduced-precision forward pass (one product of 11-bit operands per contraction; normalised error below 5e-3)."""
     _check(_lib.sna_forward_tf32(plan, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, C, _stream(stream)))
 
 
