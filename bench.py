@@ -37,9 +37,9 @@ import numpy as np  # noqa: E402
 # ncu capture on workload c3 (bench.py cannot run ncu itself; the value is reported as `roofline.traffic` for that
 # workload only).
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    ("c3", "forward"): (44455936 + 725248) + (790744576 + 63745024),
-    ("c3", "backward_dq"): (57742592 + 2146560) + (956322304 + 63501312),
-    ("c3", "backward_dkdv"): (49276928 + 6318592) + (760281856 + 504061184),
+    ("c3", "forward"): (45483264 + 864512) + (862652160 + 59614464),
+    ("c3", "backward_dq"): (56134656 + 121088) + (1041766144 + 61313792),
+    ("c3", "backward_dkdv"): (49153536 + 5571840) + (763308544 + 493414400),
 }
 HBM_GBS_FALLBACK = 6650.0          # used only if MEASURED_PEAKS.json is absent
 L2_BYTES = 126 * 1024 * 1024
@@ -430,7 +430,7 @@ def run_ours(args, wl):
             "roofline": {"bound": dom["bound"], "kernel": dominant, "achieved": achieved, "peak": peak, "unit": unit,
                          "frac": achieved / peak, "traffic": NCU_DRAM_BYTES_PER_LAUNCH.get((wl.name, dominant)),
                          "note": f"{dom['flops_per_unit']:g} flops per pair*channel credited, {dom['bytes'] / 1e6:.0f} MB compulsory; "
-                                 f"{peak_note}; the contractions run on tensor cores (TF32 main term + stacked BF16 corrections, "
+                                 f"{peak_note}; the contractions run on tensor cores (three terms of FP16 hi/lo parts, "
                                  "tcgen05 for whole-ring and wide windows); traffic = recorded ncu DRAM bytes read+written per "
                                  "stage (dense + band kernel), null when this workload has no capture"},
             "e2e": {"value": world * units / (ms_e2e_step_max * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
@@ -444,9 +444,9 @@ def run_ours(args, wl):
             t = time_steps(torch, prob, 10, 3, prob.step_tf32, flush)
             result["variants"] = {"tf32": {"ms_forward": t["ms_forward"], "ms_backward": t["ms_backward_dkdv"],
                                            "ms_per_step": t["ms_per_step"], "frac": roof_ms / t["ms_per_step"],
-                                           "note": "sna_forward_tf32 + sna_backward_tf32: one TF32 product per contraction, "
+                                           "note": "sna_forward_tf32 + sna_backward_tf32: one product of 11-bit operands per contraction, "
                                                    "tolerance 5e-3 instead of 1e-5 / 1e-4; not the headline"}}
-            # channels-first entry points on the same workload: the layout changes (HBM-bound transposes) run inside the calls
+            # channels-first entry points on the same workload: the layout changes run inside the calls
             cf = lambda x: x.permute(0, 1, 4, 2, 3).reshape(x.shape[0], -1, x.shape[2], x.shape[3]).contiguous()
             cf_in = [cf(x) for x in (prob.q, prob.k, prob.v, prob.dout)]
             cf_out = [torch.empty_like(cf_in[0]), torch.empty_like(cf_in[0]), torch.empty_like(cf_in[1]), torch.empty_like(cf_in[1])]
@@ -462,12 +462,12 @@ def run_ours(args, wl):
                                     cf_out[3], wl.B, wl.H, C, prob.stream)
 
             t = time_steps(torch, prob, 10, 3, step_cf, flush)
-            moved = 2 * 4 * sum(x.numel() for x in cf_in + cf_out)
+            moved = 2 * 4 * sum(x.numel() for x in cf_in)      # out, dq, dk and dv are written once, in place
             result["variants"]["channels_first"] = {
                 "ms_forward": t["ms_forward"], "ms_backward": t["ms_backward_dkdv"], "ms_per_step": t["ms_per_step"],
                 "layout_bytes_per_step": moved, "layout_ms_at_hbm_peak": moved / (hbm_gbs * 1e6),
-                "note": "sna_forward_cf + sna_backward_cf on [B, H*C, nlat, nlon] tensors: eight tiled transposes per step around "
-                        "the same kernels (each element read once and written once)"}
+                "note": "sna_forward_cf + sna_backward_cf on [B, H*C, nlat, nlon] tensors: tiled transposes of q, k, v and dout; "
+                        "the band kernels write out, dq, dk and dv channels first"}
             del cf_in, cf_out, state, scratch
             torch.cuda.empty_cache()
             step_prec()

@@ -93,9 +93,9 @@ sna_status_t sna_plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon_ou
  * Plan for GLOBAL spherical attention (Eq. s2_attention_discrete; App. B.1-B.2): every output point attends to every
  * input point, i.e. softmax attention over the whole input grid with the additive bias log omega_j.  Equivalent to
  * sna_plan_create with theta_cutoff >= pi, but no per-pair structure is built or stored: the plan holds only the grids,
- * the quadrature weights and the per-ring lists the dense tensor-core kernels walk.  All compute calls accept it; with
- * C = 32 they run entirely on the dense tcgen05 kernels (the backward pass runs fastest with out and lse
- * from sna_forward_ex); other shapes use the generic kernels.
+ * the quadrature weights, the per-ring lists the dense tensor-core kernels walk (C = 32) and one list of all points that the
+ * band kernels walk (any C up to 64).  All compute calls accept it (the backward pass runs fastest with out and lse from
+ * sna_forward_ex); other shapes use the generic kernels.
  */
 sna_status_t sna_plan_create_global(int nlat_in, int nlon_in, int nlat_out, int nlon_out,
                                     sna_grid_t grid_in, sna_grid_t grid_out, sna_plan_t** plan_out);
@@ -228,10 +228,10 @@ sna_status_t sna_backward_cf(const sna_plan_t* plan, const float* dout_cf, const
 /*
  * Reduced-precision variant of the forward and backward pass.  The paper lists "neither reduced precision nor tensor
  * core" support as a limitation of its kernels (Sec. 5, Limitations); here every contraction of
- * Eq. s2_attention_discrete_detailed and App. B.4 is taken as ONE TF32 tensor-core product (operands rounded to 11
- * significand bits, fp32 accumulation, fp32 softmax) instead of the error-compensated products of the default path.
+ * Eq. s2_attention_discrete_detailed and App. B.4 is taken as ONE tensor-core product (operands rounded to the 11
+ * significand bits of TF32, fp32 accumulation, fp32 softmax) instead of the error-compensated products of the default path.
  * Same arguments, layouts and semantics as sna_forward_ex / sna_backward_ex.  Accuracy: normalised maximum error
- * max|x - ref| / max|ref| per tensor below 5e-3 against an fp64 evaluation (measured ~1e-3); about 1.5x faster.
+ * max|x - ref| / max|ref| per tensor below 5e-3 against an fp64 evaluation (measured ~1e-3); about 1.2x faster.
  * Needs C in {16, 32, 64} and nlon_out >= 32 (SNA_ERR_UNSUPPORTED otherwise).
  */
 sna_status_t sna_forward_tf32(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
