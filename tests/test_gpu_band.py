@@ -112,3 +112,38 @@ def test_global_attention_on_the_band_kernels(shape, C, slices, grid, recompute)
         assert rel(x, r) <= (TOL if C != 32 else 1e-5), name       # (C = 32: a pass may run on the dense kernels, 2^-21 per operand)
     if grid == 2:
         assert not grads[1][..., 0, :, :].any() and not grads[2][..., 0, :, :].any()
+
+
+@pytest.mark.parametrize("shape, slices", [((128, 256, 128, 256, 0.1), 8), ((96, 384, 48, 192, 0.15), 12)], ids=["same_grid", "down2"])
+def test_band_kernels_that_start_before_the_dense_ones_have_finished(shape, slices):
+    """Calls in a row on one stream, on several streams and replayed from a captured graph give the same bits: nothing is read before
+    the dense kernels have written it, and the next call waits for both."""
+    nlat_in, nlon_in, nlat_out, nlon_out, theta = shape
+    with sna.Plan(nlat_in, nlon_in, nlat_out, nlon_out, 0, 0, theta) as plan:
+        gen = torch.Generator(device="cuda").manual_seed(76)
+        q, dout = (torch.randn(1, slices, nlat_out, nlon_out, 32, generator=gen, device="cuda") for _ in range(2))
+        k, v = (torch.randn(1, slices, nlat_in, nlon_in, 32, generator=gen, device="cuda") for _ in range(2))
+
+        def step():
+            out, lse = plan.forward(q, k, v, return_lse=True)
+            return [out, lse, *plan.backward(q, k, v, dout, out=out, lse=lse)]
+
+        ref = [t.clone() for t in step()]
+        for _ in range(10):
+            again = [torch.full_like(t, math.nan) for t in ref]
+            plan.forward(q, k, v, out=again[0], lse=again[1], return_lse=True)
+            plan.backward(q, k, v, dout, out=again[0], lse=again[1], dq=again[2], dk=again[3], dv=again[4])
+            assert all(torch.equal(a, b) for a, b in zip(again, ref))
+        torch.cuda.synchronize()
+        streams, results = [torch.cuda.Stream() for _ in range(3)], []
+        for s in streams:
+            with torch.cuda.stream(s):
+                results.append(step())
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            results.append(step())
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for r in results for a, b in zip(r, ref))
+        sna.sna_plan_check(plan.handle)
