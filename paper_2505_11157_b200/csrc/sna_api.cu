@@ -235,6 +235,7 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     d.dense_blocks = dense.blocks;
     d.dense_longest = dense.longest;
     d.dense_fraction = hp.nnz > 0 ? (float)((double)dense.pairs / (double)hp.nnz) : 0.f;
+    d.dense_all = dense.pairs == hp.nnz ? 1 : 0;
     d.is_global = global ? 1 : 0;
     d.t_consecutive = t_consecutive ? 1 : 0;
     sna::DevBand* dev_bands[4] = {&d.fwd, &d.fwdb, &d.t, &d.tb};

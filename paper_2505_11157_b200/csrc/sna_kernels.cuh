@@ -49,6 +49,7 @@ struct DevPlan {
     int n_t_dense_rows;
     long long dense_blocks, dense_longest;      // 128-column blocks that the tiles of one longitude range walk: all of them, the longest
     float dense_fraction;           // share of the table's entries that the dense kernels' windows cover
+    int dense_all;                  // 1: they cover every one (a share that rounds to 1 may still leave narrow windows out)
     int* dev_status;                // set to non-zero by a kernel whose bounded wait ran out
     int t_consecutive;              // 1: transposed tiles are 8 consecutive input columns; 0: split by residue mod ps
     int is_global;                  // 1: every window is a whole ring; the band streams have one row
@@ -78,7 +79,7 @@ cudaError_t launch_backward_dkdv_band(const DevPlan& p, const float* q, const fl
 cudaError_t dense2_prepare_device();   // once per device: opt in to the kernels' shared-memory sizes
 bool dense2_path_chosen(const DevPlan& p, int C, int N);
 cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t stream);
-bool dense2_global_supported(const DevPlan& p, int C);   // every window is a whole ring and the dense kernels can do all the work
+bool dense2_global_supported(const DevPlan& p, int C);   // the dense kernels can do all the work: no window is left to the band kernels
 enum class Pass { FORWARD, DQ, DKDV };
 bool dense2_global_chosen(const DevPlan& p, int C, int N, Pass pass);   // ... and are faster than the band kernels
 cudaError_t launch_forward_dense2(const DevPlan& p, const float* q, const float* k, const float* v, float* out, float* lse,

@@ -1394,7 +1394,7 @@ cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t 
 }
 
 bool dense2_path_chosen(const DevPlan& p, int C, int N) {
-    if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || p.dense_fraction >= 0.999f || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
+    if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || p.dense_all || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
     // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time, in which the band kernel fills
     // only the SMs that it leaves idle; with too little work per SM the band kernels alone, which share long streams between warps,
     // are faster.  Measured (fwd / dq / dkdv us, with : without the dense kernels; work in longest lists per SM): 128x256, cutoff 4
@@ -1407,7 +1407,7 @@ bool dense2_path_chosen(const DevPlan& p, int C, int N) {
 }
 
 bool dense2_global_supported(const DevPlan& p, int C) {
-    return C == C2 && (p.is_global || p.dense_fraction >= 0.999f) && p.n_dense_rows > 0 && p.n_t_dense_rows > 0 && encode_fn2() != nullptr &&
+    return C == C2 && p.dense_all && p.n_dense_rows > 0 && p.n_t_dense_rows > 0 && encode_fn2() != nullptr &&
            (long long)p.nlat_in * p.nlon_in * C < (1LL << 32) && (long long)p.nlat_out * p.nlon_out * C < (1LL << 32);
 }
 
@@ -1474,7 +1474,7 @@ cudaError_t launch_forward_dense2(const DevPlan& p, const float* q, const float*
     if (e == cudaSuccess) e = make_map2(&mk, k, N * p.nlat_in, p.nlon_in);
     if (e == cudaSuccess) e = make_map2(&mv, v, N * p.nlat_in, p.nlon_in);
     if (e != cudaSuccess) return e;
-    if (p.dense_fraction >= 0.999f)   // every window is a whole ring
+    if (p.dense_all)   // whole rings, in all but a few blocks
         forward_dense2_kernel<true><<<(unsigned)blocks, THREADS2, DENSE2_SMEM, stream>>>(p, mq, mk, mv, out, lse, N, LOG2E_2 / sqrtf((float)C), tiles_per_row);
     else
         forward_dense2_kernel<false><<<(unsigned)blocks, THREADS2, DENSE2_SMEM, stream>>>(p, mq, mk, mv, out, lse, N, LOG2E_2 / sqrtf((float)C), tiles_per_row);

@@ -1,0 +1,47 @@
+"""Which kernels a plan's passes run on, at the edges of the rules that choose them, against the fp64 CPU oracle.
+
+Tolerances: 5e-6 per tensor where the band kernels run alone, 1e-5 where the dense kernels take part (their first products keep
+19 to 21 bits of an operand); measured 3e-7 to 7e-6.
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import sna_oracle as orc
+from paper_2505_11157_b200 import sna
+from paper_2505_11157_b200.synthetic import make_inputs, small_workload
+
+pytestmark = pytest.mark.gpu
+
+TOL_DENSE = 1e-5
+
+
+def rel(x, ref):
+    return float(np.linalg.norm(x.detach().cpu().numpy().reshape(ref.shape).astype(np.float64) - ref) / np.linalg.norm(ref))
+
+
+def check(wl, tol):
+    """Forward with and without lse, backward with and without saved state; the gradients start as NaN."""
+    q, k, v, dout = make_inputs(wl)
+    g = orc.geometry(wl.nlat_in, wl.nlon_in, wl.nlat_out, wl.nlon_out, wl.grid_in, wl.grid_out, wl.theta_cutoff)
+    dev = [torch.from_numpy(a).cuda() for a in (q, k, v, dout)]
+    ref, refs = orc.forward(g, q, k, v), orc.backward(g, q, k, v, dout)
+    with sna.Plan(wl.nlat_in, wl.nlon_in, wl.nlat_out, wl.nlon_out, wl.grid_in, wl.grid_out, wl.theta_cutoff) as plan:
+        out, lse = plan.forward(*dev[:3], return_lse=True)
+        assert rel(out, ref) <= tol
+        assert rel(plan.forward(*dev[:3]), ref) <= tol
+        for state in ({"out": out, "lse": lse}, {}):
+            grads = [torch.full_like(dev[i], math.nan) for i in range(3)]
+            plan.backward(*dev, dq=grads[0], dk=grads[1], dv=grads[2], **state)
+            for name, x, r in zip(("dq", "dk", "dv"), grads, refs):
+                assert rel(x, r) <= tol, (name, bool(state))
+        torch.cuda.synchronize()
+        sna.sna_plan_check(plan.handle)
+
+
+@pytest.mark.parametrize("slices", [1, 4])
+def test_a_few_narrow_windows_beside_whole_rings_are_not_left_out(slices):
+    """14x256, cutoff 2.66: all but 26 of the table's entries (0.06 %) lie in whole rings or windows of 128 columns and more."""
+    check(small_workload("nearly_global", 14, 256, 14, 256, 0, 0, 2.66, 1, slices, 32, 81), TOL_DENSE)
