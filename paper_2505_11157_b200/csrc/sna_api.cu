@@ -44,7 +44,7 @@ struct sna_plan {
     sna::DevPlan dev{};
     std::vector<int32_t> band_lengths[4];      // of the four band streams (DevBand::lengths)
     int device = 0;
-    std::vector<int> zero_rings;       // input rings of quadrature weight zero (no kernel of a global plan visits them)
+    std::vector<int> unvisited;        // input rings that the dense dk/dv kernel does not write (weight zero, or in no window)
     bool is_global = false;            // created by sna_plan_create_global: every window is a whole ring
     void* dev_blob = nullptr;          // one allocation holding every device table
     mutable std::mutex ws_mutex;
@@ -139,7 +139,6 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     sna::HostPlan weighted;
     const bool dropped = sna::drop_zero_weight_rings(plan->host, weighted);
     const sna::HostPlan& hp = dropped ? weighted : plan->host;
-    for (int h = 0; h < hp.nlat_in; ++h) if (!(hp.omega[h] > 0.0)) plan->zero_rings.push_back(h);
     // heavy-first orders
     std::vector<int32_t> row_order(hp.nlat_out), t_row_order(hp.nlat_in);
     std::iota(row_order.begin(), row_order.end(), 0);
@@ -230,6 +229,7 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     d.dense_ptr = at(9); d.dense_lat = at(10); d.dense_m = at(11); d.dense_rows = at(12);
     d.t_dense_ptr = at(13); d.t_dense_lat = at(14); d.t_dense_m = at(15); d.t_dense_rows = at(16);
     d.dev_status = (int*)((char*)plan->dev_blob + pieces[17].offset);
+    for (int h = 0; h < hp.nlat_in; ++h) if (t_dense.ptr[h + 1] == t_dense.ptr[h]) plan->unvisited.push_back(h);
     d.n_dense_rows = (int)dense.rows.size();
     d.n_t_dense_rows = (int)t_dense.rows.size();
     d.dense_blocks = dense.blocks;
@@ -469,13 +469,13 @@ static sna_status_t backward_dkdv_into(const sna_plan_t* plan, const float* q, c
     if (!all_aligned(q, k, v, dout, dk, dv) || ((reinterpret_cast<uintptr_t>(lse) | reinterpret_cast<uintptr_t>(D)) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     cudaError_t e;
     if (sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::DKDV)) {
-        // the dense kernel writes only the rings some window refers to; rings of weight zero get their (zero) gradient here
+        // the dense kernel writes only the rings some window refers to; the others get their (zero) gradient here
         const size_t ring_bytes = (size_t)plan->host.nlon_in * C * sizeof(float), pitch = ring_bytes * plan->host.nlat_in;
-        for (size_t i = 0; i < plan->zero_rings.size(); ++i) {
-            const size_t off = ring_bytes * plan->zero_rings[i];
+        for (size_t i = 0; i < plan->unvisited.size(); ++i) {
+            const size_t off = ring_bytes * plan->unvisited[i];
             e = cudaMemset2DAsync((char*)dk + off, pitch, 0, ring_bytes, (size_t)B * H, (cudaStream_t)cuda_stream);
             if (e == cudaSuccess) e = cudaMemset2DAsync((char*)dv + off, pitch, 0, ring_bytes, (size_t)B * H, (cudaStream_t)cuda_stream);
-            if (e != cudaSuccess) return cuda_fail(e, "clearing the gradients of zero-weight rings");
+            if (e != cudaSuccess) return cuda_fail(e, "clearing the gradients of input rings without windows");
         }
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
     } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_chosen(plan->dev, C, B * H)) {

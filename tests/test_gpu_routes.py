@@ -45,3 +45,10 @@ def check(wl, tol):
 def test_a_few_narrow_windows_beside_whole_rings_are_not_left_out(slices):
     """14x256, cutoff 2.66: all but 26 of the table's entries (0.06 %) lie in whole rings or windows of 128 columns and more."""
     check(small_workload("nearly_global", 14, 256, 14, 256, 0, 0, 2.66, 1, slices, 32, 81), TOL_DENSE)
+
+
+@pytest.mark.parametrize("slices", [1, 8])
+def test_input_rings_that_no_window_reaches_get_zero_gradients(slices):
+    """Output rings at the two poles only: every window is a whole ring, and ten of the sixteen input rings are in none."""
+    wl = small_workload("poles", 16, 128, 2, 128, 0, 0, 0.5, 1, slices, 32, 82)
+    check(wl, TOL_DENSE)
