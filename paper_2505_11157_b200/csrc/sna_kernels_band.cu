@@ -62,9 +62,9 @@ __device__ __forceinline__ void acc2(float& a, float& b, float x, float y) { unp
 // Scales, all powers of two
 // ---------------------------------------------------------------------------------------------------------
 constexpr int TOP = 14;              // exponent of the largest element of a scaled tile row
-// exponent bits of a magnitude, not below 2^-100
+// exponent bits of a magnitude, not below 2^-100 (zero: of 1)
 __device__ __forceinline__ uint32_t exponent_bits(float amax) {
-    return max(__float_as_uint(amax) & 0x7f800000u, (uint32_t)(127 - 100) << 23);
+    return amax == 0.f ? 127u << 23 : max(__float_as_uint(amax) & 0x7f800000u, (uint32_t)(127 - 100) << 23);
 }
 __device__ __forceinline__ float pow2_to(int target, uint32_t ebits) { return __uint_as_float(((uint32_t)(254 + target) << 23) - ebits); }   // 2^(target - e)
 __device__ __forceinline__ float pow2_back(int target, uint32_t ebits) { return __uint_as_float(ebits - ((uint32_t)target << 23)); }        // 2^(e - target)
@@ -90,7 +90,10 @@ struct StreamScale {
 };
 
 // Scale of a warp's weights whose size is not known beforehand: it changes only when a weight above 2^15 appears (and for the first
-// one); then the largest is brought to about 2^11, and growth by 2^4 fits without another change.
+// one); then the largest is brought to about 2^11, and growth by 2^4 fits without another change.  A first weight may be far
+// below later ones, and the scale multiplies those before it is corrected: it is bounded, by 2^(11 + 72), so that p (t - D), whose
+// t and D are below 2^37 in the units of the tensor cores' operands, stays finite.  Weights so small that the bound leaves them
+// below FP16's range are below 2^-97 of what a weight of probability 1 would be.
 struct WeightScale {
     float scale = 1.f, limit = 0.f;
     // amax: this thread's largest scaled magnitude (called by the whole warp).  Returns the factor for the sums collected so
@@ -98,7 +101,7 @@ struct WeightScale {
     __device__ __forceinline__ float update(float amax) {
         const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(amax));
         if (!(__uint_as_float(w) > limit)) return 1.f;
-        const float f = pow2_to(11, exponent_bits(__uint_as_float(w)));
+        const float f = pow2_to(11, max(w & 0x7f800000u, (uint32_t)(127 - 72) << 23));
         scale *= f;
         limit = 32768.f;
         return f;
@@ -805,7 +808,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
 // ---------------------------------------------------------------------------------------------------------
 // backward, dq:  dq_i = scale * sum_j p_ij (t_ij - D_i) k_j,  D_i = dout_i . out_i  (App. B.4)
 // `out` and `dq` may be the same buffer: a warp reads its own 16 rows of `out` before it writes them as dq.
-// The row scale of dout is left out of t, D and ds until the end, so that ds is of the order of v for every row.
+// t, D and ds are in the units of the scaled dout row and the scaled v until the end.
 // ---------------------------------------------------------------------------------------------------------
 template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DQ)
@@ -857,9 +860,15 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
         clear(acc);
         ws = WeightScale();
         uint64_t bad = 0;
-        float nD0 = -D0 / Y.back0, nD1 = -D1 / Y.back1;      // times the weight scale
+        float nD0 = -D0 / Y.back0 * sc.b.scale, nD1 = -D1 / Y.back1 * sc.b.scale;      // times the weight scale
         walker.template run<LP && CP == 32 ? 1 : 2>(nchunks, [&](uint32_t st, uint32_t mask, auto&& release) {
-            if (!sc.known()) sc.look(st);
+            if (!sc.known()) {
+                const float before = sc.b.scale;
+                sc.look(st);
+                const float f = sc.b.scale / before;
+                nD0 *= f; nD1 *= f;
+                scale_rows(acc, f, f);
+            }
             float s[2][4], tt[2][4];
             SplitRows<CP, LP> K;
             {
@@ -872,7 +881,7 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
             release();
             rows_dot_points<CP, LP>(s, Q, K);
             note_overflow<LP>(bad, s);
-            const uint64_t f2 = both(Q.back0 * sc.a.inv), h2 = both(ws.scale * sc.b.inv);
+            const uint64_t f2 = both(Q.back0 * sc.a.inv), h2 = both(ws.scale);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(both(lse0), both(-LOG2E), bias2[j])), s[j][0], s[j][1]);
@@ -897,7 +906,7 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
         if (!sc.again(first_pass, total(acc) + sum2(bad), walker, nchunks)) break;
     }
     const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-    float f0 = scale * Y.back0 * sc.a.inv / ws.scale, f1 = scale * Y.back1 * sc.a.inv / ws.scale;
+    float f0 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back0, f1 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back1;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(acc, task.warp, 0, f0, f1);
@@ -977,9 +986,15 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
         clear(gk);
         clear(gv);
         ws = WeightScale();
+        float unit = sc.b.scale / V.back0;      // t, D and ds are in the units of the scaled dout and v until the end
         uint64_t bad = 0;
         walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
-            if (!sc.known()) sc.look(st);
+            if (!sc.known()) {
+                const float before = sc.b.scale;
+                sc.look(st);
+                unit *= sc.b.scale / before;
+                scale_rows(gk, sc.b.scale / before, sc.b.scale / before);
+            }
             float s[2][4], tt[2][4];
             SplitRows<CP, LP> Q, Y;
             Q.load(st + sc.own + S::A, sc.a.scale);
@@ -988,7 +1003,7 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
             rows_dot_points<CP, LP>(tt, V, Y);
             const uint64_t lse2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)}, D2[2] = {lds64(st + S::M1 + 8 * t), lds64(st + S::M1 + 32 + 8 * t)};
             note_overflow<LP>(bad, s);
-            const uint64_t f2 = both(K.back0 * sc.a.inv), h2 = both(V.back0 * ws.scale * sc.b.inv), nw2 = both(-ws.scale), nlog2e2 = both(-LOG2E);
+            const uint64_t f2 = both(K.back0 * sc.a.inv), h2 = both(ws.scale), nw2 = both(-ws.scale * unit), nlog2e2 = both(-LOG2E);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 // bias: log2 omega_j of the row's ring
@@ -1020,7 +1035,7 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
     }
     const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
     // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry 2^P_SHIFT.
-    float fk = scale * ex2(-P_SHIFT) * sc.a.inv / ws.scale, fv = ex2(-P_SHIFT) * sc.b.inv;
+    float fk = scale * ex2(-P_SHIFT) * sc.a.inv / ws.scale * sc.b.inv * V.back0, fv = ex2(-P_SHIFT) * sc.b.inv;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(gk, task.warp, 0, fk, fk);
