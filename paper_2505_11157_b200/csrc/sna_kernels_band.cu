@@ -940,8 +940,6 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
 //   dk_j = scale * sum_i p_ij (t_ij - D_i) q_i,   dv_j = sum_i p_ij dout_i          (App. B.4)
 // Tile rows are 8 input columns on each of the two rings of an input ring pair; stream columns are output points.
 // ---------------------------------------------------------------------------------------------------------
-constexpr float P_SHIFT = 10.f;      // weights p <= 1 are held times 2^10
-
 template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DKDV)
 backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
@@ -974,18 +972,19 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
         const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
         K.template load<true>(k + at.pt0 * C, k + at.pt1 * C, scale * LOG2E, C, t);
         V.template load<true>(v + at.pt0 * C, v + at.pt1 * C, 1.f, C, t);
-        bias0 = p.log2_omega[at.ha] + P_SHIFT; bias1 = p.log2_omega[at.hb] + P_SHIFT;
+        bias0 = p.log2_omega[at.ha]; bias1 = p.log2_omega[at.hb];
     }
     const size_t oslice = (size_t)n * p.nlat_out * p.nlon_out;
     int chunk0, nchunks;
     task.chunks(view, srow, chunk0, nchunks);
     const auto walker = make_walker<CP, true, PAD>(smem_raw, view.s, chunk0, first, p.nlon_out, 1, C, q + oslice * C, dout + oslice * C, lse + oslice, Dws + oslice);
     float gk[NT][4], gv[NT][4];
-    WeightScale ws;          // of ds
+    WeightScale wp, ws;      // of p (over global attention or for keys that little attention reaches all of them are small) and, beyond that, of ds
     for (bool first_pass = true;; first_pass = false) {
         clear(gk);
         clear(gv);
-        ws = WeightScale();
+        wp = ws = WeightScale();
+        float b0 = bias0, b1 = bias1;           // with the exponent of p's scale
         float unit = sc.b.scale / V.back0;      // t, D and ds are in the units of the scaled dout and v until the end
         uint64_t bad = 0;
         walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
@@ -1007,12 +1006,21 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 // bias: log2 omega_j of the row's ring
-                unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(lse2[j], nlog2e2, both(bias0))), s[j][0], s[j][1]);
-                unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(lse2[j], nlog2e2, both(bias1))), s[j][2], s[j][3]);
+                unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(lse2[j], nlog2e2, both(b0))), s[j][0], s[j][1]);
+                unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(lse2[j], nlog2e2, both(b1))), s[j][2], s[j][3]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
             }
             if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
+            const float pmax = max_abs(s);
+            if (__any_sync(FULL, pmax > wp.limit)) {
+                const float f = wp.update(pmax);
+                const float e = (float)((int)(__float_as_uint(f) >> 23) - 127);
+                b0 += e; b1 += e;
+                scale_rows(gv, f, f);
+                scale_rows(gk, f, f);
+                scale_rows(s, f, f);
+            }
             Weights<LP> P, W;
             P.set(s);
 #pragma unroll
@@ -1034,8 +1042,8 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
         if (!sc.again(first_pass, total(gk) + total(gv) + sum2(bad), walker, nchunks)) break;
     }
     const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
-    // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry 2^P_SHIFT.
-    float fk = scale * ex2(-P_SHIFT) * sc.a.inv / ws.scale * sc.b.inv * V.back0, fv = ex2(-P_SHIFT) * sc.b.inv;
+    // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry p's scale.
+    float fk = scale * sc.a.inv / ws.scale * sc.b.inv / wp.scale * V.back0, fv = sc.b.inv / wp.scale;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(gk, task.warp, 0, fk, fk);

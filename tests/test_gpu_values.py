@@ -33,6 +33,11 @@ def rel(x, ref):
     return float(np.linalg.norm(x - ref) / np.linalg.norm(ref))
 
 
+def rel_points(x, ref):
+    """The largest relative error of a grid point's channel vector."""
+    return float(np.max(np.linalg.norm(x - ref, axis=-1) / np.maximum(np.linalg.norm(ref, axis=-1), 1e-300)))
+
+
 @pytest.mark.parametrize("C", [16, 24, 32, 64])
 @pytest.mark.parametrize("precision", ["fp32", "tf32"])
 @pytest.mark.parametrize("slices", [2, 300])      # streams shared by a block's warps, and private
@@ -80,3 +85,30 @@ def test_a_gap_between_the_first_scores_and_the_largest(C):
             got, refs = run(SHAPE, CUTOFF, q, k, v, dout, recompute=recompute)
             for name, x, r in zip(("out", "dq", "dk", "dv"), got, refs):
                 assert rel(x, r) <= TOL["fp32"] * 4, (name, gap)       # |s| up to 100 nats in the excluded rings, 20 relative to lse
+
+
+@pytest.mark.parametrize("shape, C", [((64, 128, 64, 128), 16), ((40, 80, 40, 80), 64)], ids=["64x128", "40x80"])
+def test_small_probabilities_of_global_attention(shape, C):
+    """Near the poles each of the points gets 2^-20 and less of every output point's attention: dv there is as accurate as elsewhere."""
+    wl = small_workload("global", *shape, 0, 0, math.pi, 1, 1, C, 75)
+    got, refs = run(shape, math.pi, *make_inputs(wl), global_attention=True)
+    for name, x, r in zip(("out", "dq", "dk", "dv"), got, refs):
+        assert rel_points(x, r) <= TOL["fp32"], name
+
+
+@pytest.mark.parametrize("C", [16, 32, 64])
+def test_keys_that_little_attention_reaches(C):
+    """Pairs of rings whose keys lie `gap` nats below the others: their dk and dv are as small, not lost."""
+    wl = small_workload("little", *SHAPE, 0, 0, CUTOFF, 1, 2, C, 76)
+    q, k, v, dout = make_inputs(wl)
+    q, k = q * np.float32(0.1), k * np.float32(0.1)
+    q[..., 0] = 1.0
+    for gap in (5, 15, 30, 60):
+        k[..., 0] = 0.0
+        for h in (4, 5, 10, 11):
+            k[:, :, h, :, 0] = -gap * math.sqrt(C)
+        got, refs = run(SHAPE, CUTOFF, q, k, v, dout)
+        for name, x, r in zip(("dk", "dv"), got[2:], refs[2:]):
+            # p = e^(s - lse): relative to the gap s carries 2^-22 from its split operands and 2^-24 from each of four fp32 roundings
+            # (q log2 e, the scaled sum, lse log2 e, the difference), 2^-21 in all
+            assert rel_points(x[:, :, [4, 5, 10, 11]], r[:, :, [4, 5, 10, 11]]) <= TOL["fp32"] + gap * 2.0 ** -21, (name, gap)
