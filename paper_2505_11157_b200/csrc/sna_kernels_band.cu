@@ -69,23 +69,28 @@ __device__ __forceinline__ uint32_t exponent_bits(float amax) {
 __device__ __forceinline__ float pow2_to(int target, uint32_t ebits) { return __uint_as_float(((uint32_t)(254 + target) << 23) - ebits); }   // 2^(target - e)
 __device__ __forceinline__ float pow2_back(int target, uint32_t ebits) { return __uint_as_float(ebits - ((uint32_t)target << 23)); }        // 2^(e - target)
 
-// Scale of a warp's streamed rows of one array: taken from the first chunk that is not all zero.  It stays 1 (and the scaling is
-// skipped) if that chunk's largest element is in [2^-1, 2^8), and brings it to [2^4, 2^5) otherwise.  The error of a split element
-// is then at most 2^-23 of the element or 2^-24 of that largest one, and FP16 holds elements at least 2^8 times as large.  Rows
-// that are larger still overflow to infinities, which the sums cannot hide: such a tile is computed again with a scale from the
-// largest element of all its rows (StreamScales).
+// Scale of a warp's streamed rows of one array: taken from the first chunk that is not all zero, whose largest element it brings to
+// [2^12, 2^13).  A split element is then held to 2^-23 of itself or to 2^-25 in scaled units (the floor), which is 2^-37 of that
+// largest one, and FP16 holds elements 8 times as large.  (Where that much is not needed, `plain`, as in reduced precision, the scale
+// stays 1 and the scaling is skipped if the largest element is in [2^-1, 2^8).)  Two things can go wrong.  Larger rows overflow to
+// infinities, which the sums cannot hide: the tile is computed again with scales from the largest elements of all its rows.  And
+// sums of which all terms are far below the largest element (a small channel beside a large one, small points beside a large one that
+// is in the window of another row of the tile) may feel the floor: each kernel compares its sums with it at the end and, where one
+// is so small that the floor could be 2^-17 of it and such elements are there, computes the tile again in fp32 (dots_fp32,
+// sums_fp32), which takes four times as long.
 struct StreamScale {
     float scale = 1.f, inv = 1.f;
     bool known = false;
-    // amax: this thread's largest magnitude (called by the whole warp)
-    __device__ __forceinline__ void set(float amax) {
+    // amax: this thread's largest magnitude (called by the whole warp); top: the exponent it gets.  False if it is infinite.
+    __device__ __forceinline__ bool set(float amax, int top, bool plain) {
         const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(amax));
-        if (w == 0) return;
+        if (w == 0) return true;
         const uint32_t eb = exponent_bits(__uint_as_float(w));
         known = true;
-        const bool keep = eb >= (126u << 23) && eb < (135u << 23);
-        scale = keep ? 1.f : pow2_to(4, eb);
-        inv = keep ? 1.f : pow2_back(4, eb);
+        const bool keep = plain && eb >= (126u << 23) && eb < (135u << 23);
+        scale = keep ? 1.f : pow2_to(top, eb);
+        inv = keep ? 1.f : pow2_back(top, eb);
+        return eb < (255u << 23);
     }
 };
 
@@ -175,7 +180,8 @@ struct StreamWalker {
     uint32_t dst, meta;       // where in a stage this lane's first piece and its column's statistics go
     int first, period, stride, lane, C;
 
-    __device__ __forceinline__ void issue(uint32_t st, const int4& e) const {
+    // flat index of the partner point in its slice
+    __device__ __forceinline__ uint32_t index(const int4& e) const {
         int u = e.y;
         if (e.x >= 0) {   // relative to the tile's first point, wrapped around the ring
             u += first;
@@ -183,7 +189,11 @@ struct StreamWalker {
             if (u >= period) u -= period;
             if (u >= period) u -= period;
         }
-        const uint32_t idx = (uint32_t)(e.x & 0x7fffffff) + (uint32_t)(u * stride);      // flat index of the partner point in its slice
+        return (uint32_t)(e.x & 0x7fffffff) + (uint32_t)(u * stride);
+    }
+    __device__ __forceinline__ size_t column(int i) const { return index(__ldg(col - (lane & 15) + i)); }
+    __device__ __forceinline__ void issue(uint32_t st, const int4& e) const {
+        const uint32_t idx = index(e);
         const uint32_t elem = idx * C;      // < 2^32: checked on the host
         const uint32_t to = st + dst;
 #pragma unroll
@@ -287,13 +297,15 @@ template <int CP, bool LP>
 struct SplitRows {
     static constexpr int R = CP / 8;
     uint32_t hi[2][R], lo[LP ? 1 : 2][R];
+    // ALWAYS: the scale is hardly ever 1
+    template <bool ALWAYS = !LP>
     __device__ __forceinline__ void load(uint32_t rows, float sc) {
         using Raw = RawRows<CP>;
 #pragma unroll
         for (int part = 0; part < Raw::PARTS; ++part) {
             Raw r;
             r.load(rows, part);
-            if (sc != 1.f) {
+            if (ALWAYS || sc != 1.f) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -332,25 +344,29 @@ struct StreamScales {
         return m;
     }
     __device__ __forceinline__ bool known() const { return a.known && b.known; }
-    __device__ __forceinline__ void look(uint32_t st) {
-        if (!a.known) a.set(max_abs(st + own + Stage<CP>::A));
-        if (!b.known) b.set(max_abs(st + own + Stage<CP>::B));
+    __device__ __forceinline__ void look(uint32_t st, bool plain_a, bool plain_b) {
+        if (!a.known) a.set(max_abs(st + own + Stage<CP>::A), 12, plain_a);
+        if (!b.known) b.set(max_abs(st + own + Stage<CP>::B), 12, plain_b);
     }
-    // after a pass: whether it has to be done again, because some thread's sums (`total` is not finite if one of them is not)
-    // overflowed; sets the scales from all rows then
+    // From the largest elements of all rows; false if one is infinite.
     template <typename Walker>
-    __device__ __forceinline__ bool again(bool first_pass, float total, const Walker& walker, int nchunks) {
-        if (!__any_sync(FULL, !(fabsf(total) < INFINITY)) || !first_pass) return false;
+    __device__ __forceinline__ bool look_at_all(const Walker& walker, int nchunks) {
         float am = 0.f, bm = 0.f;
         walker.template run<1>(nchunks, [&](uint32_t st, uint32_t, auto&&) {
             am = fmaxf(am, max_abs(st + own + Stage<CP>::A));
             bm = fmaxf(bm, max_abs(st + own + Stage<CP>::B));
         });
-        a.set(am);
-        b.set(bm);
-        return true;
+        const bool fa = a.set(am, 14, false), fb = b.set(bm, 14, false);
+        return fa && fb;
     }
 };
+// After a pass: whether some thread's sums overflowed (`total` is not finite if one of them is not).
+__device__ __forceinline__ bool overflowed(float total) { return __any_sync(FULL, !(fabsf(total) < INFINITY)); }
+// Whether the floors of a tile row's and a streamed row's split operands (both below 2^16) could move a score by more than 2^-17 (log2
+// domain; 2^-11 in reduced precision).  unit: a score's value per product of scaled operands.
+template <bool LP>
+__device__ __forceinline__ bool scores_lost(float unit, int C) { return unit * (float)C > (LP ? 0.15f : 0.0024f); }
+constexpr float REDUCED = 1.f / 128.f;      // single products: sums may be that much smaller before the floor shows (11 against 18 bits)
 
 // Persistent A operand: the tile's rows g and g+8 from two points (pointers at channel 0), scaled by `mul` and by powers of
 // two, one per row or one for the warp's 16 rows (COMMON); back0, back1 undo the latter.
@@ -490,11 +506,115 @@ __device__ __forceinline__ void apply_mask(float (&x)[2][4], uint32_t mask, floa
 #pragma unroll
         for (int i = 0; i < 4; ++i) x[j][i] = (mask & (1u << (4 * j + i))) ? x[j][i] : other;
 }
-__device__ __forceinline__ float max_abs(const float (&x)[2][4]) {
-    float m = 0.f;
+// running maxima of the magnitudes in the thread's two rows
+__device__ __forceinline__ void row_max(float& m0, float& m1, const float (&x)[2][4]) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) m = fmaxf(fmaxf(fmaxf(fmaxf(m, fabsf(x[j][0])), fabsf(x[j][1])), fabsf(x[j][2])), fabsf(x[j][3]));
-    return m;
+    for (int j = 0; j < 2; ++j) {
+        asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m0) : "f"(x[j][0]), "f"(x[j][1]));
+        asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m1) : "f"(x[j][2]), "f"(x[j][3]));
+    }
+}
+__device__ __forceinline__ float group_max(float x) {
+    x = fmaxf(x, __shfl_xor_sync(FULL, x, 1));
+    return fmaxf(x, __shfl_xor_sync(FULL, x, 2));
+}
+
+// ---------------------------------------------------------------------------------------------------------
+// What follows a pass whose sums the FP16 parts may not hold.  Out of line: it takes no registers from the loops.
+// ---------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float4 lds128(uint32_t addr) {
+    float4 x;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr) : "memory");
+    return x;
+}
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float c) { return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, c)))); }
+// d = tile rows g and g+8 (at p0 and p1) . the thread's four columns of the staged rows, in the layout of rows_dot_points
+template <int CP>
+__device__ __forceinline__ void dots_fp32(float (&d)[2][4], const float* p0, const float* p1, uint32_t rows, int C, int t) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) d[j][0] = d[j][1] = d[j][2] = d[j][3] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < C; c += 4) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p0 + c)), b = __ldg(reinterpret_cast<const float4*>(p1 + c));
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float4 x = lds128(rows + (8 * j + 2 * t + i) * Stage<CP>::PITCH + 4 * c);
+                d[j][i] = dot4(a, x, d[j][i]);
+                d[j][2 + i] = dot4(b, x, d[j][2 + i]);
+            }
+    }
+}
+// sum += weights . staged rows, as weights_times_points; points of weight zero (outside the window) do not enter, whatever they hold
+template <int CP>
+__device__ __forceinline__ void sums_fp32(float (&sum)[CP / 8][4], const float (&w)[2][4], uint32_t rows, int t) {
+#pragma unroll 1
+    for (int o = 0; o < 4; ++o)      // the columns of the group's o-th thread
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float w0 = __shfl_sync(FULL, w[j][i], o, 4), w1 = __shfl_sync(FULL, w[j][2 + i], o, 4);
+#pragma unroll
+                for (int m = 0; m < CP / 16; ++m) {
+                    const float4 x = lds128(rows + (8 * j + 2 * o + i) * Stage<CP>::PITCH + 4 * Own<CP>::channel(t, 4 * m));
+                    if (w0 != 0.f) {
+                        sum[2 * m][0] = fmaf(w0, x.x, sum[2 * m][0]); sum[2 * m][1] = fmaf(w0, x.y, sum[2 * m][1]);
+                        sum[2 * m + 1][0] = fmaf(w0, x.z, sum[2 * m + 1][0]); sum[2 * m + 1][1] = fmaf(w0, x.w, sum[2 * m + 1][1]);
+                    }
+                    if (w1 != 0.f) {
+                        sum[2 * m][2] = fmaf(w1, x.x, sum[2 * m][2]); sum[2 * m][3] = fmaf(w1, x.y, sum[2 * m][3]);
+                        sum[2 * m + 1][2] = fmaf(w1, x.z, sum[2 * m + 1][2]); sum[2 * m + 1][3] = fmaf(w1, x.w, sum[2 * m + 1][3]);
+                    }
+                }
+            }
+}
+// Whether sums (small0, small1: of the thread's channels, in its two rows) are small because their terms are too small for the floor, and
+// not because terms cancel.  The streamed rows (`rows`, at the slice) tell: it is so if a row has small sums in a quarter of its
+// channels and some element of one of these is below `tiny`, or if one in 64 elements of such a channel is, which are fewer than
+// the points of one row's window.  (A single small element in a channel and at a point that are not small otherwise is left
+// alone.)  Looking at a channel takes about 2 us, computing the tile again a hundred.
+template <int CP, typename Walker>
+__device__ __noinline__ bool channels_lost(const Walker walker, int nchunks, const float* rows, float tiny, uint32_t small0, uint32_t small1, int C, int t) {
+    constexpr int QUADS = CP / 16;        // of channels per thread
+    int in_row = __popc(small0) | __popc(small1) << 16;
+    in_row += __shfl_xor_sync(FULL, in_row, 1);
+    in_row += __shfl_xor_sync(FULL, in_row, 2);
+    const bool many = __any_sync(FULL, max(in_row & 0xffff, in_row >> 16) * 4 >= C);
+#pragma unroll 1
+    for (int o = 0; o < 4 * QUADS; ++o) {
+        const int owner = o / QUADS, quad = o % QUADS;
+        const uint32_t which = __reduce_or_sync(FULL, t == owner ? (small0 | small1) >> 4 * quad & 15u : 0u);
+        if (which == 0) continue;
+        const float* at = rows + Own<CP>::channel(owner, 4 * quad);
+        int tiny_ones[4] = {0, 0, 0, 0};
+#pragma unroll 4
+        for (int col = walker.lane; col < nchunks * BAND_CHUNK; col += 32) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(at + walker.column(col) * C));
+            const float y[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tiny_ones[i] += y[i] != 0.f && fabsf(y[i]) < tiny;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int all = __reduce_add_sync(FULL, tiny_ones[i]);
+            if ((which >> i & 1u) != 0 && all > 0 && (many || all * 64LL >= nchunks * BAND_CHUNK)) return true;
+        }
+    }
+    return false;
+}
+// ... of sums below the row's limit: 0.3 % of the tiles of normally distributed data have one.
+template <int CP, typename Walker>
+__device__ __forceinline__ bool sums_lost(const float (&sum)[CP / 8][4], float limit0, float limit1, const Walker& walker, int nchunks, const float* rows, float tiny, int C, int t) {
+    uint32_t small0 = 0, small1 = 0;
+#pragma unroll
+    for (int i = 0; i < CP / 4; ++i)
+        if (Own<CP>::channel(t, i & ~3) < C) {
+            if (fabsf(sum[i / 2][i % 2]) < limit0) small0 |= 1u << i;
+            if (fabsf(sum[i / 2][2 + i % 2]) < limit1) small1 |= 1u << i;
+        }
+    return __any_sync(FULL, (small0 | small1) != 0) && channels_lost<CP>(walker, nchunks, rows, tiny, small0, small1, C, t);
 }
 __device__ __forceinline__ uint64_t lds64(uint32_t addr) {
     uint64_t x;
@@ -583,6 +703,12 @@ struct Exchange {
 #pragma unroll
             for (int i = 0; i < 4; ++i) at(warp, first + 4 * nt + i) = x[nt][i] * (i < 2 ? f0 : f1);
     }
+    __device__ __forceinline__ void get(float (&x)[CP / 8][4], int warp, int first) const {
+#pragma unroll
+        for (int nt = 0; nt < CP / 8; ++nt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[nt][i] = at(warp, first + 4 * nt + i);
+    }
     // f0, f1 [warp]: factors of the warps' rows g and g + 8
     __device__ __forceinline__ void add(float (&x)[CP / 8][4], const Task& task, int first, const float (&f0)[WARPS], const float (&f1)[WARPS]) const {
 #pragma unroll
@@ -635,6 +761,107 @@ __device__ __forceinline__ void seed(float lse, float& m, float& w) {
     w = ex2(fmaf(lse, LOG2E, -whole)) / W_UNIT;
 }
 
+// The softmax of the thread's two rows, over its columns.
+struct Softmax {
+    float m0, m1, top0, top1;          // top: scores (relative to m) up to this need no new reference
+    uint64_t l0, l1;                   // two partial sums each
+    // Starts a pass, with sums o (v unscaled): from the dense kernel's partial result of a row (normalised out and lse), one weight of
+    // value 2^lse, if `seeded` and there is one.
+    template <int CP>
+    __device__ __forceinline__ void start(bool seeded, const BandView& view, const TilePoints& at, const float* out, const float* lse, float (&o)[CP / 8][4], int C, int t) {
+        clear(o);
+        m0 = m1 = 0.f; top0 = top1 = -INFINITY;
+        l0 = l1 = 0;
+        if (!seeded) return;
+        if (view.dense_ptr[at.ha + 1] > view.dense_ptr[at.ha]) {
+            float w;
+            seed(lse[at.pt0], m0, w);
+            top0 = W_MAX;
+#pragma unroll
+            for (int m = 0; m < CP / 16; ++m) {
+                const float4 x = load_quad<CP>(out + at.pt0 * C, m, C, t);
+                o[2 * m][0] = x.x * w; o[2 * m][1] = x.y * w; o[2 * m + 1][0] = x.z * w; o[2 * m + 1][1] = x.w * w;
+            }
+            if (t == 0) l0 = pack2(w, 0.f);
+        }
+        if (view.dense_ptr[at.hb + 1] > view.dense_ptr[at.hb]) {
+            float w;
+            seed(lse[at.pt1], m1, w);
+            top1 = W_MAX;
+#pragma unroll
+            for (int m = 0; m < CP / 16; ++m) {
+                const float4 x = load_quad<CP>(out + at.pt1 * C, m, C, t);
+                o[2 * m][2] = x.x * w; o[2 * m][3] = x.y * w; o[2 * m + 1][2] = x.z * w; o[2 * m + 1][3] = x.w * w;
+            }
+            if (t == 0) l1 = pack2(w, 0.f);
+        }
+    }
+    // s: a chunk's products in, its weights out.  f2: a score per product.
+    template <int N>
+    __device__ __forceinline__ void weights(float (&s)[2][4], float (&o)[N][4], uint64_t f2, const uint64_t (&bias2)[2], uint32_t mask) {
+        const uint64_t m02 = both(m0), m12 = both(m1);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            unpack2(fma2(pack2(s[j][0], s[j][1]), f2, sub2(bias2[j], m02)), s[j][0], s[j][1]);
+            unpack2(fma2(pack2(s[j][2], s[j][3]), f2, sub2(bias2[j], m12)), s[j][2], s[j][3]);
+        }
+        if (!(mask & BAND_ALL)) apply_mask(s, mask, -INFINITY);   // some tile row skips some column of this chunk
+        float mx0 = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1])), mx1 = fmaxf(fmaxf(s[0][2], s[0][3]), fmaxf(s[1][2], s[1][3]));
+        if (__any_sync(FULL, mx0 > top0 || mx1 > top1)) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, 1));
+            mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, 2)); mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, 2));
+            const bool up0 = mx0 > top0, up1 = mx1 > top1;
+            const float d0 = up0 ? mx0 - W_SET : 0.f, d1 = up1 ? mx1 - W_SET : 0.f;
+            // (a row without a reference has collected nothing: any finite factor will do)
+            const float r0 = top0 == -INFINITY ? 1.f : ex2(-d0), r1 = top1 == -INFINITY ? 1.f : ex2(-d1);
+            m0 += d0; m1 += d1;
+            if (up0) top0 = W_MAX;
+            if (up1) top1 = W_MAX;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) { s[j][0] -= d0; s[j][1] -= d0; s[j][2] -= d1; s[j][3] -= d1; }
+            l0 = mul2(l0, both(r0)); l1 = mul2(l1, both(r1));
+            scale_rows(o, r0, r1);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
+            l0 = add2(l0, pack2(s[j][0], s[j][1]));
+            l1 = add2(l1, pack2(s[j][2], s[j][3]));
+        }
+    }
+};
+// a row's sum across the four threads of a group
+__device__ __forceinline__ float group_sum(uint64_t x) {
+    float s = sum2(x);
+    s += __shfl_xor_sync(FULL, s, 1);
+    return s + __shfl_xor_sync(FULL, s, 2);
+}
+// A warp's pass in fp32; leaves the sums, the references and the rows' sums in the warp's staging memory (Exchange).
+template <int CP, typename Walker>
+__device__ __noinline__ void forward_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const BandView& view, bool seeded, const TilePoints at,
+                                          const float* q, const float* out, const float* lse, int C, float scale_log2) {
+    using S = Stage<CP>;
+    const int t = walker.lane & 3, warp = threadIdx.x >> 5;
+    float o[CP / 8][4];
+    Softmax sm;
+    sm.start<CP>(seeded, view, at, out, lse, o, C, t);
+    walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
+        float s[2][4];
+        dots_fp32<CP>(s, q + at.pt0 * C, q + at.pt1 * C, st + S::A, C, t);
+        const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
+        sm.weights(s, o, both(scale_log2), bias2, mask);
+        sums_fp32<CP>(o, s, st + S::B, t);
+    });
+    const float ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
+    const Exchange<CP> x(smem_raw);
+    x.put(o, warp, 0, 1.f, 1.f);
+    const float rest[6] = {sm.m0, sm.m1, sm.top0, sm.top1, t == 0 ? ls0 : 0.f, t == 0 ? ls1 : 0.f};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) x.at(warp, CP / 2 + i) = rest[i];
+    __syncwarp();
+}
+
 // Blocks of 4 warps per SM: as many as the registers of the kernel allow without spills that matter.  Measured at 128x256, N = 16,
 // C = 32 (whole streams): forward 4 blocks 333 us, 5 blocks 338; dq 3 / 4 / 5 blocks 419 / 383 / 550 us; dk/dv 3 / 4 blocks
 // 455 / 589.  Single products need fewer registers: forward 5 blocks 271 us, 4 blocks 281.
@@ -668,46 +895,22 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
     task.chunks(view, group, chunk0, nchunks);
     const auto walker = make_walker<CP, false, PAD>(smem_raw, view.s, chunk0, w0, p.nlon_out, p.ps, C, k + slice, v + slice, nullptr, nullptr);
     float o[NT][4];
-    float m0, m1, top0, top1;          // top: scores (relative to m) up to this need no new reference
-    uint64_t l0, l1;                   // two partial sums each
+    Softmax sm;
     uint64_t bad;
+    const bool plain = !scores_lost<LP>(Q.back0, C);      // k needs no scale of its own for scores of this size
     for (bool first_pass = true;; first_pass = false) {
-        clear(o);
-        m0 = m1 = 0.f; top0 = top1 = -INFINITY;
-        l0 = l1 = bad = 0;
         const bool seeded = view.dense_ptr != nullptr && (!task.shared || task.warp == 0);
-        if (seeded) {
-            if (view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
-            // continue from the dense kernel's partial result of this row (normalised out and lse), one weight of value 2^lse
+        {
             const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-            if (view.dense_ptr[at.ha + 1] > view.dense_ptr[at.ha]) {
-                float w;
-                seed(lse[at.pt0], m0, w);
-                top0 = W_MAX;
-#pragma unroll
-                for (int m = 0; m < NT / 2; ++m) {
-                    const float4 x = load_quad<CP>(out + at.pt0 * C, m, C, t);
-                    o[2 * m][0] = x.x * w; o[2 * m][1] = x.y * w; o[2 * m + 1][0] = x.z * w; o[2 * m + 1][1] = x.w * w;
-                }
-                if (t == 0) l0 = pack2(w, 0.f);
-            }
-            if (view.dense_ptr[at.hb + 1] > view.dense_ptr[at.hb]) {
-                float w;
-                seed(lse[at.pt1], m1, w);
-                top1 = W_MAX;
-#pragma unroll
-                for (int m = 0; m < NT / 2; ++m) {
-                    const float4 x = load_quad<CP>(out + at.pt1 * C, m, C, t);
-                    o[2 * m][2] = x.x * w; o[2 * m][3] = x.y * w; o[2 * m + 1][2] = x.z * w; o[2 * m + 1][3] = x.w * w;
-                }
-                if (t == 0) l1 = pack2(w, 0.f);
-            }
-            scale_rows(o, sc.b.scale, sc.b.scale);
+            if (seeded && view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
+            sm.template start<CP>(seeded, view, at, out, lse, o, C, t);
         }
+        bad = 0;
+        scale_rows(o, sc.b.scale, sc.b.scale);
         walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
             if (!sc.known()) {
                 const float before = sc.b.scale;
-                sc.look(st);
+                sc.look(st, plain, LP);
                 if (seeded) scale_rows(o, sc.b.scale / before, sc.b.scale / before);
             }
             float s[2][4];
@@ -715,60 +918,50 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
             constexpr bool EARLY = CP < 64 && !LP;      // read v while the scores are computed, if there are registers for it
             {
                 SplitRows<CP, LP> K;
-                K.load(st + sc.own + S::A, sc.a.scale);
+                K.template load<false>(st + sc.own + S::A, sc.a.scale);
                 if constexpr (EARLY) V.load(st + sc.own + S::B, sc.b.scale);
                 rows_dot_points<CP, LP>(s, Q, K);
             }
             const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
             note_overflow<LP>(bad, s);
-            const uint64_t f2 = both(Q.back0 * sc.a.inv), m02 = both(m0), m12 = both(m1);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                unpack2(fma2(pack2(s[j][0], s[j][1]), f2, sub2(bias2[j], m02)), s[j][0], s[j][1]);
-                unpack2(fma2(pack2(s[j][2], s[j][3]), f2, sub2(bias2[j], m12)), s[j][2], s[j][3]);
-            }
-            if (!(mask & BAND_ALL)) apply_mask(s, mask, -INFINITY);   // some tile row skips some column of this chunk
-            float mx0 = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1])), mx1 = fmaxf(fmaxf(s[0][2], s[0][3]), fmaxf(s[1][2], s[1][3]));
-            if (__any_sync(FULL, mx0 > top0 || mx1 > top1)) {
-                mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, 1));
-                mx0 = fmaxf(mx0, __shfl_xor_sync(FULL, mx0, 2)); mx1 = fmaxf(mx1, __shfl_xor_sync(FULL, mx1, 2));
-                const bool up0 = mx0 > top0, up1 = mx1 > top1;
-                const float d0 = up0 ? mx0 - W_SET : 0.f, d1 = up1 ? mx1 - W_SET : 0.f;
-                // (a row without a reference has collected nothing: any finite factor will do)
-                const float r0 = top0 == -INFINITY ? 1.f : ex2(-d0), r1 = top1 == -INFINITY ? 1.f : ex2(-d1);
-                m0 += d0; m1 += d1;
-                if (up0) top0 = W_MAX;
-                if (up1) top1 = W_MAX;
-#pragma unroll
-                for (int j = 0; j < 2; ++j) { s[j][0] -= d0; s[j][1] -= d0; s[j][2] -= d1; s[j][3] -= d1; }
-                l0 = mul2(l0, both(r0)); l1 = mul2(l1, both(r1));
-                scale_rows(o, r0, r1);
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
-                l0 = add2(l0, pack2(s[j][0], s[j][1]));
-                l1 = add2(l1, pack2(s[j][2], s[j][3]));
-            }
+            sm.weights(s, o, both(Q.back0 * sc.a.inv), bias2, mask);
             Weights<LP> W;
             W.set(s);
             if constexpr (!EARLY) V.load(st + sc.own + S::B, sc.b.scale);
             weights_times_points<CP, LP>(o, W, V);
         });
-        if (!sc.again(first_pass, sum2(add2(l0, l1)) + sum2(bad) + total(o), walker, nchunks)) break;
+        if (overflowed(sum2(add2(sm.l0, sm.l1)) + sum2(bad) + total(o))) {
+            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
+        } else {
+            // an output's floor is 2^-25 of its scaled v, which shows from 2^-8 on
+            constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;
+            const float ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
+            const bool lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) ||
+                              (sc.b.known && sums_lost<CP>(o, ls0 * LIMIT, ls1 * LIMIT, walker, nchunks, v + slice, LIMIT * sc.b.inv, C, t));
+            if (!lost) break;
+        }
+        {
+            const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
+            forward_fp32<CP>(smem_raw, walker, nchunks, view, seeded, at, q, out, lse, C, scale_log2);
+        }
+        const Exchange<CP> x(smem_raw);
+        x.get(o, task.warp, 0);
+        sm.m0 = x.at(task.warp, CP / 2); sm.m1 = x.at(task.warp, CP / 2 + 1);
+        sm.top0 = x.at(task.warp, CP / 2 + 2); sm.top1 = x.at(task.warp, CP / 2 + 3);
+        sm.l0 = pack2(x.at(task.warp, CP / 2 + 4), 0.f); sm.l1 = pack2(x.at(task.warp, CP / 2 + 5), 0.f);
+        __syncwarp();
+        sc.b = StreamScale();
+        break;
     }
     const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-    // row sums across the four threads of a group, normalise, store
-    float ls0 = sum2(l0), ls1 = sum2(l1);
-    ls0 += __shfl_xor_sync(FULL, ls0, 1); ls1 += __shfl_xor_sync(FULL, ls1, 1);
-    ls0 += __shfl_xor_sync(FULL, ls0, 2); ls1 += __shfl_xor_sync(FULL, ls1, 2);
+    // normalise, store
+    float m0 = sm.m0, m1 = sm.m1, ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
     float back0 = sc.b.inv, back1 = sc.b.inv;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(o, task.warp, 0, sc.b.inv, sc.b.inv);
-        x.at(task.warp, CP / 2) = top0 == -INFINITY ? -INFINITY : m0;       // (a warp may have had no column for a row)
-        x.at(task.warp, CP / 2 + 1) = top1 == -INFINITY ? -INFINITY : m1;
+        x.at(task.warp, CP / 2) = sm.top0 == -INFINITY ? -INFINITY : m0;       // (a warp may have had no column for a row)
+        x.at(task.warp, CP / 2 + 1) = sm.top1 == -INFINITY ? -INFINITY : m1;
         x.at(task.warp, CP / 2 + 2) = ls0;
         x.at(task.warp, CP / 2 + 3) = ls1;
         __syncthreads();
@@ -810,6 +1003,33 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
 // `out` and `dq` may be the same buffer: a warp reads its own 16 rows of `out` before it writes them as dq.
 // t, D and ds are in the units of the scaled dout row and the scaled v until the end.
 // ---------------------------------------------------------------------------------------------------------
+// A warp's pass in fp32; leaves the sums in its staging memory.
+template <int CP, typename Walker>
+__device__ __noinline__ void dq_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const TilePoints at, const float* q, const float* dout,
+                                     float lse0, float lse1, float D0, float D1, int C, float scale_log2) {
+    using S = Stage<CP>;
+    const int t = walker.lane & 3;
+    float acc[CP / 8][4];
+    clear(acc);
+    walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
+        float s[2][4], tt[2][4];
+        dots_fp32<CP>(s, q + at.pt0 * C, q + at.pt1 * C, st + S::A, C, t);
+        dots_fp32<CP>(tt, dout + at.pt0 * C, dout + at.pt1 * C, st + S::B, C, t);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float b[2];
+            unpack2(lds64(st + S::M0 + 32 * j + 8 * t), b[0], b[1]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                s[j][i] = ex2(fmaf(s[j][i], scale_log2, fmaf(i < 2 ? lse0 : lse1, -LOG2E, b[i % 2]))) * (tt[j][i] - (i < 2 ? D0 : D1));
+        }
+        apply_mask(s, mask, 0.f);
+        sums_fp32<CP>(acc, s, st + S::A, t);
+    });
+    Exchange<CP>(smem_raw).put(acc, threadIdx.x >> 5, 0, 1.f, 1.f);
+    __syncwarp();
+}
+
 template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DQ)
 backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
@@ -856,15 +1076,19 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
     const auto walker = make_walker<CP, false, PAD>(smem_raw, view.s, chunk0, w0, p.nlon_out, p.ps, C, k + slice, v + slice, nullptr, nullptr);
     float acc[NT][4];
     WeightScale ws;          // of ds
+    float nD0, nD1;          // -D times the weight scale
+    float max0, max1;        // largest |ds| of the thread's columns
+    float f0, f1;            // dq per sum
     for (bool first_pass = true;; first_pass = false) {
         clear(acc);
         ws = WeightScale();
         uint64_t bad = 0;
-        float nD0 = -D0 / Y.back0 * sc.b.scale, nD1 = -D1 / Y.back1 * sc.b.scale;      // times the weight scale
+        nD0 = -D0 / Y.back0 * sc.b.scale; nD1 = -D1 / Y.back1 * sc.b.scale;
+        max0 = max1 = 0.f;
         walker.template run<LP && CP == 32 ? 1 : 2>(nchunks, [&](uint32_t st, uint32_t mask, auto&& release) {
             if (!sc.known()) {
                 const float before = sc.b.scale;
-                sc.look(st);
+                sc.look(st, LP, LP);
                 const float f = sc.b.scale / before;
                 nD0 *= f; nD1 *= f;
                 scale_rows(acc, f, f);
@@ -892,21 +1116,42 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
                 unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, both(nD1))), s[j][2], s[j][3]);
             }
             if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
-            const float wmax = max_abs(s);
-            if (__any_sync(FULL, wmax > ws.limit)) {
-                const float f = ws.update(wmax);
+            row_max(max0, max1, s);
+            if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
+                const float f = ws.update(fmaxf(max0, max1));
                 scale_rows(acc, f, f);
                 scale_rows(s, f, f);
                 nD0 *= f; nD1 *= f;
+                max0 *= f; max1 *= f;
             }
             Weights<LP> W;
             W.set(s);
             weights_times_points<CP, LP>(acc, W, K);
         });
-        if (!sc.again(first_pass, total(acc) + sum2(bad), walker, nchunks)) break;
+        f0 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back0; f1 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back1;
+        if (overflowed(total(acc) + sum2(bad))) {
+            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
+        } else {
+            // The floors: of ds, 2^-25; of t, below 2^-8 in units of ds's scale.  They are compared with the row's largest ds or, if
+            // t and D nearly cancel, with p D, whose rounding is an error of ds in any case (the row's p add up to 1).
+            const float r0 = group_max(max0), r1 = group_max(max1), least = (LP ? REDUCED : 1.f) * fmaxf(1.f / 128.f, 1024.f * ws.scale);
+            const float any = 1.f / (64.f * (float)nchunks);
+            const bool low = (r0 > 0.f && fmaxf(r0, any * fabsf(nD0)) < least) || (r1 > 0.f && fmaxf(r1, any * fabsf(nD1)) < least);
+            constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;         // of k, in a sum
+            const bool lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) || (sc.b.known && __any_sync(FULL, low)) ||
+                              (sc.a.known && sums_lost<CP>(acc, r0 * LIMIT, r1 * LIMIT, walker, nchunks, k + slice, LIMIT * sc.a.inv, C, t));
+            if (!lost) break;
+        }
+        {
+            const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
+            dq_fp32<CP>(smem_raw, walker, nchunks, at, q, dout, lse0, lse1, D0, D1, C, scale * LOG2E);
+        }
+        Exchange<CP>(smem_raw).get(acc, task.warp, 0);
+        __syncwarp();
+        f0 = f1 = scale;
+        break;
     }
     const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-    float f0 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back0, f1 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back1;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(acc, task.warp, 0, f0, f1);
@@ -940,6 +1185,41 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
 //   dk_j = scale * sum_i p_ij (t_ij - D_i) q_i,   dv_j = sum_i p_ij dout_i          (App. B.4)
 // Tile rows are 8 input columns on each of the two rings of an input ring pair; stream columns are output points.
 // ---------------------------------------------------------------------------------------------------------
+// A warp's pass in fp32; leaves the sums in its staging memory.
+template <int CP, typename Walker>
+__device__ __noinline__ void dkdv_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const TilePoints at, const float* k, const float* v,
+                                       float bias0, float bias1, int C, float scale_log2) {
+    using S = Stage<CP>;
+    const int t = walker.lane & 3;
+    float gk[CP / 8][4], gv[CP / 8][4];
+    clear(gk);
+    clear(gv);
+    walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
+        float s[2][4], tt[2][4];
+        dots_fp32<CP>(s, k + at.pt0 * C, k + at.pt1 * C, st + S::A, C, t);
+        dots_fp32<CP>(tt, v + at.pt0 * C, v + at.pt1 * C, st + S::B, C, t);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float l[2], D[2];
+            unpack2(lds64(st + S::M0 + 32 * j + 8 * t), l[0], l[1]);
+            unpack2(lds64(st + S::M1 + 32 * j + 8 * t), D[0], D[1]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[j][i] = ex2(fmaf(s[j][i], scale_log2, fmaf(l[i % 2], -LOG2E, i < 2 ? bias0 : bias1)));
+                tt[j][i] = s[j][i] * (tt[j][i] - D[i % 2]);
+            }
+        }
+        apply_mask(s, mask, 0.f);
+        apply_mask(tt, mask, 0.f);
+        sums_fp32<CP>(gv, s, st + S::B, t);
+        sums_fp32<CP>(gk, tt, st + S::A, t);
+    });
+    const Exchange<CP> x(smem_raw);
+    x.put(gk, threadIdx.x >> 5, 0, 1.f, 1.f);
+    x.put(gv, threadIdx.x >> 5, CP / 2, 1.f, 1.f);
+    __syncwarp();
+}
+
 template <int CP, bool LP, bool PAD, bool CF>
 __global__ void __launch_bounds__(THREADS, Blocks<CP, LP>::DKDV)
 backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v,
@@ -979,18 +1259,26 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
     task.chunks(view, srow, chunk0, nchunks);
     const auto walker = make_walker<CP, true, PAD>(smem_raw, view.s, chunk0, first, p.nlon_out, 1, C, q + oslice * C, dout + oslice * C, lse + oslice, Dws + oslice);
     float gk[NT][4], gv[NT][4];
-    WeightScale wp, ws;      // of p (over global attention or for keys that little attention reaches all of them are small) and, beyond that, of ds
+    // The scale of p: over global attention, and for keys that little attention reaches, all of them are small.  It brings the largest
+    // of the first chunk that has some to [2^3, 2^4), so that a p 2^12 times as large still fits; if one does not, the pass is
+    // repeated with 2^15, which holds p = 1.
+    float p_scale;
+    WeightScale ws;          // of ds, beyond that
+    float pmax0, pmax1, max0, max1;      // largest p and |ds| of the thread's columns
+    float fk, fv;            // dk and dv per sum
     for (bool first_pass = true;; first_pass = false) {
         clear(gk);
         clear(gv);
-        wp = ws = WeightScale();
-        float b0 = bias0, b1 = bias1;           // with the exponent of p's scale
+        ws = WeightScale();
+        p_scale = first_pass ? 0.f : 32768.f;       // 0: not known
+        float b0 = first_pass ? bias0 : bias0 + 15.f, b1 = first_pass ? bias1 : bias1 + 15.f;           // with the exponent of p's scale
         float unit = sc.b.scale / V.back0;      // t, D and ds are in the units of the scaled dout and v until the end
         uint64_t bad = 0;
+        pmax0 = pmax1 = max0 = max1 = 0.f;
         walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
             if (!sc.known()) {
                 const float before = sc.b.scale;
-                sc.look(st);
+                sc.look(st, LP, LP);
                 unit *= sc.b.scale / before;
                 scale_rows(gk, sc.b.scale / before, sc.b.scale / before);
             }
@@ -1012,14 +1300,16 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
                 for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
             }
             if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
-            const float pmax = max_abs(s);
-            if (__any_sync(FULL, pmax > wp.limit)) {
-                const float f = wp.update(pmax);
-                const float e = (float)((int)(__float_as_uint(f) >> 23) - 127);
-                b0 += e; b1 += e;
-                scale_rows(gv, f, f);
-                scale_rows(gk, f, f);
-                scale_rows(s, f, f);
+            row_max(pmax0, pmax1, s);
+            if (p_scale == 0.f) {
+                const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(fmaxf(pmax0, pmax1)));
+                if (w != 0) {
+                    p_scale = pow2_to(3, max(w & 0x7f800000u, (uint32_t)(127 - 72) << 23));
+                    const float e = (float)((int)(__float_as_uint(p_scale) >> 23) - 127);
+                    b0 += e; b1 += e;
+                    scale_rows(s, p_scale, p_scale);
+                    pmax0 *= p_scale; pmax1 *= p_scale;
+                }
             }
             Weights<LP> P, W;
             P.set(s);
@@ -1029,21 +1319,44 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
                 unpack2(mul2(pack2(s[j][0], s[j][1]), fma2(pack2(tt[j][0], tt[j][1]), h2, nD2)), s[j][0], s[j][1]);      // ds
                 unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, nD2)), s[j][2], s[j][3]);
             }
-            const float wmax = max_abs(s);
-            if (__any_sync(FULL, wmax > ws.limit)) {
-                const float f = ws.update(wmax);
+            row_max(max0, max1, s);
+            if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
+                const float f = ws.update(fmaxf(max0, max1));
                 scale_rows(gk, f, f);
                 scale_rows(s, f, f);
+                max0 *= f; max1 *= f;
             }
             W.set(s);
             weights_times_points<CP, LP>(gv, P, Y);
             weights_times_points<CP, LP>(gk, W, Q);
         });
-        if (!sc.again(first_pass, total(gk) + total(gv) + sum2(bad), walker, nchunks)) break;
+        // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry p's scale.
+        const float p_back = p_scale == 0.f ? 0.f : 1.f / p_scale;       // (0: no p at all)
+        fk = scale * sc.a.inv / ws.scale * sc.b.inv * p_back * V.back0; fv = sc.b.inv * p_back;
+        if (overflowed(total(gk) + total(gv) + sum2(bad))) {
+            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
+        } else {
+            // The floors: of p and ds, 2^-25; of t, below 2^-8 in units of ds's scale and times p.
+            const float p0 = group_max(pmax0), p1 = group_max(pmax1), r0 = group_max(max0), r1 = group_max(max1);
+            constexpr float LEAST = (LP ? REDUCED : 1.f) / 128.f, LIMIT = (LP ? REDUCED : 1.f) / 256.f;      // (LIMIT: of q and dout, in a sum)
+            const float of_t = (LP ? REDUCED : 1.f) * 1024.f * ws.scale;
+            const bool low = (p0 > 0.f && p0 < LEAST) || (p1 > 0.f && p1 < LEAST) || (r0 > 0.f && r0 < fmaxf(LEAST, of_t * p0)) || (r1 > 0.f && r1 < fmaxf(LEAST, of_t * p1));
+            const bool lost = (sc.a.known && scores_lost<LP>(K.back0 * sc.a.inv, C)) || __any_sync(FULL, low) ||
+                              (sc.b.known && sums_lost<CP>(gv, p0 * LIMIT, p1 * LIMIT, walker, nchunks, dout + oslice * C, LIMIT * sc.b.inv, C, t)) ||
+                              (sc.a.known && sums_lost<CP>(gk, r0 * LIMIT, r1 * LIMIT, walker, nchunks, q + oslice * C, LIMIT * sc.a.inv, C, t));
+            if (!lost) break;
+        }
+        {
+            const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
+            dkdv_fp32<CP>(smem_raw, walker, nchunks, at, k, v, bias0, bias1, C, scale * LOG2E);
+        }
+        Exchange<CP>(smem_raw).get(gk, task.warp, 0);
+        Exchange<CP>(smem_raw).get(gv, task.warp, CP / 2);
+        __syncwarp();
+        fk = scale; fv = 1.f;
+        break;
     }
     const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
-    // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry p's scale.
-    float fk = scale * sc.a.inv / ws.scale * sc.b.inv / wp.scale * V.back0, fv = sc.b.inv / wp.scale;
     if (task.shared) {
         const Exchange<CP> x(smem_raw);
         x.put(gk, task.warp, 0, fk, fk);
