@@ -70,27 +70,27 @@ __device__ __forceinline__ float pow2_to(int target, uint32_t ebits) { return __
 __device__ __forceinline__ float pow2_back(int target, uint32_t ebits) { return __uint_as_float(ebits - ((uint32_t)target << 23)); }        // 2^(e - target)
 
 // Scale of a warp's streamed rows of one array: taken from the first chunk that is not all zero, whose largest element it brings to
-// [2^12, 2^13).  A split element is then held to 2^-23 of itself or to 2^-25 in scaled units (the floor), which is 2^-37 of that
-// largest one, and FP16 holds elements 8 times as large.  (Where that much is not needed, `plain`, as in reduced precision, the scale
+// [2^11, 2^12).  A split element is then held to 2^-23 of itself or to 2^-25 in scaled units (the floor), which is 2^-36 of that
+// largest one, and FP16 holds elements 16 times as large.  (Where that much is not needed, `plain`, as in reduced precision, the scale
 // stays 1 and the scaling is skipped if the largest element is in [2^-1, 2^8).)  Two things can go wrong.  Larger rows overflow to
-// infinities, which the sums cannot hide: the tile is computed again with scales from the largest elements of all its rows.  And
-// sums of which all terms are far below the largest element (a small channel beside a large one, small points beside a large one that
-// is in the window of another row of the tile) may feel the floor: each kernel compares its sums with it at the end and, where one
-// is so small that the floor could be 2^-17 of it and such elements are there, computes the tile again in fp32 (dots_fp32,
-// sums_fp32), which takes four times as long.
+// infinities, which the sums cannot hide.  And sums of which all terms are far below the largest element (a small channel beside a
+// large one, small points beside a large one that is in the window of another row of the tile) may feel the floor: each kernel
+// compares its sums with it at the end.  Where they overflowed, or one is so small that the floor could be 2^-17 of it and such
+// elements are there, the warp computes its part of the tile again in fp32 (dots_fp32, sums_fp32), which takes four times as long.
+// What the scaling and the checks cost (128x256, cutoff 4 rings, C = 32, N = 16, us forward / dq / dk+dv): 333/362/447 -> 349/370/472.
+// A second pass with scales from all rows, for overflows, cost as much again in registers.
 struct StreamScale {
     float scale = 1.f, inv = 1.f;
     bool known = false;
-    // amax: this thread's largest magnitude (called by the whole warp); top: the exponent it gets.  False if it is infinite.
-    __device__ __forceinline__ bool set(float amax, int top, bool plain) {
+    // amax: this thread's largest magnitude (called by the whole warp)
+    __device__ __forceinline__ void set(float amax, bool plain) {
         const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(amax));
-        if (w == 0) return true;
+        if (w == 0) return;
         const uint32_t eb = exponent_bits(__uint_as_float(w));
         known = true;
         const bool keep = plain && eb >= (126u << 23) && eb < (135u << 23);
-        scale = keep ? 1.f : pow2_to(top, eb);
-        inv = keep ? 1.f : pow2_back(top, eb);
-        return eb < (255u << 23);
+        scale = keep ? 1.f : pow2_to(11, eb);
+        inv = keep ? 1.f : pow2_back(11, eb);
     }
 };
 
@@ -345,19 +345,8 @@ struct StreamScales {
     }
     __device__ __forceinline__ bool known() const { return a.known && b.known; }
     __device__ __forceinline__ void look(uint32_t st, bool plain_a, bool plain_b) {
-        if (!a.known) a.set(max_abs(st + own + Stage<CP>::A), 12, plain_a);
-        if (!b.known) b.set(max_abs(st + own + Stage<CP>::B), 12, plain_b);
-    }
-    // From the largest elements of all rows; false if one is infinite.
-    template <typename Walker>
-    __device__ __forceinline__ bool look_at_all(const Walker& walker, int nchunks) {
-        float am = 0.f, bm = 0.f;
-        walker.template run<1>(nchunks, [&](uint32_t st, uint32_t, auto&&) {
-            am = fmaxf(am, max_abs(st + own + Stage<CP>::A));
-            bm = fmaxf(bm, max_abs(st + own + Stage<CP>::B));
-        });
-        const bool fa = a.set(am, 14, false), fb = b.set(bm, 14, false);
-        return fa && fb;
+        if (!a.known) a.set(max_abs(st + own + Stage<CP>::A), plain_a);
+        if (!b.known) b.set(max_abs(st + own + Stage<CP>::B), plain_b);
     }
 };
 // After a pass: whether some thread's sums overflowed (`total` is not finite if one of them is not).
@@ -366,7 +355,7 @@ __device__ __forceinline__ bool overflowed(float total) { return __any_sync(FULL
 // domain; 2^-11 in reduced precision).  unit: a score's value per product of scaled operands.
 template <bool LP>
 __device__ __forceinline__ bool scores_lost(float unit, int C) { return unit * (float)C > (LP ? 0.15f : 0.0024f); }
-constexpr float REDUCED = 1.f / 128.f;      // single products: sums may be that much smaller before the floor shows (11 against 18 bits)
+constexpr float REDUCED = 1.f / 256.f;      // single products: sums may be that much smaller before the floor shows beside their 10 bits
 
 // Persistent A operand: the tile's rows g and g+8 from two points (pointers at channel 0), scaled by `mul` and by powers of
 // two, one per row or one for the warp's 16 rows (COMMON); back0, back1 undo the latter.
@@ -520,7 +509,7 @@ __device__ __forceinline__ float group_max(float x) {
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// What follows a pass whose sums the FP16 parts may not hold.  Out of line: it takes no registers from the loops.
+// What follows a pass whose sums the FP16 parts may not hold
 // ---------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 lds128(uint32_t addr) {
     float4 x;
@@ -576,7 +565,7 @@ __device__ __forceinline__ void sums_fp32(float (&sum)[CP / 8][4], const float (
 // the points of one row's window.  (A single small element in a channel and at a point that are not small otherwise is left
 // alone.)  Looking at a channel takes about 2 us, computing the tile again a hundred.
 template <int CP, typename Walker>
-__device__ __noinline__ bool channels_lost(const Walker walker, int nchunks, const float* rows, float tiny, uint32_t small0, uint32_t small1, int C, int t) {
+__device__ __forceinline__ bool channels_lost(const Walker walker, int nchunks, const float* rows, float tiny, uint32_t small0, uint32_t small1, int C, int t) {
     constexpr int QUADS = CP / 16;        // of channels per thread
     int in_row = __popc(small0) | __popc(small1) << 16;
     in_row += __shfl_xor_sync(FULL, in_row, 1);
@@ -607,6 +596,17 @@ __device__ __noinline__ bool channels_lost(const Walker walker, int nchunks, con
 // ... of sums below the row's limit: 0.3 % of the tiles of normally distributed data have one.
 template <int CP, typename Walker>
 __device__ __forceinline__ bool sums_lost(const float (&sum)[CP / 8][4], float limit0, float limit1, const Walker& walker, int nchunks, const float* rows, float tiny, int C, int t) {
+    float least0 = INFINITY, least1 = INFINITY;
+#pragma unroll
+    for (int m = 0; m < CP / 16; ++m)
+        if (Own<CP>::channel(t, 4 * m) < C) {
+#pragma unroll
+            for (int i = 2 * m; i < 2 * m + 2; ++i) {
+                asm("min.abs.f32 %0, %0, %1, %2;" : "+f"(least0) : "f"(sum[i][0]), "f"(sum[i][1]));
+                asm("min.abs.f32 %0, %0, %1, %2;" : "+f"(least1) : "f"(sum[i][2]), "f"(sum[i][3]));
+            }
+        }
+    if (!__any_sync(FULL, least0 < limit0 || least1 < limit1)) return false;
     uint32_t small0 = 0, small1 = 0;
 #pragma unroll
     for (int i = 0; i < CP / 4; ++i)
@@ -614,7 +614,7 @@ __device__ __forceinline__ bool sums_lost(const float (&sum)[CP / 8][4], float l
             if (fabsf(sum[i / 2][i % 2]) < limit0) small0 |= 1u << i;
             if (fabsf(sum[i / 2][2 + i % 2]) < limit1) small1 |= 1u << i;
         }
-    return __any_sync(FULL, (small0 | small1) != 0) && channels_lost<CP>(walker, nchunks, rows, tiny, small0, small1, C, t);
+    return channels_lost<CP>(walker, nchunks, rows, tiny, small0, small1, C, t);
 }
 __device__ __forceinline__ uint64_t lds64(uint32_t addr) {
     uint64_t x;
@@ -702,12 +702,6 @@ struct Exchange {
         for (int nt = 0; nt < CP / 8; ++nt)
 #pragma unroll
             for (int i = 0; i < 4; ++i) at(warp, first + 4 * nt + i) = x[nt][i] * (i < 2 ? f0 : f1);
-    }
-    __device__ __forceinline__ void get(float (&x)[CP / 8][4], int warp, int first) const {
-#pragma unroll
-        for (int nt = 0; nt < CP / 8; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) x[nt][i] = at(warp, first + 4 * nt + i);
     }
     // f0, f1 [warp]: factors of the warps' rows g and g + 8
     __device__ __forceinline__ void add(float (&x)[CP / 8][4], const Task& task, int first, const float (&f0)[WARPS], const float (&f1)[WARPS]) const {
@@ -837,14 +831,12 @@ __device__ __forceinline__ float group_sum(uint64_t x) {
     s += __shfl_xor_sync(FULL, s, 1);
     return s + __shfl_xor_sync(FULL, s, 2);
 }
-// A warp's pass in fp32; leaves the sums, the references and the rows' sums in the warp's staging memory (Exchange).
+// A warp's pass in fp32.
 template <int CP, typename Walker>
-__device__ __noinline__ void forward_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const BandView& view, bool seeded, const TilePoints at,
-                                          const float* q, const float* out, const float* lse, int C, float scale_log2) {
+__device__ __forceinline__ void forward_fp32(const Walker& walker, int nchunks, const BandView& view, bool seeded, const TilePoints& at, const float* q,
+                                             const float* out, const float* lse, Softmax& sm, float (&o)[CP / 8][4], int C, float scale_log2) {
     using S = Stage<CP>;
-    const int t = walker.lane & 3, warp = threadIdx.x >> 5;
-    float o[CP / 8][4];
-    Softmax sm;
+    const int t = walker.lane & 3;
     sm.start<CP>(seeded, view, at, out, lse, o, C, t);
     walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
         float s[2][4];
@@ -853,13 +845,6 @@ __device__ __noinline__ void forward_fp32(unsigned char* smem_raw, const Walker 
         sm.weights(s, o, both(scale_log2), bias2, mask);
         sums_fp32<CP>(o, s, st + S::B, t);
     });
-    const float ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
-    const Exchange<CP> x(smem_raw);
-    x.put(o, warp, 0, 1.f, 1.f);
-    const float rest[6] = {sm.m0, sm.m1, sm.top0, sm.top1, t == 0 ? ls0 : 0.f, t == 0 ? ls1 : 0.f};
-#pragma unroll
-    for (int i = 0; i < 6; ++i) x.at(warp, CP / 2 + i) = rest[i];
-    __syncwarp();
 }
 
 // Blocks of 4 warps per SM: as many as the registers of the kernel allow without spills that matter.  Measured at 128x256, N = 16,
@@ -898,60 +883,48 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
     Softmax sm;
     uint64_t bad;
     const bool plain = !scores_lost<LP>(Q.back0, C);      // k needs no scale of its own for scores of this size
-    for (bool first_pass = true;; first_pass = false) {
-        const bool seeded = view.dense_ptr != nullptr && (!task.shared || task.warp == 0);
+    const bool seeded = view.dense_ptr != nullptr && (!task.shared || task.warp == 0);
+    {
+        const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
+        if (seeded && view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
+        sm.template start<CP>(seeded, view, at, out, lse, o, C, t);
+    }
+    bad = 0;
+    walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
+        if (!sc.known()) {
+            const float before = sc.b.scale;
+            sc.look(st, plain, LP);
+            if (seeded) scale_rows(o, sc.b.scale / before, sc.b.scale / before);
+        }
+        float s[2][4];
+        SplitRows<CP, LP> V;
+        constexpr bool EARLY = CP < 64 && !LP;      // read v while the scores are computed, if there are registers for it
         {
-            const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-            if (seeded && view.has_dense(group * TILE_LAT, p.nlat_out)) wait_for_dense();
-            sm.template start<CP>(seeded, view, at, out, lse, o, C, t);
+            SplitRows<CP, LP> K;
+            K.template load<false>(st + sc.own + S::A, sc.a.scale);
+            if constexpr (EARLY) V.load(st + sc.own + S::B, sc.b.scale);
+            rows_dot_points<CP, LP>(s, Q, K);
         }
-        bad = 0;
-        scale_rows(o, sc.b.scale, sc.b.scale);
-        walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
-            if (!sc.known()) {
-                const float before = sc.b.scale;
-                sc.look(st, plain, LP);
-                if (seeded) scale_rows(o, sc.b.scale / before, sc.b.scale / before);
-            }
-            float s[2][4];
-            SplitRows<CP, LP> V;
-            constexpr bool EARLY = CP < 64 && !LP;      // read v while the scores are computed, if there are registers for it
-            {
-                SplitRows<CP, LP> K;
-                K.template load<false>(st + sc.own + S::A, sc.a.scale);
-                if constexpr (EARLY) V.load(st + sc.own + S::B, sc.b.scale);
-                rows_dot_points<CP, LP>(s, Q, K);
-            }
-            const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
-            note_overflow<LP>(bad, s);
-            sm.weights(s, o, both(Q.back0 * sc.a.inv), bias2, mask);
-            Weights<LP> W;
-            W.set(s);
-            if constexpr (!EARLY) V.load(st + sc.own + S::B, sc.b.scale);
-            weights_times_points<CP, LP>(o, W, V);
-        });
-        if (overflowed(sum2(add2(sm.l0, sm.l1)) + sum2(bad) + total(o))) {
-            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
-        } else {
-            // an output's floor is 2^-25 of its scaled v, which shows from 2^-8 on
-            constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;
-            const float ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
-            const bool lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) ||
-                              (sc.b.known && sums_lost<CP>(o, ls0 * LIMIT, ls1 * LIMIT, walker, nchunks, v + slice, LIMIT * sc.b.inv, C, t));
-            if (!lost) break;
-        }
-        {
-            const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-            forward_fp32<CP>(smem_raw, walker, nchunks, view, seeded, at, q, out, lse, C, scale_log2);
-        }
-        const Exchange<CP> x(smem_raw);
-        x.get(o, task.warp, 0);
-        sm.m0 = x.at(task.warp, CP / 2); sm.m1 = x.at(task.warp, CP / 2 + 1);
-        sm.top0 = x.at(task.warp, CP / 2 + 2); sm.top1 = x.at(task.warp, CP / 2 + 3);
-        sm.l0 = pack2(x.at(task.warp, CP / 2 + 4), 0.f); sm.l1 = pack2(x.at(task.warp, CP / 2 + 5), 0.f);
-        __syncwarp();
+        const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
+        note_overflow<LP>(bad, s);
+        sm.weights(s, o, both(Q.back0 * sc.a.inv), bias2, mask);
+        Weights<LP> W;
+        W.set(s);
+        if constexpr (!EARLY) V.load(st + sc.own + S::B, sc.b.scale);
+        weights_times_points<CP, LP>(o, W, V);
+    });
+    bool lost = overflowed(sum2(add2(sm.l0, sm.l1)) + sum2(bad) + total(o));
+    if (!lost) {
+        // an output's floor is 2^-25 of its scaled v, which shows from 2^-8 on
+        constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;
+        const float ls0 = group_sum(sm.l0), ls1 = group_sum(sm.l1);
+        lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) ||
+               (sc.b.known && sums_lost<CP>(o, ls0 * LIMIT, ls1 * LIMIT, walker, nchunks, v + slice, LIMIT * sc.b.inv, C, t));
+    }
+    if (lost) {
+        const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
+        forward_fp32<CP>(walker, nchunks, view, seeded, at, q, out, lse, sm, o, C, scale_log2);
         sc.b = StreamScale();
-        break;
     }
     const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
     // normalise, store
@@ -1003,13 +976,12 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
 // `out` and `dq` may be the same buffer: a warp reads its own 16 rows of `out` before it writes them as dq.
 // t, D and ds are in the units of the scaled dout row and the scaled v until the end.
 // ---------------------------------------------------------------------------------------------------------
-// A warp's pass in fp32; leaves the sums in its staging memory.
+// A warp's pass in fp32.
 template <int CP, typename Walker>
-__device__ __noinline__ void dq_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const TilePoints at, const float* q, const float* dout,
-                                     float lse0, float lse1, float D0, float D1, int C, float scale_log2) {
+__device__ __forceinline__ void dq_fp32(const Walker& walker, int nchunks, const TilePoints& at, const float* q, const float* dout,
+                                        float lse0, float lse1, float D0, float D1, float (&acc)[CP / 8][4], int C, float scale_log2) {
     using S = Stage<CP>;
     const int t = walker.lane & 3;
-    float acc[CP / 8][4];
     clear(acc);
     walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
         float s[2][4], tt[2][4];
@@ -1026,8 +998,6 @@ __device__ __noinline__ void dq_fp32(unsigned char* smem_raw, const Walker walke
         apply_mask(s, mask, 0.f);
         sums_fp32<CP>(acc, s, st + S::A, t);
     });
-    Exchange<CP>(smem_raw).put(acc, threadIdx.x >> 5, 0, 1.f, 1.f);
-    __syncwarp();
 }
 
 template <int CP, bool LP, bool PAD, bool CF>
@@ -1079,77 +1049,70 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
     float nD0, nD1;          // -D times the weight scale
     float max0, max1;        // largest |ds| of the thread's columns
     float f0, f1;            // dq per sum
-    for (bool first_pass = true;; first_pass = false) {
-        clear(acc);
-        ws = WeightScale();
-        uint64_t bad = 0;
-        nD0 = -D0 / Y.back0 * sc.b.scale; nD1 = -D1 / Y.back1 * sc.b.scale;
-        max0 = max1 = 0.f;
-        walker.template run<LP && CP == 32 ? 1 : 2>(nchunks, [&](uint32_t st, uint32_t mask, auto&& release) {
-            if (!sc.known()) {
-                const float before = sc.b.scale;
-                sc.look(st, LP, LP);
-                const float f = sc.b.scale / before;
-                nD0 *= f; nD1 *= f;
-                scale_rows(acc, f, f);
-            }
-            float s[2][4], tt[2][4];
-            SplitRows<CP, LP> K;
-            {
-                SplitRows<CP, LP> V;
-                V.load(st + sc.own + S::B, sc.b.scale);
-                rows_dot_points<CP, LP>(tt, Y, V);
-            }
-            K.load(st + sc.own + S::A, sc.a.scale);
-            const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
-            release();
-            rows_dot_points<CP, LP>(s, Q, K);
-            note_overflow<LP>(bad, s);
-            const uint64_t f2 = both(Q.back0 * sc.a.inv), h2 = both(ws.scale);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(both(lse0), both(-LOG2E), bias2[j])), s[j][0], s[j][1]);
-                unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(both(lse1), both(-LOG2E), bias2[j])), s[j][2], s[j][3]);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
-                unpack2(mul2(pack2(s[j][0], s[j][1]), fma2(pack2(tt[j][0], tt[j][1]), h2, both(nD0))), s[j][0], s[j][1]);       // ds
-                unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, both(nD1))), s[j][2], s[j][3]);
-            }
-            if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
-            row_max(max0, max1, s);
-            if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
-                const float f = ws.update(fmaxf(max0, max1));
-                scale_rows(acc, f, f);
-                scale_rows(s, f, f);
-                nD0 *= f; nD1 *= f;
-                max0 *= f; max1 *= f;
-            }
-            Weights<LP> W;
-            W.set(s);
-            weights_times_points<CP, LP>(acc, W, K);
-        });
-        f0 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back0; f1 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back1;
-        if (overflowed(total(acc) + sum2(bad))) {
-            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
-        } else {
-            // The floors: of ds, 2^-25; of t, below 2^-8 in units of ds's scale.  They are compared with the row's largest ds or, if
-            // t and D nearly cancel, with p D, whose rounding is an error of ds in any case (the row's p add up to 1).
-            const float r0 = group_max(max0), r1 = group_max(max1), least = (LP ? REDUCED : 1.f) * fmaxf(1.f / 128.f, 1024.f * ws.scale);
-            const float any = 1.f / (64.f * (float)nchunks);
-            const bool low = (r0 > 0.f && fmaxf(r0, any * fabsf(nD0)) < least) || (r1 > 0.f && fmaxf(r1, any * fabsf(nD1)) < least);
-            constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;         // of k, in a sum
-            const bool lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) || (sc.b.known && __any_sync(FULL, low)) ||
-                              (sc.a.known && sums_lost<CP>(acc, r0 * LIMIT, r1 * LIMIT, walker, nchunks, k + slice, LIMIT * sc.a.inv, C, t));
-            if (!lost) break;
+    clear(acc);
+    ws = WeightScale();
+    uint64_t bad = 0;
+    nD0 = -D0 / Y.back0 * sc.b.scale; nD1 = -D1 / Y.back1 * sc.b.scale;
+    max0 = max1 = 0.f;
+    walker.template run<LP && CP == 32 ? 1 : 2>(nchunks, [&](uint32_t st, uint32_t mask, auto&& release) {
+        if (!sc.known()) {
+            const float before = sc.b.scale;
+            sc.look(st, LP, LP);
+            const float f = sc.b.scale / before;
+            nD0 *= f; nD1 *= f;
+            scale_rows(acc, f, f);
         }
+        float s[2][4], tt[2][4];
+        SplitRows<CP, LP> K;
         {
-            const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
-            dq_fp32<CP>(smem_raw, walker, nchunks, at, q, dout, lse0, lse1, D0, D1, C, scale * LOG2E);
+            SplitRows<CP, LP> V;
+            V.load(st + sc.own + S::B, sc.b.scale);
+            rows_dot_points<CP, LP>(tt, Y, V);
         }
-        Exchange<CP>(smem_raw).get(acc, task.warp, 0);
-        __syncwarp();
+        K.load(st + sc.own + S::A, sc.a.scale);
+        const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
+        release();
+        rows_dot_points<CP, LP>(s, Q, K);
+        note_overflow<LP>(bad, s);
+        const uint64_t f2 = both(Q.back0 * sc.a.inv), h2 = both(ws.scale);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(both(lse0), both(-LOG2E), bias2[j])), s[j][0], s[j][1]);
+            unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(both(lse1), both(-LOG2E), bias2[j])), s[j][2], s[j][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
+            unpack2(mul2(pack2(s[j][0], s[j][1]), fma2(pack2(tt[j][0], tt[j][1]), h2, both(nD0))), s[j][0], s[j][1]);       // ds
+            unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, both(nD1))), s[j][2], s[j][3]);
+        }
+        if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
+        row_max(max0, max1, s);
+        if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
+            const float f = ws.update(fmaxf(max0, max1));
+            scale_rows(acc, f, f);
+            scale_rows(s, f, f);
+            nD0 *= f; nD1 *= f;
+            max0 *= f; max1 *= f;
+        }
+        Weights<LP> W;
+        W.set(s);
+        weights_times_points<CP, LP>(acc, W, K);
+    });
+    f0 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back0; f1 = scale * sc.a.inv / ws.scale * sc.b.inv * Y.back1;
+    bool lost = overflowed(total(acc) + sum2(bad));
+    if (!lost) {
+        // The floors: of ds, 2^-25; of t, below 2^-8 in units of ds's scale.  They are compared with the row's largest ds or, if
+        // t and D nearly cancel, with p D, whose rounding is an error of ds in any case (the row's p add up to 1).
+        const float r0 = group_max(max0), r1 = group_max(max1), least = (LP ? REDUCED : 1.f) * fmaxf(1.f / 128.f, 1024.f * ws.scale);
+        const float any = 1.f / (64.f * (float)nchunks);
+        const bool low = (r0 > 0.f && fmaxf(r0, any * fabsf(nD0)) < least) || (r1 > 0.f && fmaxf(r1, any * fabsf(nD1)) < least);
+        constexpr float LIMIT = (LP ? REDUCED : 1.f) / 256.f;         // of k, in a sum
+        lost = (sc.a.known && scores_lost<LP>(Q.back0 * sc.a.inv, C)) || (sc.b.known && __any_sync(FULL, low)) ||
+               (sc.a.known && sums_lost<CP>(acc, r0 * LIMIT, r1 * LIMIT, walker, nchunks, k + slice, LIMIT * sc.a.inv, C, t));
+    }
+    if (lost) {
+        const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
+        dq_fp32<CP>(walker, nchunks, at, q, dout, lse0, lse1, D0, D1, acc, C, scale * LOG2E);
         f0 = f1 = scale;
-        break;
     }
     const TilePoints at(n, group * TILE_LAT, w0 + g, p.nlat_out, p.nlon_out);
     if (task.shared) {
@@ -1185,13 +1148,13 @@ backward_dq_band_kernel(DevPlan p, const __grid_constant__ BandView view, const 
 //   dk_j = scale * sum_i p_ij (t_ij - D_i) q_i,   dv_j = sum_i p_ij dout_i          (App. B.4)
 // Tile rows are 8 input columns on each of the two rings of an input ring pair; stream columns are output points.
 // ---------------------------------------------------------------------------------------------------------
-// A warp's pass in fp32; leaves the sums in its staging memory.
+// A warp's pass in fp32.
 template <int CP, typename Walker>
-__device__ __noinline__ void dkdv_fp32(unsigned char* smem_raw, const Walker walker, int nchunks, const TilePoints at, const float* k, const float* v,
-                                       float bias0, float bias1, int C, float scale_log2) {
+__device__ __forceinline__ void dkdv_fp32(const Walker& walker, int nchunks, const TilePoints& at, const float* k, const float* v, const float* log2_omega,
+                                          float (&gk)[CP / 8][4], float (&gv)[CP / 8][4], int C, float scale_log2) {
     using S = Stage<CP>;
     const int t = walker.lane & 3;
-    float gk[CP / 8][4], gv[CP / 8][4];
+    const float bias0 = log2_omega[at.ha], bias1 = log2_omega[at.hb];
     clear(gk);
     clear(gv);
     walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
@@ -1214,10 +1177,6 @@ __device__ __noinline__ void dkdv_fp32(unsigned char* smem_raw, const Walker wal
         sums_fp32<CP>(gv, s, st + S::B, t);
         sums_fp32<CP>(gk, tt, st + S::A, t);
     });
-    const Exchange<CP> x(smem_raw);
-    x.put(gk, threadIdx.x >> 5, 0, 1.f, 1.f);
-    x.put(gv, threadIdx.x >> 5, CP / 2, 1.f, 1.f);
-    __syncwarp();
 }
 
 template <int CP, bool LP, bool PAD, bool CF>
@@ -1247,12 +1206,12 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
         srow = group * p.ps + r;
     }
     TileOperand<CP, LP> K, V;
-    float bias0, bias1;
+    float b0, b1;                 // log2 omega, later with the exponent of p's scale
     {
         const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
         K.template load<true>(k + at.pt0 * C, k + at.pt1 * C, scale * LOG2E, C, t);
         V.template load<true>(v + at.pt0 * C, v + at.pt1 * C, 1.f, C, t);
-        bias0 = p.log2_omega[at.ha]; bias1 = p.log2_omega[at.hb];
+        b0 = p.log2_omega[at.ha]; b1 = p.log2_omega[at.hb];
     }
     const size_t oslice = (size_t)n * p.nlat_out * p.nlon_out;
     int chunk0, nchunks;
@@ -1260,101 +1219,91 @@ backward_dkdv_band_kernel(DevPlan p, const __grid_constant__ BandView view, cons
     const auto walker = make_walker<CP, true, PAD>(smem_raw, view.s, chunk0, first, p.nlon_out, 1, C, q + oslice * C, dout + oslice * C, lse + oslice, Dws + oslice);
     float gk[NT][4], gv[NT][4];
     // The scale of p: over global attention, and for keys that little attention reaches, all of them are small.  It brings the largest
-    // of the first chunk that has some to [2^3, 2^4), so that a p 2^12 times as large still fits; if one does not, the pass is
-    // repeated with 2^15, which holds p = 1.
+    // of the first chunk that has some to [2^3, 2^4), so that a p 2^12 times as large still fits.
     float p_scale;
     WeightScale ws;          // of ds, beyond that
     float pmax0, pmax1, max0, max1;      // largest p and |ds| of the thread's columns
     float fk, fv;            // dk and dv per sum
-    for (bool first_pass = true;; first_pass = false) {
-        clear(gk);
-        clear(gv);
-        ws = WeightScale();
-        p_scale = first_pass ? 0.f : 32768.f;       // 0: not known
-        float b0 = first_pass ? bias0 : bias0 + 15.f, b1 = first_pass ? bias1 : bias1 + 15.f;           // with the exponent of p's scale
-        float unit = sc.b.scale / V.back0;      // t, D and ds are in the units of the scaled dout and v until the end
-        uint64_t bad = 0;
-        pmax0 = pmax1 = max0 = max1 = 0.f;
-        walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
-            if (!sc.known()) {
-                const float before = sc.b.scale;
-                sc.look(st, LP, LP);
-                unit *= sc.b.scale / before;
-                scale_rows(gk, sc.b.scale / before, sc.b.scale / before);
-            }
-            float s[2][4], tt[2][4];
-            SplitRows<CP, LP> Q, Y;
-            Q.load(st + sc.own + S::A, sc.a.scale);
-            rows_dot_points<CP, LP>(s, K, Q);
-            Y.load(st + sc.own + S::B, sc.b.scale);
-            rows_dot_points<CP, LP>(tt, V, Y);
-            const uint64_t lse2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)}, D2[2] = {lds64(st + S::M1 + 8 * t), lds64(st + S::M1 + 32 + 8 * t)};
-            note_overflow<LP>(bad, s);
-            const uint64_t f2 = both(K.back0 * sc.a.inv), h2 = both(ws.scale), nw2 = both(-ws.scale * unit), nlog2e2 = both(-LOG2E);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                // bias: log2 omega_j of the row's ring
-                unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(lse2[j], nlog2e2, both(b0))), s[j][0], s[j][1]);
-                unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(lse2[j], nlog2e2, both(b1))), s[j][2], s[j][3]);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
-            }
-            if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
-            row_max(pmax0, pmax1, s);
-            if (p_scale == 0.f) {
-                const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(fmaxf(pmax0, pmax1)));
-                if (w != 0) {
-                    p_scale = pow2_to(3, max(w & 0x7f800000u, (uint32_t)(127 - 72) << 23));
-                    const float e = (float)((int)(__float_as_uint(p_scale) >> 23) - 127);
-                    b0 += e; b1 += e;
-                    scale_rows(s, p_scale, p_scale);
-                    pmax0 *= p_scale; pmax1 *= p_scale;
-                }
-            }
-            Weights<LP> P, W;
-            P.set(s);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint64_t nD2 = mul2(D2[j], nw2);
-                unpack2(mul2(pack2(s[j][0], s[j][1]), fma2(pack2(tt[j][0], tt[j][1]), h2, nD2)), s[j][0], s[j][1]);      // ds
-                unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, nD2)), s[j][2], s[j][3]);
-            }
-            row_max(max0, max1, s);
-            if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
-                const float f = ws.update(fmaxf(max0, max1));
-                scale_rows(gk, f, f);
-                scale_rows(s, f, f);
-                max0 *= f; max1 *= f;
-            }
-            W.set(s);
-            weights_times_points<CP, LP>(gv, P, Y);
-            weights_times_points<CP, LP>(gk, W, Q);
-        });
-        // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry p's scale.
-        const float p_back = p_scale == 0.f ? 0.f : 1.f / p_scale;       // (0: no p at all)
-        fk = scale * sc.a.inv / ws.scale * sc.b.inv * p_back * V.back0; fv = sc.b.inv * p_back;
-        if (overflowed(total(gk) + total(gv) + sum2(bad))) {
-            if (first_pass && sc.look_at_all(walker, nchunks)) continue;
-        } else {
-            // The floors: of p and ds, 2^-25; of t, below 2^-8 in units of ds's scale and times p.
-            const float p0 = group_max(pmax0), p1 = group_max(pmax1), r0 = group_max(max0), r1 = group_max(max1);
-            constexpr float LEAST = (LP ? REDUCED : 1.f) / 128.f, LIMIT = (LP ? REDUCED : 1.f) / 256.f;      // (LIMIT: of q and dout, in a sum)
-            const float of_t = (LP ? REDUCED : 1.f) * 1024.f * ws.scale;
-            const bool low = (p0 > 0.f && p0 < LEAST) || (p1 > 0.f && p1 < LEAST) || (r0 > 0.f && r0 < fmaxf(LEAST, of_t * p0)) || (r1 > 0.f && r1 < fmaxf(LEAST, of_t * p1));
-            const bool lost = (sc.a.known && scores_lost<LP>(K.back0 * sc.a.inv, C)) || __any_sync(FULL, low) ||
-                              (sc.b.known && sums_lost<CP>(gv, p0 * LIMIT, p1 * LIMIT, walker, nchunks, dout + oslice * C, LIMIT * sc.b.inv, C, t)) ||
-                              (sc.a.known && sums_lost<CP>(gk, r0 * LIMIT, r1 * LIMIT, walker, nchunks, q + oslice * C, LIMIT * sc.a.inv, C, t));
-            if (!lost) break;
+    clear(gk);
+    clear(gv);
+    ws = WeightScale();
+    p_scale = 0.f;        // not known
+    float unit = sc.b.scale / V.back0;      // t, D and ds are in the units of the scaled dout and v until the end
+    uint64_t bad = 0;
+    pmax0 = pmax1 = max0 = max1 = 0.f;
+    walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
+        if (!sc.known()) {
+            const float before = sc.b.scale;
+            sc.look(st, LP, LP);
+            unit *= sc.b.scale / before;
+            scale_rows(gk, sc.b.scale / before, sc.b.scale / before);
         }
-        {
-            const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
-            dkdv_fp32<CP>(smem_raw, walker, nchunks, at, k, v, bias0, bias1, C, scale * LOG2E);
+        float s[2][4], tt[2][4];
+        SplitRows<CP, LP> Q, Y;
+        Q.load(st + sc.own + S::A, sc.a.scale);
+        rows_dot_points<CP, LP>(s, K, Q);
+        Y.load(st + sc.own + S::B, sc.b.scale);
+        rows_dot_points<CP, LP>(tt, V, Y);
+        const uint64_t lse2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)}, D2[2] = {lds64(st + S::M1 + 8 * t), lds64(st + S::M1 + 32 + 8 * t)};
+        note_overflow<LP>(bad, s);
+        const uint64_t f2 = both(K.back0 * sc.a.inv), h2 = both(ws.scale), nw2 = both(-ws.scale * unit), nlog2e2 = both(-LOG2E);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            // bias: log2 omega_j of the row's ring
+            unpack2(fma2(pack2(s[j][0], s[j][1]), f2, fma2(lse2[j], nlog2e2, both(b0))), s[j][0], s[j][1]);
+            unpack2(fma2(pack2(s[j][2], s[j][3]), f2, fma2(lse2[j], nlog2e2, both(b1))), s[j][2], s[j][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[j][i] = ex2(s[j][i]);
         }
-        Exchange<CP>(smem_raw).get(gk, task.warp, 0);
-        Exchange<CP>(smem_raw).get(gv, task.warp, CP / 2);
-        __syncwarp();
+        if (!(mask & BAND_ALL)) apply_mask(s, mask, 0.f);
+        row_max(pmax0, pmax1, s);
+        if (p_scale == 0.f) {
+            const uint32_t w = __reduce_max_sync(FULL, __float_as_uint(fmaxf(pmax0, pmax1)));
+            if (w != 0) {
+                p_scale = pow2_to(3, max(w & 0x7f800000u, (uint32_t)(127 - 72) << 23));
+                const float e = (float)((int)(__float_as_uint(p_scale) >> 23) - 127);
+                b0 += e; b1 += e;
+                scale_rows(s, p_scale, p_scale);
+                pmax0 *= p_scale; pmax1 *= p_scale;
+            }
+        }
+        Weights<LP> P, W;
+        P.set(s);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const uint64_t nD2 = mul2(D2[j], nw2);
+            unpack2(mul2(pack2(s[j][0], s[j][1]), fma2(pack2(tt[j][0], tt[j][1]), h2, nD2)), s[j][0], s[j][1]);      // ds
+            unpack2(mul2(pack2(s[j][2], s[j][3]), fma2(pack2(tt[j][2], tt[j][3]), h2, nD2)), s[j][2], s[j][3]);
+        }
+        row_max(max0, max1, s);
+        if (__any_sync(FULL, fmaxf(max0, max1) > ws.limit)) {
+            const float f = ws.update(fmaxf(max0, max1));
+            scale_rows(gk, f, f);
+            scale_rows(s, f, f);
+            max0 *= f; max1 *= f;
+        }
+        W.set(s);
+        weights_times_points<CP, LP>(gv, P, Y);
+        weights_times_points<CP, LP>(gk, W, Q);
+    });
+    // k was pre-multiplied by scale*log2e for the scores only; dk carries the plain scale.  Both sums carry p's scale.
+    const float p_back = p_scale == 0.f ? 0.f : 1.f / p_scale;       // (0: no p at all)
+    fk = scale * sc.a.inv / ws.scale * sc.b.inv * p_back * V.back0; fv = sc.b.inv * p_back;
+    bool lost = overflowed(total(gk) + total(gv) + sum2(bad));
+    if (!lost) {
+        // The floors: of p and ds, 2^-25; of t, below 2^-8 in units of ds's scale and times p.
+        const float p0 = group_max(pmax0), p1 = group_max(pmax1), r0 = group_max(max0), r1 = group_max(max1);
+        constexpr float LEAST = (LP ? REDUCED : 1.f) / 128.f, LIMIT = (LP ? REDUCED : 1.f) / 256.f;      // (LIMIT: of q and dout, in a sum)
+        const float of_t = (LP ? REDUCED : 1.f) * 1024.f * ws.scale;
+        const bool low = (p0 > 0.f && p0 < LEAST) || (p1 > 0.f && p1 < LEAST) || (r0 > 0.f && r0 < fmaxf(LEAST, of_t * p0)) || (r1 > 0.f && r1 < fmaxf(LEAST, of_t * p1));
+        lost = (sc.a.known && scores_lost<LP>(K.back0 * sc.a.inv, C)) || __any_sync(FULL, low) ||
+               (sc.b.known && sums_lost<CP>(gv, p0 * LIMIT, p1 * LIMIT, walker, nchunks, dout + oslice * C, LIMIT * sc.b.inv, C, t)) ||
+               (sc.a.known && sums_lost<CP>(gk, r0 * LIMIT, r1 * LIMIT, walker, nchunks, q + oslice * C, LIMIT * sc.a.inv, C, t));
+    }
+    if (lost) {
+        const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
+        dkdv_fp32<CP>(walker, nchunks, at, k, v, p.log2_omega, gk, gv, C, scale * LOG2E);
         fk = scale; fv = 1.f;
-        break;
     }
     const TilePoints at(n, group * TILE_LAT, col, p.nlat_in, p.nlon_in);
     if (task.shared) {

@@ -220,3 +220,17 @@ def test_what_is_not_finite_stays_with_the_points_that_attend_to_it(C, value):
             assert rel_points(got[..., ~touched, :], ref[..., ~touched, :]) <= 4 * TOL["fp32"], name
             if name != "k":     # (a key that is not finite may get a weight of zero)
                 assert not np.isfinite(got[..., touched, :]).any(), name
+
+
+@pytest.mark.parametrize("C, precision", [(16, "fp32"), (32, "fp32"), (64, "fp32"), (32, "tf32")])
+def test_channels_and_regions_of_zeros(C, precision):
+    """Zeros are not small values: a channel of v, the dout of a region, and all of v."""
+    wl = small_workload("zeros", *SHAPE, 0, 0, CUTOFF, 1, 2, C, 79)
+    q, k, v, dout = make_inputs(wl)
+    v[..., 3] = 0.0
+    dout[:, :, 6:, 10:20] = 0.0
+    for x in ((q, k, v, dout), (q, k, 0 * v, dout), (q, k, v, 0 * dout)):
+        got, refs = run(SHAPE, CUTOFF, *x, precision)
+        for name, a, r in zip(("out", "dq", "dk", "dv"), got, refs):
+            assert not a[r == 0].any() or name == "dq", name       # (dq of a point whose t is D: zero but for rounding)
+            assert np.linalg.norm(a - r) <= 2 * TOL[precision] * np.linalg.norm(r), name
