@@ -41,6 +41,15 @@ void check(int status) {
 float* data(const at::Tensor& t) { return t.data_ptr<float>(); }
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// Saved tensors come back through hooks (offloading, compression): the kernels read raw pointers, so anything but the tensor that was
+// saved, or its equal, is refused here.
+void check_saved(const at::Tensor& t, const char* name, at::IntArrayRef shape, const at::Tensor& dout) {
+    TORCH_CHECK_VALUE(t.defined() && t.scalar_type() == at::kFloat, name, " must be float32");
+    TORCH_CHECK_VALUE(t.sizes() == shape, name, " has shape ", t.sizes(), ", expected ", shape);
+    TORCH_CHECK_VALUE(t.is_contiguous(), name, " must be contiguous");
+    TORCH_CHECK_VALUE(t.is_cuda() && t.device() == dout.device(), name, " must be a CUDA tensor on the device of dout (", dout.device(), "), got ", t.device());
+}
+
 class Attention : public torch::autograd::Function<Attention> {
 public:
     static at::Tensor forward(AutogradContext* ctx, const c10::intrusive_ptr<Plan>& plan, at::Tensor q, at::Tensor k, at::Tensor v) {
@@ -56,7 +65,11 @@ public:
         const at::Tensor &q = saved[0], &k = saved[1], &v = saved[2], &out = saved[3], &lse = saved[4];
         const auto plan = c10::static_intrusive_pointer_cast<Plan>(ctx->saved_data["plan"].toCapsule());
         const at::Tensor dout = grads[0].contiguous().to(at::kFloat);
-        const int B = (int)q.size(0), H = (int)q.size(1), C = (int)q.size(4);
+        const at::IntArrayRef on = dout.sizes();
+        const int64_t in[5] = {on[0], on[1], plan->nlat_in, plan->nlon_in, on[4]};
+        check_saved(q, "q", on, dout); check_saved(k, "k", in, dout); check_saved(v, "v", in, dout);
+        check_saved(out, "out", on, dout); check_saved(lse, "lse", on.slice(0, 4), dout);
+        const int B = (int)on[0], H = (int)on[1], C = (int)on[4];
         at::Tensor dq = at::empty_like(q), dk = at::empty_like(k), dv = at::empty_like(k);
         sna_plan_t* handle = plan->handle;
         const size_t bytes = sna_workspace_bytes(handle, B, H, C);

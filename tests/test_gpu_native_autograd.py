@@ -78,3 +78,26 @@ def test_threads_share_a_plan_from_its_first_use():
         torch.cuda.synchronize()
     for r in results[1:]:
         assert all(torch.equal(a, b) for a, b in zip(r, results[0]))
+
+
+@pytest.mark.parametrize("saved", range(5), ids=["q", "k", "v", "out", "lse"])
+@pytest.mark.parametrize("change, says", [(lambda t: t.cpu(), "CUDA tensor"), (lambda t: t.half(), "float32"), (lambda t: t[..., :1], "has shape"),
+                                          (lambda t: t.transpose(2, 3).contiguous().transpose(2, 3), "contiguous"), (lambda t: t + 0, None)],
+                         ids=["host", "half", "shape", "strides", "copy"])
+def test_saved_tensors_that_hooks_return_are_checked(saved, change, says):
+    q, k, v = inputs()
+    seen = []
+
+    def unpack(t):
+        seen.append(t)
+        return change(t) if len(seen) == saved + 1 else t
+
+    with sna.Plan(12, 24, 12, 24, 0, 0, 0.6) as plan:
+        ref = torch.autograd.grad(attention(plan, q, k, v).sum(), (q, k, v))
+        with torch.autograd.graph.saved_tensors_hooks(lambda t: t, unpack):
+            total = attention(plan, q, k, v).sum()
+        if says:
+            with pytest.raises(ValueError, match=says):
+                torch.autograd.grad(total, (q, k, v))
+        else:
+            assert all(torch.equal(a, b) for a, b in zip(torch.autograd.grad(total, (q, k, v)), ref))
