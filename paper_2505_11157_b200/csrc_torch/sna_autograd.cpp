@@ -6,6 +6,7 @@
 #include <torch/extension.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 
 #include <atomic>
 
@@ -30,12 +31,15 @@ struct Plan : torch::CustomClassHolder {
     }
 };
 
-struct StatusError : std::runtime_error {
-    int status;
-    explicit StatusError(int s) : std::runtime_error(std::string(sna_status_string((sna_status_t)s)) + ": " + sna_last_error_message()), status(s) {}
-};
+// Raises sna.SnaError: as Python's own exception, the only kind that the autograd engine hands on as it is.
 void check(int status) {
-    if (status != SNA_OK) throw StatusError(status);
+    if (status == SNA_OK) return;
+    py::gil_scoped_acquire gil;
+    const py::object type = py::module_::import("paper_2505_11157_b200.sna").attr("SnaError");
+    PyErr_SetObject(type.ptr(), type(status).ptr());
+    python_error e;
+    e.persist();
+    throw e;
 }
 
 float* data(const at::Tensor& t) { return t.data_ptr<float>(); }
@@ -96,14 +100,6 @@ std::optional<at::Tensor> attention(const c10::intrusive_ptr<Plan>& plan, const 
 }  // namespace
 
 PYBIND11_MODULE(_sna_torch, m) {
-    py::register_exception_translator([](std::exception_ptr p) {
-        try {
-            if (p) std::rethrow_exception(p);
-        } catch (const StatusError& e) {
-            py::object type = py::module_::import("paper_2505_11157_b200.sna").attr("SnaError");
-            py::set_error(type, py::cast(e.status));
-        }
-    });
     py::class_<Plan, c10::intrusive_ptr<Plan>>(m, "Plan")
         .def(py::init([](uintptr_t h, int64_t a, int64_t b, int64_t c, int64_t d) { return c10::make_intrusive<Plan>(h, a, b, c, d); }))
         .def("close", &Plan::close);

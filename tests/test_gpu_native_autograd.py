@@ -101,3 +101,14 @@ def test_saved_tensors_that_hooks_return_are_checked(saved, change, says):
                 torch.autograd.grad(total, (q, k, v))
         else:
             assert all(torch.equal(a, b) for a, b in zip(torch.autograd.grad(total, (q, k, v)), ref))
+
+
+def test_a_failing_call_raises_the_same_error_in_forward_and_backward():
+    q, k, v = inputs()
+    plan = sna.Plan(12, 24, 12, 24, 0, 0, 0.6)
+    out = attention(plan, q, k, v)
+    plan.close()
+    for call in (lambda: torch.autograd.grad(out.sum(), q), lambda: attention(plan, q, k, v)):
+        with pytest.raises(sna.SnaError, match="plan is NULL") as e:
+            call()
+        assert e.value.status == sna.SNA_ERR_INVALID_ARG
