@@ -112,3 +112,22 @@ def test_a_failing_call_raises_the_same_error_in_forward_and_backward():
         with pytest.raises(sna.SnaError, match="plan is NULL") as e:
             call()
         assert e.value.status == sna.SNA_ERR_INVALID_ARG
+
+
+@pytest.mark.filterwarnings("ignore")
+def test_a_trace_and_a_tensor_subclass_run_the_operator():
+    class Sub(torch.Tensor):
+        pass
+
+    with sna.Plan(12, 24, 12, 24, 0, 0, 0.6) as plan:
+        q, k, v = inputs()
+        traced = torch.jit.trace(lambda a, b, c: 2 * attention(plan, a, b, c), (q, k, v), check_trace=False)
+        q, k, v = inputs()
+        ref = attention(plan, q, k, v)
+        again = traced(q, k, v)
+        assert torch.equal(again, 2 * ref)
+        for a, b in zip(torch.autograd.grad(again.sum(), (q, k, v)), torch.autograd.grad(2 * ref.sum(), (q, k, v))):
+            assert torch.equal(a, b)
+        with torch.no_grad():
+            out = attention(plan, q.as_subclass(Sub), k, v)
+        assert type(out) is Sub and torch.equal(out.as_subclass(torch.Tensor), ref)
