@@ -255,7 +255,8 @@ class Problem:
                             self.ws.numel(), wl.B, wl.H, wl.C, self.stream)
 
     def launches_per_step(self):
-        return self.sna.sna_forward_kernel_count(self.plan.handle, self.wl.C, True) + 2   # forward (dense + band, or one) + dq + dk/dv
+        shape = (self.plan.handle, self.wl.B, self.wl.H, self.wl.C)      # a pass is one kernel, or dense + band
+        return self.sna.sna_forward_kernel_count_for(*shape, True) + self.sna.sna_backward_kernel_count_for(*shape)
 
     def close(self):
         self.plan.close()

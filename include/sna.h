@@ -151,10 +151,13 @@ size_t sna_workspace_bytes(const sna_plan_t* plan, int B, int H, int C);
 sna_status_t sna_forward(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
                          int B, int H, int C, void* cuda_stream);
 
-/* Number of GPU kernels sna_forward_ex launches for this plan and channel count (with_lse != 0: an lse buffer is
- * passed).  1, or 2 when whole-ring and wide windows take the dense tensor-core kernel first, which they do if the problem
- * is large enough to fill the GPU with them.  0 for invalid arguments. */
+/* The largest number of GPU kernels sna_forward_ex launches for this plan and channel count (with_lse != 0: an lse buffer is
+ * passed): 1, or 2 if whole-ring and wide windows take the dense tensor-core kernel first when B * H is large enough to fill
+ * the GPU with them.  0 for invalid arguments. */
 int sna_forward_kernel_count(const sna_plan_t* plan, int C, int with_lse);
+/* The numbers of GPU kernels that sna_forward_ex and sna_backward_ex (with out and lse given) launch for this problem. */
+int sna_forward_kernel_count_for(const sna_plan_t* plan, int B, int H, int C, int with_lse);
+int sna_backward_kernel_count_for(const sna_plan_t* plan, int B, int H, int C);
 
 /* Forward pass that also stores lse[n,h,w] = log(sum_j exp(s_j) omega_j) (device, may be NULL), which the
  * backward pass can reuse. */

@@ -385,6 +385,25 @@ int sna_forward_kernel_count(const sna_plan_t* plan, int C, int with_lse) {
     return (with_lse && sna::dense2_path_chosen(plan->dev, C, 1 << 20)) ? 2 : 1;
 }
 
+// The passes that run on the dense and the band kernels, one after the other (where the dense ones do not run alone).
+static bool forward_on_both(const sna_plan_t* plan, int N, int C, bool with_lse) { return with_lse && sna::dense2_path_chosen(plan->dev, C, N); }
+// The dense backward kernels take the whole-ring and wide windows when they are at least a tenth of the work (measured on the
+// benchmark configurations: -8 % on the dq stage at a 22 % share, -6 % at 13 %).
+static bool dq_on_both(const sna_plan_t* plan, int N, int C) { return plan->dev.dense_fraction >= 0.10f && sna::dense2_path_chosen(plan->dev, C, N); }
+static bool dkdv_on_both(const sna_plan_t* plan, int N, int C) { return plan->dev.n_t_dense_rows > 0 && dq_on_both(plan, N, C); }
+
+int sna_forward_kernel_count_for(const sna_plan_t* plan, int B, int H, int C, int with_lse) {
+    if (check_problem(plan, B, H, C) != SNA_OK) return 0;
+    return !sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::FORWARD) && forward_on_both(plan, B * H, C, with_lse != 0) ? 2 : 1;
+}
+
+int sna_backward_kernel_count_for(const sna_plan_t* plan, int B, int H, int C) {
+    if (check_problem(plan, B, H, C) != SNA_OK) return 0;
+    const int N = B * H;
+    return (!sna::dense2_global_chosen(plan->dev, C, N, sna::Pass::DQ) && dq_on_both(plan, N, C) ? 2 : 1) +
+           (!sna::dense2_global_chosen(plan->dev, C, N, sna::Pass::DKDV) && dkdv_on_both(plan, N, C) ? 2 : 1);
+}
+
 // out_cf: if not null, the output is wanted there too, channels first (the band kernels write it themselves)
 static sna_status_t forward_into(const sna_plan_t* plan, const float* q, const float* k, const float* v, float* out,
                             float* lse, int B, int H, int C, void* cuda_stream, float* out_cf) {
@@ -397,7 +416,7 @@ static sna_status_t forward_into(const sna_plan_t* plan, const float* q, const f
         // every window is a whole ring (a global plan, or a cutoff that reaches every point): the dense kernel alone
         // produces the final out and, if asked for, lse (64x128, N = 4, without lse: 5.44 ms on the generic kernel, 0.25 ms here)
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (lse != nullptr && sna::dense2_path_chosen(plan->dev, C, B * H)) {
+    } else if (forward_on_both(plan, B * H, C, lse != nullptr)) {
         // whole-ring and wide windows on the tcgen05 kernel (its partial result travels in out / lse), the rest on the band kernel
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, true, false, (cudaStream_t)cuda_stream, out_cf);
@@ -433,11 +452,9 @@ static sna_status_t backward_dq_into(const sna_plan_t* plan, const float* q, con
     if (!q || !k || !v || !dout || !lse || !dq || !D) { set_error("q, k, v, dout, lse, dq and D must not be NULL"); return SNA_ERR_INVALID_ARG; }
     if (!all_aligned(q, k, v, dout, dq, out) || ((reinterpret_cast<uintptr_t>(lse) | reinterpret_cast<uintptr_t>(D)) & 3u)) { set_error("device pointers must be 16-byte aligned"); return SNA_ERR_INVALID_ARG; }
     cudaError_t e;
-    // The dense dq kernel takes the whole-ring and wide windows when they are at least a tenth of the work (measured on the
-    // benchmark configurations: -8 % on the dq stage at a 22 % share, -6 % at 13 %).
     if (out != nullptr && out != dq && sna::dense2_global_chosen(plan->dev, C, B * H, sna::Pass::DQ)) {
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (out != nullptr && out != dq && plan->dev.dense_fraction >= 0.10f && sna::dense2_path_chosen(plan->dev, C, B * H)) {
+    } else if (out != nullptr && out != dq && dq_on_both(plan, B * H, C)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dq is written first), the rest is added by the band kernel
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, nullptr, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, true, false, (cudaStream_t)cuda_stream, dq_cf);
@@ -478,7 +495,7 @@ static sna_status_t backward_dkdv_into(const sna_plan_t* plan, const float* q, c
             if (e != cudaSuccess) return cuda_fail(e, "clearing the gradients of input rings without windows");
         }
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
-    } else if (plan->dev.dense_fraction >= 0.10f && plan->dev.n_t_dense_rows > 0 && sna::dense2_path_chosen(plan->dev, C, B * H)) {
+    } else if (dkdv_on_both(plan, B * H, C)) {
         // whole-ring and wide windows on the tcgen05 kernel (its part of dk, dv is written first), the band kernel adds the rest
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, true, false, (cudaStream_t)cuda_stream, dk_cf, dv_cf);

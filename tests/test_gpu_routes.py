@@ -52,3 +52,35 @@ def test_input_rings_that_no_window_reaches_get_zero_gradients(slices):
     """Output rings at the two poles only: every window is a whole ring, and ten of the sixteen input rings are in none."""
     wl = small_workload("poles", 16, 128, 2, 128, 0, 0, 0.5, 1, slices, 32, 82)
     check(wl, TOL_DENSE)
+
+
+def launches(call):
+    """Kernel nodes of a captured call."""
+    from cuda.bindings import runtime
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = runtime.cudaGraph_t(graph.raw_cuda_graph())
+    _, _, count = runtime.cudaGraphGetNodes(raw)
+    _, nodes, _ = runtime.cudaGraphGetNodes(raw, count)
+    kernel = runtime.cudaGraphNodeType.cudaGraphNodeTypeKernel
+    return sum(runtime.cudaGraphNodeGetType(n)[1] == kernel for n in nodes[:count])
+
+
+@pytest.mark.parametrize("slices", [1, 24])
+@pytest.mark.parametrize("C", [16, 32])
+@pytest.mark.parametrize("args", [dict(theta_cutoff=0.25), dict(global_attention=True)], ids=["band", "global"])
+def test_kernel_counts(args, C, slices):
+    """What the queries say for a problem is what its calls launch; for a plan and a width, what the largest problem would."""
+    with sna.Plan(40, 160, 40, 160, 0, 0, **args) as plan:
+        q, k, v, dout = (torch.randn(1, slices, 40, 160, C, device="cuda") for _ in range(4))
+        out, lse = plan.forward(q, k, v, return_lse=True)
+        ws = torch.empty(plan.workspace_bytes(1, slices, C), dtype=torch.uint8, device="cuda")
+        grads = [torch.empty_like(t) for t in (q, k, v)]
+        counts = [sna.sna_forward_kernel_count_for(plan.handle, 1, slices, C, lse_wanted) for lse_wanted in (False, True)]
+        assert counts[0] == launches(lambda: plan.forward(q, k, v, out=out))
+        assert counts[1] == launches(lambda: plan.forward(q, k, v, out=out, lse=lse))
+        assert sna.sna_backward_kernel_count_for(plan.handle, 1, slices, C) == launches(
+            lambda: plan.backward(q, k, v, dout, out=out, lse=lse, dq=grads[0], dk=grads[1], dv=grads[2], workspace=ws))
+        limit = [sna.sna_forward_kernel_count(plan.handle, C, lse_wanted) for lse_wanted in (False, True)]
+        assert counts[1] <= limit[1] and (slices == 1 or counts == limit)
