@@ -236,6 +236,9 @@ static sna_status_t plan_create(int nlat_in, int nlon_in, int nlat_out, int nlon
     d.dense_longest = dense.longest;
     d.dense_fraction = hp.nnz > 0 ? (float)((double)dense.pairs / (double)hp.nnz) : 0.f;
     d.dense_all = dense.pairs == hp.nnz ? 1 : 0;
+    d.pairs = hp.nnz * hp.nlon_out;
+    d.longest_row = *std::max_element(hp.row_nnz.begin(), hp.row_nnz.end());
+    d.longest_t_row = *std::max_element(hp.t_row_nnz.begin(), hp.t_row_nnz.end()) / hp.ps;
     d.is_global = global ? 1 : 0;
     d.t_consecutive = t_consecutive ? 1 : 0;
     sna::DevBand* dev_bands[4] = {&d.fwd, &d.fwdb, &d.t, &d.tb};
@@ -421,7 +424,7 @@ static sna_status_t forward_into(const sna_plan_t* plan, const float* q, const f
         e = sna::launch_forward_dense2(plan->dev, q, k, v, out, lse, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, true, false, (cudaStream_t)cuda_stream, out_cf);
         out_cf = nullptr;
-    } else if (sna::band_path_supported(plan->dev, C)) {
+    } else if (sna::band_path_supported(plan->dev, C) && !sna::generic_chosen(plan->dev, C, B * H, sna::Pass::FORWARD)) {
         e = sna::launch_forward_band(plan->dev, q, k, v, out, lse, B * H, C, false, false, (cudaStream_t)cuda_stream, out_cf);
         out_cf = nullptr;
     } else {
@@ -459,7 +462,7 @@ static sna_status_t backward_dq_into(const sna_plan_t* plan, const float* q, con
         e = sna::launch_backward_dq_dense2(plan->dev, q, k, v, dout, out, lse, dq, nullptr, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, true, false, (cudaStream_t)cuda_stream, dq_cf);
         dq_cf = nullptr;
-    } else if (out != nullptr && sna::band_path_supported(plan->dev, C)) {
+    } else if (out != nullptr && sna::band_path_supported(plan->dev, C) && (out == dq || !sna::generic_chosen(plan->dev, C, B * H, sna::Pass::DQ))) {
         e = sna::launch_backward_dq_band(plan->dev, q, k, v, dout, out, lse, dq, D, B * H, C, false, false, (cudaStream_t)cuda_stream, dq_cf);
         dq_cf = nullptr;
     } else {
@@ -500,7 +503,7 @@ static sna_status_t backward_dkdv_into(const sna_plan_t* plan, const float* q, c
         e = sna::launch_backward_dkdv_dense2(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, (cudaStream_t)cuda_stream);
         if (e == cudaSuccess) e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, true, false, (cudaStream_t)cuda_stream, dk_cf, dv_cf);
         dk_cf = nullptr;
-    } else if (sna::band_path_supported(plan->dev, C)) {
+    } else if (sna::band_path_supported(plan->dev, C) && !sna::generic_chosen(plan->dev, C, B * H, sna::Pass::DKDV)) {
         e = sna::launch_backward_dkdv_band(plan->dev, q, k, v, dout, lse, D, dk, dv, B * H, C, false, false, (cudaStream_t)cuda_stream, dk_cf, dv_cf);
         dk_cf = nullptr;
     } else {

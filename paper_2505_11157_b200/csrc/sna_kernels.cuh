@@ -50,6 +50,7 @@ struct DevPlan {
     long long dense_blocks, dense_longest;      // 128-column blocks that the tiles of one longitude range walk: all of them, the longest
     float dense_fraction;           // share of the table's entries that the dense kernels' windows cover
     int dense_all;                  // 1: they cover every one (a share that rounds to 1 may still leave narrow windows out)
+    long long pairs, longest_row, longest_t_row;      // table entries of a slice; of the output point and of the input point with most
     int* dev_status;                // set to non-zero by a kernel whose bounded wait ran out
     int t_consecutive;              // 1: transposed tiles are 8 consecutive input columns; 0: split by residue mod ps
     int is_global;                  // 1: every window is a whole ring; the band streams have one row
@@ -97,6 +98,7 @@ cudaError_t launch_cf_to_cl(const float* src, float* dst, int slices, int C, lon
 cudaError_t launch_cl_to_cf(const float* src, float* dst, int slices, int C, long long P, cudaStream_t stream);
 
 // Generic kernels (any supported C): C/4 lanes cooperate on one grid point.
+bool generic_chosen(const DevPlan& p, int C, int N, Pass pass);      // they are faster than the band kernels
 // forward: out and/or lse may be null (lse-only pass = softmax statistics).
 cudaError_t launch_forward_generic(const DevPlan& p, const float* q, const float* k, const float* v, float* out,
                                    float* lse, int N, int C, cudaStream_t stream);

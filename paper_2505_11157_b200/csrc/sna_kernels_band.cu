@@ -1386,7 +1386,9 @@ bool make_view(const DevPlan& p, bool transposed, bool band, int N, int blocks_p
     v.N = N;
     const long long per_group = (long long)v.tiles * N, total = per_group * v.s.groups;
     if (total > 0x7fffffffLL) return false;
-    // Share the streams that alone would take long in comparison with the whole launch.
+    // Share the streams that alone would take long in comparison with the whole launch.  They are counted from the front of the order.
+    // (Behind a dense kernel the groups that wait for it come later and are not shared: where those kernels are used, a launch has
+    // at most two that exceed the limit, by less than a tenth.)
     const double fair = (double)v.s.chunks * (transposed && !p.t_consecutive ? v.tiles / p.ps : v.tiles) * N / ((double)p.num_sms * blocks_per_sm * WARPS);
     const double above = v.s.one_row ? SHARE_EQUAL_ABOVE : SHARE_ABOVE;
     const double longest = fair * above > SHARE_MIN ? fair * above : SHARE_MIN;

@@ -4,7 +4,9 @@
 // online in registers.
 // Forward: Eq. (s2_attention_discrete_detailed); backward: App. B.4.
 #include "sna_kernels.cuh"
+#include "sna_plan.hpp"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace sna {
@@ -231,6 +233,25 @@ cudaError_t dispatch_lp(int C, F&& f) {
 }
 
 }  // namespace
+
+// One or two lanes per point (C <= 8) do a pair's work in a quarter or half of the 16 channels that the band kernels pad to, so in
+// large launches, where the longest row no longer matters, they are faster - the more the emptier the band kernels' tiles are.  Both
+// times are estimated (ns): pairs per block of THREADS lanes (the last one of a ring may be partly empty), at least the longest
+// row's; chunks.  Measured generic : band (us, forward / dq / dkdv) at C = 4: 128x256, cutoff 0.04, N = 64 190/155/230 : 361/451/484,
+// N = 4 71/55/159 : 39/39/42, cutoff 0.1, N = 16 209/186/412 : 227/248/307; 361x720, cutoff 0.03, N = 16 1362/1132/1740 :
+// 1584/1804/2202; 48x96 from 96x192, N = 64 323/277/243 : 189/203/281.  C = 8, 128x256, cutoff 0.04, N = 64 372/339/581 : 365/459/486.
+bool generic_chosen(const DevPlan& p, int C, int N, Pass pass) {
+    if (C > 8) return false;
+    const bool gather = pass == Pass::DKDV;
+    const int lanes = C / 4, ring = gather ? p.nlon_in : p.nlon_out, per_block = THREADS / lanes, tiles = (ring + per_block - 1) / per_block;
+    const double pair = (pass == Pass::FORWARD ? 2.1e-3 : pass == Pass::DQ ? 1.9e-3 : 2.9e-3) * lanes * tiles * per_block / ring;
+    const double step = pass == Pass::FORWARD ? 170 : pass == Pass::DQ ? 110 : 310;
+    const double chunk = pass == Pass::FORWARD ? 0.36 : pass == Pass::DQ ? 0.42 : 0.55;
+    const double generic = std::max(pair * (double)p.pairs * N, step * (double)(gather ? p.longest_t_row : p.longest_row)) + 15e3;
+    const DevBand& band = gather ? p.t : p.fwd;
+    const int band_tiles = gather && p.t_consecutive ? (p.nlon_in + TILE_LON - 1) / TILE_LON : (p.nlon_out + TILE_LON - 1) / TILE_LON;
+    return generic < chunk * (double)band.chunks * band_tiles * N + 25e3;
+}
 
 cudaError_t launch_forward_generic(const DevPlan& p, const float* q, const float* k, const float* v, float* out,
                                    float* lse, int N, int C, cudaStream_t stream) {

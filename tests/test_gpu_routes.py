@@ -84,3 +84,20 @@ def test_kernel_counts(args, C, slices):
             lambda: plan.backward(q, k, v, dout, out=out, lse=lse, dq=grads[0], dk=grads[1], dv=grads[2], workspace=ws))
         limit = [sna.sna_forward_kernel_count(plan.handle, C, lse_wanted) for lse_wanted in (False, True)]
         assert counts[1] <= limit[1] and (slices == 1 or counts == limit)
+
+
+@pytest.mark.parametrize("slices", [1, 300])
+@pytest.mark.parametrize("C", [4, 8])
+@pytest.mark.parametrize("shape", [(9, 256, 9, 256), (12, 512, 6, 256)], ids=["same_grid", "down2"])
+def test_narrow_heads_in_small_and_large_launches(shape, C, slices):
+    """C = 4 and 8: band kernels for few slices; for many, passes on the generic kernels where those are faster."""
+    wl = small_workload("narrow", *shape, 0, 0, 0.45, 1, 1, C, 83)
+    one = make_inputs(wl)
+    g = orc.geometry(*shape, 0, 0, 0.45)
+    refs = [orc.forward(g, *one[:3]), *orc.backward(g, *one)]
+    dev = [torch.from_numpy(a).cuda().expand(1, slices, -1, -1, -1).contiguous() for a in one]
+    with sna.Plan(*shape, 0, 0, 0.45) as plan:
+        out, lse = plan.forward(*dev[:3], return_lse=True)
+        for state in ({"out": out, "lse": lse}, {}):
+            for x, r in zip((out, *plan.backward(*dev, **state)), refs):
+                assert rel(x[:, -1:], r) <= 5e-6 and torch.equal(x[:, 0], x[:, -1])
