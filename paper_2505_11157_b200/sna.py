@@ -283,6 +283,13 @@ class Plan:
         except Exception:
             pass
 
+    # A copy of a module that holds a plan (an averaged model, say) shares it: there is one handle, and nothing in it changes.
+    def __copy__(self):
+        return self
+
+    def __deepcopy__(self, memo):
+        return self
+
     def __enter__(self):
         return self
 

@@ -1,4 +1,5 @@
 """The native autograd function: who owns the plan, and what it says about arguments that the plan does not take."""
+import copy
 import gc
 import threading
 
@@ -131,3 +132,13 @@ def test_a_trace_and_a_tensor_subclass_run_the_operator():
         with torch.no_grad():
             out = attention(plan, q.as_subclass(Sub), k, v)
         assert type(out) is Sub and torch.equal(out.as_subclass(torch.Tensor), ref)
+
+
+def test_copies_share_the_plan():
+    q, k, v = inputs()
+    plan = sna.Plan(12, 24, 12, 24, 0, 0, 0.6)
+    ref = attention(plan, q, k, v)
+    copies = [copy.copy(plan), copy.deepcopy({"plan": plan})["plan"]]
+    del plan
+    gc.collect()
+    assert all(torch.equal(attention(p, q, k, v), ref) for p in copies)

@@ -164,7 +164,7 @@ def test_unequal_magnitudes(which, C, precision, slices):
     wl = small_workload("spread", *SHAPE, 0, 0, CUTOFF, 1, 1, C, 77)
     q, k, v, dout = spread(which, *make_inputs(wl))
     yards = yardsticks(q, k, v, dout)
-    same = [np.ascontiguousarray(np.broadcast_to(a, (1, slices, *a.shape[2:]))) for a in (q, k, v, dout)]
+    same = [np.array(np.broadcast_to(a, (1, slices, *a.shape[2:])), order="C") for a in (q, k, v, dout)]
     g = orc.geometry(*SHAPE, 0, 0, CUTOFF)
     refs = [orc.forward(g, q, k, v), *orc.backward(g, q, k, v, dout)]
     dev = [torch.from_numpy(a).cuda() for a in same]
