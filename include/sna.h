@@ -29,7 +29,11 @@
  *     calls that run concurrently do not share a workspace (see sna_backward).
  *   - Accuracy: results are fp32; against an fp64 evaluation of the same formulas the normalised maximum
  *     error max|x - ref| / max|ref| per tensor is below 1e-5 for out and below 1e-4 for dq, dk, dv
- *     (measured 2e-6 and 2e-5).  No atomics are used: the same call on the same inputs gives the same bits.
+ *     (measured 2e-6 and 2e-5).  Inputs may be of very unequal magnitudes: an element of a result carries an error of about
+ *     2^-17 of the sum of the magnitudes of its own terms at most, however large other points or channels are, except that
+ *     terms whose softmax weight is below 2^-15 of the largest in their row are held to 2^-35 of that weight.  A point that is
+ *     not finite reaches the results that depend on it; with C = 32 it may also reach those of points that share a tile of the
+ *     dense kernels.  No atomics are used: the same call on the same inputs gives the same bits.
  */
 #ifndef SNA_H
 #define SNA_H
@@ -231,8 +235,9 @@ sna_status_t sna_backward_cf(const sna_plan_t* plan, const float* dout_cf, const
 /*
  * Reduced-precision variant of the forward and backward pass.  The paper lists "neither reduced precision nor tensor
  * core" support as a limitation of its kernels (Sec. 5, Limitations); here every contraction of
- * Eq. s2_attention_discrete_detailed and App. B.4 is taken as ONE tensor-core product (operands rounded to the 11
- * significand bits of TF32, fp32 accumulation, fp32 softmax) instead of the error-compensated products of the default path.
+ * Eq. s2_attention_discrete_detailed and App. B.4 is taken as ONE FP16 tensor-core product (operands scaled by powers of two and
+ * rounded to 11 significand bits, as TF32 has; fp32 accumulation, fp32 softmax) instead of the error-compensated products of the
+ * default path.  Parts of a problem that FP16's range does not hold are computed in fp32.
  * Same arguments, layouts and semantics as sna_forward_ex / sna_backward_ex.  Accuracy: normalised maximum error
  * max|x - ref| / max|ref| per tensor below 5e-3 against an fp64 evaluation (measured ~1e-3); about 1.2x faster.
  * Needs C in {16, 32, 64} and nlon_out >= 32 (SNA_ERR_UNSUPPORTED otherwise).
