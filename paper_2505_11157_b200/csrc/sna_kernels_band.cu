@@ -11,12 +11,12 @@
 // registers, where they are the B operands of the scores and, transposed by movmatrix, of the weighted sums.  Warps do not
 // synchronise with each other, except at the end of a stream that is long for its launch: the warps of a block share it.
 //
-// What bounds them (128x256, cutoff 4 rings, C = 32): per chunk of 16 columns a forward warp issues 357 instructions and moves 110
+// What bounds them (128x256, cutoff 4 rings, C = 32): per chunk of 16 columns a forward warp issues 362 instructions and moves 110
 // wavefronts through the SM's shared-memory pipe (cp.async writes 44, row reads 38, transpositions 16, the rest global), so with
-// 16 warps per SM that pipe is busy 69 % of the time, issue slots 58 %, tensor cores 30 %; DRAM and L2 are below 20 %.  Measures
+// 16 warps per SM that pipe is busy 68 % of the time, issue slots 58 %, tensor cores 30 %; DRAM and L2 are below 20 %.  Measures
 // that took instructions or wavefronts out (us forward / dq / dk+dv, N = 16, whole streams): scales from the first chunk instead of
 // a maximum per chunk 368/459/559 -> 359/414/481; x - h by one mixed-precision multiply-add, and no scaling of data that needs
-// none -> 348/397/466; movmatrix instead of writing the split rows back for ldmatrix -> 327/388/455 and, with pieces in an order
+// none (given up again for the range that it costs, see StreamScale) -> 348/397/466; movmatrix instead of writing the split rows back for ldmatrix -> 327/388/455 and, with pieces in an order
 // without bank conflicts, C = 64, N = 8 from 432/472/549 to 334/369/445.
 //
 // Fragment conventions (g = lane / 4, t = lane % 4): a thread holds CP/4 channels of a point (Own::channel).  As an A operand
@@ -71,8 +71,8 @@ __device__ __forceinline__ float pow2_back(int target, uint32_t ebits) { return 
 
 // Scale of a warp's streamed rows of one array: taken from the first chunk that is not all zero, whose largest element it brings to
 // [2^11, 2^12).  A split element is then held to 2^-23 of itself or to 2^-25 in scaled units (the floor), which is 2^-36 of that
-// largest one, and FP16 holds elements 16 times as large.  (Where that much is not needed, `plain`, as in reduced precision, the scale
-// stays 1 and the scaling is skipped if the largest element is in [2^-1, 2^8).)  Two things can go wrong.  Larger rows overflow to
+// largest one, and FP16 holds elements 16 times as large.  (Where that much is not needed, `plain` - for scores, in the backward pass in
+// reduced precision - the scale stays 1 and the scaling is skipped if the largest element is in [2^-1, 2^8).)  Two things can go wrong.  Larger rows overflow to
 // infinities, which the sums cannot hide.  And sums of which all terms are far below the largest element (a small channel beside a
 // large one, small points beside a large one that is in the window of another row of the tile) may feel the floor: each kernel
 // compares its sums with it at the end.  Where they overflowed, or one is so small that the floor could be 2^-17 of it and such
@@ -893,7 +893,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
     walker.template run<1>(nchunks, [&](uint32_t st, uint32_t mask, auto&&) {
         if (!sc.known()) {
             const float before = sc.b.scale;
-            sc.look(st, plain, LP);
+            sc.look(st, plain, false);
             if (seeded) scale_rows(o, sc.b.scale / before, sc.b.scale / before);
         }
         float s[2][4];
@@ -902,7 +902,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
         {
             SplitRows<CP, LP> K;
             K.template load<false>(st + sc.own + S::A, sc.a.scale);
-            if constexpr (EARLY) V.load(st + sc.own + S::B, sc.b.scale);
+            if constexpr (EARLY) V.template load<true>(st + sc.own + S::B, sc.b.scale);
             rows_dot_points<CP, LP>(s, Q, K);
         }
         const uint64_t bias2[2] = {lds64(st + S::M0 + 8 * t), lds64(st + S::M0 + 32 + 8 * t)};
@@ -910,7 +910,7 @@ forward_band_kernel(DevPlan p, const __grid_constant__ BandView view, const floa
         sm.weights(s, o, both(Q.back0 * sc.a.inv), bias2, mask);
         Weights<LP> W;
         W.set(s);
-        if constexpr (!EARLY) V.load(st + sc.own + S::B, sc.b.scale);
+        if constexpr (!EARLY) V.template load<true>(st + sc.own + S::B, sc.b.scale);
         weights_times_points<CP, LP>(o, W, V);
     });
     bool lost = overflowed(sum2(add2(sm.l0, sm.l1)) + sum2(bad) + total(o));
