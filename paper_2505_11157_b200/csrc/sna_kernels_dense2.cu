@@ -52,6 +52,7 @@ constexpr int M2 = 128;          // tile rows
 constexpr int BN2 = 128;         // columns per block
 constexpr int C2 = 32;           // channels
 constexpr int THREADS2 = 640;        // five warpgroups: softmax (two column halves) | TMA, S issuer | four P V issuers | converters
+constexpr int THREADS_DKDV = 768;    // six: element-wise (two column halves) | TMA, first GEMMs, statistics | four issuers | converters of q, of dout
 constexpr int WAIT2 = 1 << 17;     // polls of one wait (each may suspend for up to ~2 us) before the thread gives up
 constexpr float LOG2E_2 = 1.4426950408889634f;
 constexpr float LN2_2 = 0.6931471805599453f;
@@ -83,6 +84,15 @@ enum { B_KFULL = 0, B_KCONV = 2, B_KFREE = 4, B_VFULL = 6, B_VRAWFREE = 8, B_VCO
 // Lets a band kernel that was launched to follow this one (its programmatic dependent) take the SMs that the last blocks leave idle.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// One lane of a whole warp, for the MMAs that one thread issues.  (With lane 0 picked by comparison the compiler does not know that
+// one lane is left, and each tcgen05.mma takes 55 cycles to issue and the first eight of a batch 580, against 16 and 85.  It pays where
+// many short MMAs are issued: a first-GEMM issuer of the dk/dv kernel was busy 1250 of 1880 cycles per block, now 490 of 1690.  In the
+// forward kernel, whose 128-column MMAs keep the tensor core busy for 66 cycles each, it changes nothing: 499 : 502 us on 64x128, N = 8.)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ float ex2f(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float trunc19f(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
@@ -891,7 +901,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 tma_tile(sbase + s * QST + 2 * TILE_Q, &map_v, c0, n * p.nlat_in + hp, s32(&bars[Q_VFULL + s]));
             }
         }
-        if ((warp == 9 || warp == 10) && lane == 0) {
+        if ((warp == 9 || warp == 10) && elect_one()) {
             // -------------------------------------------------------------- S = Q K^T (warp 9) and T = dY V^T (warp 10)
             const bool isT = warp == 10;
             ok = mb_wait(s32(&bars[Q_AREADY]), 0, ok);
@@ -920,7 +930,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
         // ------------------------------------------------------------------ dq_part = dS K over two 8-column steps
-        if (lane == 0) {
+        if (elect_one()) {
             const int part = warp - 12, grp = part >> 1;
             const uint32_t idO = idesc_tf32(C2);
             const uint32_t tO = tm + TQ_ACC + part * 32;
@@ -994,7 +1004,9 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
 //   S^T = K Q^T, T^T = V dY^T (one issuing thread each);  p = exp2(s + log2 omega_j - lse_i),  ds = p (t - D_i);
 //   dV += P dY,  dK += scale * dS Q   (A operands P, dS from TMEM; B operands: q and dout blocks transposed by the converters).
 // Two groups of 128 threads do the element-wise work for one half of the block's columns each and write P over S^T, dS
-// over T^T and the two lo parts beside them; four threads issue the second GEMMs (dV or dK, one column half each) into
+// over T^T and the two lo parts beside them; one warp fetches the partner points' statistics, two groups of converters prepare the q and
+// the dout blocks (with one group for both, and that latency in it, the converters were busy 1600 of the 1880 cycles that a block took;
+// 64x128 global, N = 8: 1010 -> 883 us, 128x256, cutoff 4 rings, N = 16, with the band kernel: 476 -> 457); four threads issue the second GEMMs (dV or dK, one column half each) into
 // their own accumulators, which collect FOLDK blocks in TMEM before the row's threads fold them into registers.  TMEM:
 // 128 columns of fixed operands, two buffers of 128 (S^T, T^T, P_lo, dS_lo of 32 columns each) and 128 of accumulators.
 // With two buffers the first GEMMs of block j+1 run while the element-wise threads work on block j and the second
@@ -1013,7 +1025,7 @@ constexpr int TK_S = 0, TK_T = 32, TK_PLO = 64, TK_DSLO = 96;      // offsets in
 enum { K_QFULL = 0, K_YFULL = NSK, K_QCONV = 2 * NSK, K_YCONV = 3 * NSK, K_FREE = 4 * NSK /* all [stage] */, K_STFULL = 5 * NSK /* [buffer] */,
        K_READY = 5 * NSK + 2 /* [group][buffer] */, K_G2DONE = 5 * NSK + 6 /* [group][buffer] */, K_AREADY = 5 * NSK + 10, K_COUNT = 5 * NSK + 11 };
 
-__global__ void __launch_bounds__(THREADS2, 1)
+__global__ void __launch_bounds__(THREADS_DKDV, 1)
 backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_y,
                             const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ lse,
                             const float* __restrict__ Dws, float* __restrict__ dk, float* __restrict__ dv, int N, float scale,
@@ -1045,7 +1057,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
         for (int s = 0; s < NSK; ++s) {
             mb_init(s32(&bars[K_QFULL + s]), 1);
             mb_init(s32(&bars[K_YFULL + s]), 1);
-            mb_init(s32(&bars[K_QCONV + s]), 128);
+            mb_init(s32(&bars[K_QCONV + s]), 128 + 32);      // converters, statistics
             mb_init(s32(&bars[K_YCONV + s]), 128);
             mb_init(s32(&bars[K_FREE + s]), 6);         // both first GEMMs and the four second-GEMM issuers
         }
@@ -1074,9 +1086,9 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
     PROF_DECL
 
     if (warp < 8) {
-        // register budget of the block: 640 threads x 96 at launch; a warpgroup can only grow by what the others give back:
-        // 256 x 160 + 256 x 40 + 128 x 72 = 60416 <= 61440
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 160;");
+        // register budget of the block: 768 threads x 80 at launch; a warpgroup can only grow by what the others give back:
+        // 256 x 152 + 256 x 32 + 256 x 56 = 61440
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
         // ------------------------------------------------------------------ element-wise: thread (grp, r) owns tile row r (an
         // input point) for the partner columns [16 grp, 16 grp + 16) of every block
         const int grp = warp >> 2, r = tid & 127;
@@ -1219,7 +1231,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             }
         }
     } else if (warp < 12) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         if (warp == 8 && lane == 0) {
             // -------------------------------------------------------------- TMA producer: q and dout blocks of the partner rings
             TileWalk wk(p.t_dense_lat, p.t_dense_m, e_begin, e_end, p.nlon_out, BNK, a_lo, a_hi, p.ps);
@@ -1234,7 +1246,20 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 tma_tile(sbase + s * KST + 2 * TILE_K, &map_y, w0, n * p.nlat_out + h, s32(&bars[K_YFULL + s]));
             }
         }
-        if ((warp == 9 || warp == 10) && lane == 0) {
+        if (warp == 11) {
+            // -------------------------------------------------------------- the partner points' statistics, up to NSK blocks ahead
+            TileWalk wk(p.t_dense_lat, p.t_dense_m, e_begin, e_end, p.nlon_out, BNK, a_lo, a_hi, p.ps);
+            for (int it = 0; it < total && ok; ++it, wk.advance()) {
+                const int s = it % NSK, u = it / NSK;
+                if (u > 0) ok = mb_wait(s32(&bars[K_FREE + s]), (u - 1) & 1, ok);
+                const size_t o = (size_t)(n * p.nlat_out + wk.ring) * p.nlon_out + min(wk.col() + lane, p.nlon_out - 1);
+                float* nlc = reinterpret_cast<float*>(base + s * KST + 8 * TILE_K);
+                nlc[lane] = fmaf(-__ldg(lse + o), LOG2E_2, p.log2_omega[hp]);   // log2 omega_j - lse_i in the log2 domain
+                nlc[BNK + lane] = __ldg(Dws + o);
+                mb_arrive(s32(&bars[K_QCONV + s]));
+            }
+        }
+        if ((warp == 9 || warp == 10) && elect_one()) {
             // -------------------------------------------------------------- S^T = K Q^T (warp 9) and T^T = V dY^T (warp 10)
             const bool isT = warp == 10;
             ok = mb_wait(s32(&bars[K_AREADY]), 0, ok);
@@ -1261,9 +1286,9 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             }
         }
     } else if (warp < 16) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         // ------------------------------------------------------------------ second GEMMs: part = (kind, column half)
-        if (lane == 0) {
+        if (elect_one()) {
             const int part = warp - 12, kind = part >> 1, grp = part & 1;      // kind 0: dV = P dY, kind 1: dK = dS Q
             const uint32_t idO = idesc_tf32(C2);
             const uint32_t tO = tm + TK_ACC + part * 32;
@@ -1288,12 +1313,18 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             }
         }
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-        // ------------------------------------------------------------------ converters (warps 16-19, 128 threads)
-        const int ct = tid - 512, cw = ct >> 5;
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        // ------------------------------------------------------------------ converters: warps 16-19 of the q blocks, 20-23 of the dout blocks
+        const bool isY = warp >= 20;
+        const int ct = tid & 127, cw = ct >> 5;
+        const uint32_t full = s32(&bars[isY ? K_YFULL : K_QFULL]), conv = s32(&bars[isY ? K_YCONV : K_QCONV]);
         // lo tile (same swizzled positions) and transposed hi / lo tiles of one raw tile (one K block of 32 points: row =
         // channel, 128 bytes of points): warp cw takes the 8 columns [8 cw, 8 cw + 8), lane = channel
-        auto convert = [&](unsigned char* raw, unsigned char* lo, unsigned char* th) {
+        for (int it = 0; it < total && ok; ++it) {
+            const int s = it % NSK, u = it / NSK;
+            unsigned char* raw = base + s * KST + (isY ? 2 * TILE_K : 0);
+            unsigned char *lo = raw + TILE_K, *th = base + s * KST + (isY ? 6 : 4) * TILE_K;
+            PROF_WAIT(0, ok = mb_wait(full + 8 * s, u & 1, ok));
 #pragma unroll
             for (int j = 0; j < BNK * 4 / 128; ++j) stack_b16(raw, lo, (j * 128 + ct) >> 2, ct & 3);
 #pragma unroll
@@ -1306,27 +1337,8 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 *reinterpret_cast<float4*>(th + sw_off(lane, chunk)) = make_float4(hi[0], hi[1], hi[2], hi[3]);
                 *reinterpret_cast<float4*>(th + TILE_K + sw_off(lane, chunk)) = make_float4(lw[0], lw[1], lw[2], lw[3]);
             }
-        };
-        TileWalk wk(p.t_dense_lat, p.t_dense_m, e_begin, e_end, p.nlon_out, BNK, a_lo, a_hi, p.ps);
-        for (int it = 0; it < total && ok; ++it, wk.advance()) {
-            const int s = it % NSK, u = it / NSK;
-            unsigned char* st = base + s * KST;
-            const int h = wk.ring;
-            const int w0 = wk.col();
-            PROF_WAIT(0, ok = mb_wait(s32(&bars[K_QFULL + s]), u & 1, ok));       // also: the stage (and its statistics arrays) is free
-            if (ct < BNK) {
-                const size_t o = (size_t)(n * p.nlat_out + h) * p.nlon_out + min(w0 + ct, p.nlon_out - 1);
-                float* nlc = reinterpret_cast<float*>(st + 8 * TILE_K);
-                nlc[ct] = fmaf(-__ldg(lse + o), LOG2E_2, p.log2_omega[hp]);   // log2 omega_j - lse_i in the log2 domain
-                nlc[BNK + ct] = __ldg(Dws + o);
-            }
-            convert(st, st + TILE_K, st + 4 * TILE_K);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mb_arrive(s32(&bars[K_QCONV + s]));
-            PROF_WAIT(1, ok = mb_wait(s32(&bars[K_YFULL + s]), u & 1, ok) && ok);
-            convert(st + 2 * TILE_K, st + 3 * TILE_K, st + 6 * TILE_K);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mb_arrive(s32(&bars[K_YCONV + s]));
+            mb_arrive(conv + 8 * s);
         }
     }
     if (!ok) atomicExch(&fail_s, 1);
@@ -1458,7 +1470,7 @@ cudaError_t launch_backward_dkdv_dense2(const DevPlan& p, const float* q, const 
     cudaError_t e = make_map2(&mq, q, N * p.nlat_out, p.nlon_out, BNK);
     if (e == cudaSuccess) e = make_map2(&my, dout, N * p.nlat_out, p.nlon_out, BNK);
     if (e != cudaSuccess) return e;
-    backward_dkdv_dense2_kernel<<<(unsigned)blocks, THREADS2, DKDV2_SMEM, stream>>>(p, mq, my, k, v, lse, Dws, dk, dv, N, 1.0f / sqrtf((float)C), tiles_per_row);
+    backward_dkdv_dense2_kernel<<<(unsigned)blocks, THREADS_DKDV, DKDV2_SMEM, stream>>>(p, mq, my, k, v, lse, Dws, dk, dv, N, 1.0f / sqrtf((float)C), tiles_per_row);
     return cudaGetLastError();
 }
 
