@@ -354,164 +354,167 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
         float corr_prev = 1.f;
         const int ctr = p.ps * w;                          // this row's window centre, in input columns
         TileWalk wk(p.dense_lat, p.dense_m, e_begin, e_end, p.nlon_in, BN2, a_lo, a_hi, 1);
-        for (int it = 0; it <= total && ok; ++it) {
-            float corr = 1.f;
-            if (it > 0) {
-                // fold P V of the previous block (this half's two partial results, fixed order); waiting for it here also
-                // frees this half's P_lo columns and accumulators
-                const int bp = (it - 1) & 1, up = (it - 1) >> 1;
-                ok = mb_wait(s32(&bars[B_PVDONE + 2 * half + bp]), up & 1, ok) && ok;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                uint32_t oa[32], ob[32];
-                tm_ld32_issue(oa, tm + T_O + half * 64 + lanebits);
-                tm_ld32_issue(ob, tm + T_O + half * 64 + 32 + lanebits);
+        // folds P V of a block (this half's two partial results, fixed order); waiting for it also frees this half's P_lo columns and
+        // accumulators
+        auto fold = [&](int it) {
+            ok = mb_wait(s32(&bars[B_PVDONE + 2 * half + (it & 1)]), (it >> 1) & 1, ok) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int c0 = 0; c0 < C2; c0 += 16) {
+                uint32_t oa[16], ob[16];
+                tm_ld16_issue(oa, tm + T_O + half * 64 + lanebits + c0);
+                tm_ld16_issue(ob, tm + T_O + half * 64 + 32 + lanebits + c0);
                 tm_ld_wait();
 #pragma unroll
-                for (int j = 0; j < C2; j += 2)
-                    unpack2(fma2(pack2(o[j], o[j + 1]), pack2(corr_prev, corr_prev),
+                for (int j = 0; j < 16; j += 2)
+                    unpack2(fma2(pack2(o[c0 + j], o[c0 + j + 1]), pack2(corr_prev, corr_prev),
                                  add2(pack2(__uint_as_float(oa[j]), __uint_as_float(oa[j + 1])), pack2(__uint_as_float(ob[j]), __uint_as_float(ob[j + 1])))),
-                            o[j], o[j + 1]);
+                            o[c0 + j], o[c0 + j + 1]);
             }
-            if (it < total) {
-                const int b = it & 1, u = it >> 1;
-                const float bias = p.log2_omega[wk.ring];
-                // the columns [jl, jh] of this thread's half that exist and lie in this row's window
-                int jl = max(0, ctr - wk.m - wk.u) - half * HC, jh = min(wk.seg_end - wk.u, ctr + wk.m - wk.u) - half * HC;
-                if (!row_ok || jh < jl || jh < 0 || jl >= HC) { jl = HC; jh = HC; }     // none
-                const uint32_t span = (uint32_t)(jh - jl);
-                const bool full = __all_sync(0xffffffffu, jl <= 0 && jh >= HC - 1);     // no masking anywhere in this warp
-                wk.advance();
-                ok = mb_wait(s32(&bars[B_SFULL + b]), u & 1, ok) && ok;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tS = tm + (b ? T_S1 : T_S0) + half * HC + lanebits;
-                uint64_t ps2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};      // four running sums of P, as two packed pairs
-                if constexpr (SPLIT) {
-                    // all-whole plans: the thread's 64 scores are loaded from TMEM once and stay in registers for both passes
-                    // pass 1: maximum of the raw scores (the scale is positive and the bias is the same for the whole block)
-                    uint32_t sq[4][16];
-    #pragma unroll
-                    for (int qd = 0; qd < 4; ++qd) tm_ld16_issue(sq[qd], tS + 16 * qd);
-                    tm_ld_wait();
-                    float mxr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    if (full) {
-    #pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            mxr[j & 3] = fmaxf(mxr[j & 3], fmaxf(fmaxf(__uint_as_float(sq[0][j]), __uint_as_float(sq[1][j])),
-                                                                 fmaxf(__uint_as_float(sq[2][j]), __uint_as_float(sq[3][j]))));
-                    } else {
-    #pragma unroll
-                        for (int qd = 0; qd < 4; ++qd)
-    #pragma unroll
-                            for (int j = 0; j < 16; ++j)
-                                if ((uint32_t)(16 * qd + j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sq[qd][j]));
-                    }
-                    // (a half without any valid column keeps its state: exp2(-inf) = 0 below, and m stays -inf only if nothing was ever seen)
-                    const float mblk = fmaf(fmaxf(fmaxf(mxr[0], mxr[1]), fmaxf(mxr[2], mxr[3])), scale_log2, bias);
-                    const float mx = fmaxf(m, mblk);
-                    const float msafe = mx == -INFINITY ? 0.f : mx;
-                    corr = ex2f(m - msafe);
-                    m = mx;
-                    const float nb = bias - msafe;
-                    // pass 2: P over S (its top 19 bits are the hi part) and P_lo = P - trunc19(P) beside it
-                    auto pass2 = [&](auto unmasked) {
-                        constexpr bool UNMASKED = decltype(unmasked)::value;
-                        const uint64_t scale2 = pack2(scale_log2, scale_log2), nb2 = pack2(nb, nb);
-    #pragma unroll
-                        for (int qd = 0; qd < 4; ++qd) {
-                            uint32_t (&x)[16] = sq[qd];
-                            const int c0 = 16 * qd;
-                            uint32_t lo[16];
-    #pragma unroll
-                            for (int j = 0; j < 16; j += 2) {
-                                float x0, x1, l0, l1;
-                                unpack2(fma2(pack2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])), scale2, nb2), x0, x1);
-                                float p0 = ex2f(x0), p1 = ex2f(x1);
-                                if (!UNMASKED && !full && (uint32_t)(c0 + j - jl) > span) p0 = 0.f;
-                                if (!UNMASKED && !full && (uint32_t)(c0 + j + 1 - jl) > span) p1 = 0.f;
-                                const uint64_t p2 = pack2(p0, p1);
-                                ps2[(j >> 1) & 1] = add2(ps2[(j >> 1) & 1], p2);
-                                unpack2(sub2(p2, pack2(trunc19f(p0), trunc19f(p1))), l0, l1);
-                                x[j] = __float_as_uint(p0); x[j + 1] = __float_as_uint(p1);
-                                lo[j] = __float_as_uint(l0); lo[j + 1] = __float_as_uint(l1);
-                            }
-                            tm_st16(tS + c0, x);
-                            tm_st16(tm + T_PLO + half * HC + lanebits + c0, lo);
-                        }
-                    };
-                    if (SPLIT && full) pass2(std::true_type{}); else pass2(std::false_type{});
+        };
+        for (int it = 0; it < total && ok; ++it) {
+            float corr = 1.f;
+            const int b = it & 1, u = it >> 1;
+            const float bias = p.log2_omega[wk.ring];
+            // the columns [jl, jh] of this thread's half that exist and lie in this row's window
+            int jl = max(0, ctr - wk.m - wk.u) - half * HC, jh = min(wk.seg_end - wk.u, ctr + wk.m - wk.u) - half * HC;
+            if (!row_ok || jh < jl || jh < 0 || jl >= HC) { jl = HC; jh = HC; }     // none
+            const uint32_t span = (uint32_t)(jh - jl);
+            const bool full = __all_sync(0xffffffffu, jl <= 0 && jh >= HC - 1);     // no masking anywhere in this warp
+            wk.advance();
+            ok = mb_wait(s32(&bars[B_SFULL + b]), u & 1, ok) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t tS = tm + (b ? T_S1 : T_S0) + half * HC + lanebits;
+            uint64_t ps2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};      // four running sums of P, as two packed pairs
+            if constexpr (SPLIT) {
+                // all-whole plans: the thread's 64 scores are loaded from TMEM once and stay in registers for both passes
+                // pass 1: maximum of the raw scores (the scale is positive and the bias is the same for the whole block)
+                uint32_t sq[4][16];
+#pragma unroll
+                for (int qd = 0; qd < 4; ++qd) tm_ld16_issue(sq[qd], tS + 16 * qd);
+                tm_ld_wait();
+                float mxr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                if (full) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        mxr[j & 3] = fmaxf(mxr[j & 3], fmaxf(fmaxf(__uint_as_float(sq[0][j]), __uint_as_float(sq[1][j])),
+                                                             fmaxf(__uint_as_float(sq[2][j]), __uint_as_float(sq[3][j]))));
                 } else {
-                    // plans with masked blocks: two loads per score (fewer live registers; measured 0.4 % faster there)
-                    // pass 1: maximum of the raw scores (the scale is positive and the bias is the same for the whole block)
-                    float mxr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    {
-                        uint32_t sa[32], sb[32];
-                        tm_ld32_issue(sa, tS);
-                        tm_ld32_issue(sb, tS + 32);
-                        tm_ld_wait();
-                        if (full) {
-    #pragma unroll
-                            for (int j = 0; j < 32; ++j) mxr[j & 3] = fmaxf(mxr[j & 3], fmaxf(__uint_as_float(sa[j]), __uint_as_float(sb[j])));
-                        } else {
-    #pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                if ((uint32_t)(j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sa[j]));
-                                if ((uint32_t)(32 + j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sb[j]));
-                            }
+#pragma unroll
+                    for (int qd = 0; qd < 4; ++qd)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if ((uint32_t)(16 * qd + j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sq[qd][j]));
+                }
+                // (a half without any valid column keeps its state: exp2(-inf) = 0 below, and m stays -inf only if nothing was ever seen)
+                const float mblk = fmaf(fmaxf(fmaxf(mxr[0], mxr[1]), fmaxf(mxr[2], mxr[3])), scale_log2, bias);
+                if (it > 0) fold(it - 1);      // (not before the maximum: P V runs while it is found; 64x128, N = 8: 502 -> 457 us)
+                const float mx = fmaxf(m, mblk);
+                const float msafe = mx == -INFINITY ? 0.f : mx;
+                corr = ex2f(m - msafe);
+                m = mx;
+                const float nb = bias - msafe;
+                // pass 2: P over S (its top 19 bits are the hi part) and P_lo = P - trunc19(P) beside it
+                auto pass2 = [&](auto unmasked) {
+                    constexpr bool UNMASKED = decltype(unmasked)::value;
+                    const uint64_t scale2 = pack2(scale_log2, scale_log2), nb2 = pack2(nb, nb);
+#pragma unroll
+                    for (int qd = 0; qd < 4; ++qd) {
+                        uint32_t (&x)[16] = sq[qd];
+                        const int c0 = 16 * qd;
+                        uint32_t lo[16];
+#pragma unroll
+                        for (int j = 0; j < 16; j += 2) {
+                            float x0, x1, l0, l1;
+                            unpack2(fma2(pack2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])), scale2, nb2), x0, x1);
+                            float p0 = ex2f(x0), p1 = ex2f(x1);
+                            if (!UNMASKED && !full && (uint32_t)(c0 + j - jl) > span) p0 = 0.f;
+                            if (!UNMASKED && !full && (uint32_t)(c0 + j + 1 - jl) > span) p1 = 0.f;
+                            const uint64_t p2 = pack2(p0, p1);
+                            ps2[(j >> 1) & 1] = add2(ps2[(j >> 1) & 1], p2);
+                            unpack2(sub2(p2, pack2(trunc19f(p0), trunc19f(p1))), l0, l1);
+                            x[j] = __float_as_uint(p0); x[j + 1] = __float_as_uint(p1);
+                            lo[j] = __float_as_uint(l0); lo[j + 1] = __float_as_uint(l1);
+                        }
+                        tm_st16(tS + c0, x);
+                        tm_st16(tm + T_PLO + half * HC + lanebits + c0, lo);
+                    }
+                };
+                if (SPLIT && full) pass2(std::true_type{}); else pass2(std::false_type{});
+            } else {
+                // plans with masked blocks: two loads per score (fewer live registers; measured 0.4 % faster there)
+                // pass 1: maximum of the raw scores (the scale is positive and the bias is the same for the whole block)
+                float mxr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                {
+                    uint32_t sa[32], sb[32];
+                    tm_ld32_issue(sa, tS);
+                    tm_ld32_issue(sb, tS + 32);
+                    tm_ld_wait();
+                    if (full) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) mxr[j & 3] = fmaxf(mxr[j & 3], fmaxf(__uint_as_float(sa[j]), __uint_as_float(sb[j])));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            if ((uint32_t)(j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sa[j]));
+                            if ((uint32_t)(32 + j - jl) <= span) mxr[j & 3] = fmaxf(mxr[j & 3], __uint_as_float(sb[j]));
                         }
                     }
-                    // (a half without any valid column keeps its state: exp2(-inf) = 0 below, and m stays -inf only if nothing was ever seen)
-                    const float mblk = fmaf(fmaxf(fmaxf(mxr[0], mxr[1]), fmaxf(mxr[2], mxr[3])), scale_log2, bias);
-                    const float mx = fmaxf(m, mblk);
-                    const float msafe = mx == -INFINITY ? 0.f : mx;
-                    corr = ex2f(m - msafe);
-                    m = mx;
-                    const float nb = bias - msafe;
-                    // pass 2: P over S (its top 19 bits are the hi part) and P_lo = P - trunc19(P) beside it
-                    auto pass2 = [&](auto unmasked) {
-                        constexpr bool UNMASKED = decltype(unmasked)::value;
-                        uint32_t bufa[16], bufb[16];
-                        auto softmax16 = [&](uint32_t (&x)[16], int c0) {
-                            uint32_t lo[16];
-                            const uint64_t scale2 = pack2(scale_log2, scale_log2), nb2 = pack2(nb, nb);
-    #pragma unroll
-                            for (int j = 0; j < 16; j += 2) {
-                                float x0, x1, l0, l1;
-                                unpack2(fma2(pack2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])), scale2, nb2), x0, x1);
-                                float p0 = ex2f(x0), p1 = ex2f(x1);
-                                if (!UNMASKED && !full && (uint32_t)(c0 + j - jl) > span) p0 = 0.f;
-                                if (!UNMASKED && !full && (uint32_t)(c0 + j + 1 - jl) > span) p1 = 0.f;
-                                const uint64_t p2 = pack2(p0, p1);
-                                ps2[(j >> 1) & 1] = add2(ps2[(j >> 1) & 1], p2);
-                                unpack2(sub2(p2, pack2(trunc19f(p0), trunc19f(p1))), l0, l1);
-                                x[j] = __float_as_uint(p0); x[j + 1] = __float_as_uint(p1);
-                                lo[j] = __float_as_uint(l0); lo[j + 1] = __float_as_uint(l1);
-                            }
-                            tm_st16(tS + c0, x);
-                            tm_st16(tm + T_PLO + half * HC + lanebits + c0, lo);
-                        };
-                        tm_ld16_issue(bufa, tS);
-    #pragma unroll
-                        for (int c0 = 0; c0 < HC; c0 += 32) {
-                            tm_ld_wait();
-                            tm_ld16_issue(bufb, tS + c0 + 16);            // in flight while the first 16 columns are processed
-                            softmax16(bufa, c0);
-                            tm_ld_wait();
-                            if (c0 + 32 < HC) tm_ld16_issue(bufa, tS + c0 + 32);
-                            softmax16(bufb, c0 + 16);
-                        }
-                    };
-                    if (SPLIT && full) pass2(std::true_type{}); else pass2(std::false_type{});
                 }
-                float ps[4];
-                unpack2(ps2[0], ps[0], ps[1]);
-                unpack2(ps2[1], ps[2], ps[3]);
-                l = fmaf(l, corr, (ps[0] + ps[1]) + (ps[2] + ps[3]));
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mb_arrive(s32(&bars[B_PREADY + 2 * half + b]));
+                // (a half without any valid column keeps its state: exp2(-inf) = 0 below, and m stays -inf only if nothing was ever seen)
+                const float mblk = fmaf(fmaxf(fmaxf(mxr[0], mxr[1]), fmaxf(mxr[2], mxr[3])), scale_log2, bias);
+                if (it > 0) fold(it - 1);
+                const float mx = fmaxf(m, mblk);
+                const float msafe = mx == -INFINITY ? 0.f : mx;
+                corr = ex2f(m - msafe);
+                m = mx;
+                const float nb = bias - msafe;
+                // pass 2: P over S (its top 19 bits are the hi part) and P_lo = P - trunc19(P) beside it
+                auto pass2 = [&](auto unmasked) {
+                    constexpr bool UNMASKED = decltype(unmasked)::value;
+                    uint32_t bufa[16], bufb[16];
+                    auto softmax16 = [&](uint32_t (&x)[16], int c0) {
+                        uint32_t lo[16];
+                        const uint64_t scale2 = pack2(scale_log2, scale_log2), nb2 = pack2(nb, nb);
+#pragma unroll
+                        for (int j = 0; j < 16; j += 2) {
+                            float x0, x1, l0, l1;
+                            unpack2(fma2(pack2(__uint_as_float(x[j]), __uint_as_float(x[j + 1])), scale2, nb2), x0, x1);
+                            float p0 = ex2f(x0), p1 = ex2f(x1);
+                            if (!UNMASKED && !full && (uint32_t)(c0 + j - jl) > span) p0 = 0.f;
+                            if (!UNMASKED && !full && (uint32_t)(c0 + j + 1 - jl) > span) p1 = 0.f;
+                            const uint64_t p2 = pack2(p0, p1);
+                            ps2[(j >> 1) & 1] = add2(ps2[(j >> 1) & 1], p2);
+                            unpack2(sub2(p2, pack2(trunc19f(p0), trunc19f(p1))), l0, l1);
+                            x[j] = __float_as_uint(p0); x[j + 1] = __float_as_uint(p1);
+                            lo[j] = __float_as_uint(l0); lo[j + 1] = __float_as_uint(l1);
+                        }
+                        tm_st16(tS + c0, x);
+                        tm_st16(tm + T_PLO + half * HC + lanebits + c0, lo);
+                    };
+                    tm_ld16_issue(bufa, tS);
+#pragma unroll
+                    for (int c0 = 0; c0 < HC; c0 += 32) {
+                        tm_ld_wait();
+                        tm_ld16_issue(bufb, tS + c0 + 16);            // in flight while the first 16 columns are processed
+                        softmax16(bufa, c0);
+                        tm_ld_wait();
+                        if (c0 + 32 < HC) tm_ld16_issue(bufa, tS + c0 + 32);
+                        softmax16(bufb, c0 + 16);
+                    }
+                };
+                if (SPLIT && full) pass2(std::true_type{}); else pass2(std::false_type{});
             }
+            float ps[4];
+            unpack2(ps2[0], ps[0], ps[1]);
+            unpack2(ps2[1], ps[2], ps[3]);
+            l = fmaf(l, corr, (ps[0] + ps[1]) + (ps[2] + ps[3]));
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mb_arrive(s32(&bars[B_PREADY + 2 * half + b]));
             corr_prev = corr;
         }
+        if (total > 0) fold(total - 1);
         // merge the two column halves of every row: half 1 hands its state over through shared memory
         float* xs = reinterpret_cast<float*>(base + OFF_K);         // [34][128] floats in the k stages, which are dead by now
         if (half == 1) {
