@@ -817,31 +817,34 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 PROF_WAIT(0, ok = mb_wait(s32(&bars[Q_STFULL + b]), u & 1, ok) && ok);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tS = tm + TQ_BUF + 128 * b + grp * GC + lanebits, tT = tS + BNQ;
-                uint32_t sv[32], tv[32];
-                tm_ld32_issue(sv, tS);
-                tm_ld32_issue(tv, tT);
+                uint32_t sv[2][16], tv[2][16];      // two pieces: the first is stored while the second is worked on (64x128, N = 8: 518 -> 500 us)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) { tm_ld16_issue(sv[i], tS + 16 * i); tm_ld16_issue(tv[i], tT + 16 * i); }
                 tm_ld_wait();
                 // (two instantiations: blocks in which no row of the warp is masked skip the per-element range test)
                 auto elementwise = [&](auto unmasked) {
                     constexpr bool UNMASKED = decltype(unmasked)::value;
                     const uint64_t scale2 = pack2(scale_log2, scale_log2), nbias2 = pack2(nbias, nbias), D2 = pack2(D, D);
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        float x0, x1, ds0, ds1, l0, l1;
-                        unpack2(fma2(pack2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), scale2, nbias2), x0, x1);
-                        float p0 = ex2f(x0), p1 = ex2f(x1);
-                        if (!UNMASKED && (uint32_t)(j - jl) > span) p0 = 0.f;
-                        if (!UNMASKED && (uint32_t)(j + 1 - jl) > span) p1 = 0.f;
-                        const uint64_t ds2 = mul2(pack2(p0, p1), sub2(pack2(__uint_as_float(tv[j]), __uint_as_float(tv[j + 1])), D2));
-                        unpack2(ds2, ds0, ds1);
-                        unpack2(sub2(ds2, pack2(trunc19f(ds0), trunc19f(ds1))), l0, l1);
-                        sv[j] = __float_as_uint(ds0); sv[j + 1] = __float_as_uint(ds1);       // dS over S
-                        tv[j] = __float_as_uint(l0); tv[j + 1] = __float_as_uint(l1);         // dS_lo over T
+                    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+                        for (int j = 0; j < 16; j += 2) {
+                            float x0, x1, ds0, ds1, l0, l1;
+                            unpack2(fma2(pack2(__uint_as_float(sv[i][j]), __uint_as_float(sv[i][j + 1])), scale2, nbias2), x0, x1);
+                            float p0 = ex2f(x0), p1 = ex2f(x1);
+                            if (!UNMASKED && (uint32_t)(16 * i + j - jl) > span) p0 = 0.f;
+                            if (!UNMASKED && (uint32_t)(16 * i + j + 1 - jl) > span) p1 = 0.f;
+                            const uint64_t ds2 = mul2(pack2(p0, p1), sub2(pack2(__uint_as_float(tv[i][j]), __uint_as_float(tv[i][j + 1])), D2));
+                            unpack2(ds2, ds0, ds1);
+                            unpack2(sub2(ds2, pack2(trunc19f(ds0), trunc19f(ds1))), l0, l1);
+                            sv[i][j] = __float_as_uint(ds0); sv[i][j + 1] = __float_as_uint(ds1);       // dS over S
+                            tv[i][j] = __float_as_uint(l0); tv[i][j + 1] = __float_as_uint(l1);         // dS_lo over T
+                        }
+                        tm_st16(tS + 16 * i, sv[i]);
+                        tm_st16(tT + 16 * i, tv[i]);
                     }
                 };
                 if (full) elementwise(std::true_type{}); else elementwise(std::false_type{});
-                tm_st32(tS, sv);
-                tm_st32(tT, tv);
             }
             if (it > 0 && (it % FOLDQ == 0 || it == total)) {
                 // fold dS K of the blocks since the last fold (this half's two parts, fixed order): the tensor core has
