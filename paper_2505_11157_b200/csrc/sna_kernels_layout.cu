@@ -49,7 +49,8 @@ __global__ void __launch_bounds__(LT_THREADS) cf_to_cl_kernel(const float* __res
 // The same for channels in groups of 32 and planes of whole 16-byte pieces: a thread reads four channels of four points, turns them
 // round in registers, and hands them on through rows of eight 16-byte pieces, rotated so that neither side meets a bank conflict;
 // all accesses are 16 bytes, four in flight.  The tile above stores 4 bytes at a time to shared memory, four lanes to a bank.  A training
-// step on channels-first tensors (128x256, N = 16, C = 32, four transposes of 134 MB) took 1262 us with it, 1238 with this one.
+// step on channels-first tensors (128x256, N = 16, C = 32; four transposes of 134 MB) went from 1278 to 1238 us with this one and a dense
+// dk/dv kernel that takes 17 less.
 __global__ void __launch_bounds__(LT_THREADS) cf_to_cl_32_kernel(const float* __restrict__ src, float* __restrict__ dst, int C, long long P) {
     __shared__ float4 tile[128 * 8];      // [point][piece of four channels]
     const long long p0 = (long long)blockIdx.x * 128;
