@@ -111,6 +111,11 @@ __device__ __forceinline__ bool mb_wait_polls(uint32_t bar, uint32_t parity, int
 __device__ __forceinline__ bool mb_wait(uint32_t bar, uint32_t parity, bool healthy) {
     return mb_wait_polls(bar, parity, healthy ? WAIT2 : 4);
 }
+// A wait that has run out in one lane has run out for its warp: the element-wise warps go on to warp-collective instructions
+// (tcgen05.ld / st, votes) and must leave their loops as one.  They agree while their TMEM loads are in flight (64x128 global, N = 8, us,
+// without : with: forward 451 : 451, dq 498 : 500, dk/dv 875 : 885; directly after each wait dq takes 10 more).  The other roles
+// issue nothing collective.
+__device__ __forceinline__ bool all_lanes(bool ok) { return __all_sync(0xffffffffu, ok); }
 __device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int col, int ring, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                  ::"r"(dst), "l"(map), "r"(0), "r"(col), "r"(ring), "r"(bar) : "memory");
@@ -364,6 +369,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                 uint32_t oa[16], ob[16];
                 tm_ld16_issue(oa, tm + T_O + half * 64 + lanebits + c0);
                 tm_ld16_issue(ob, tm + T_O + half * 64 + 32 + lanebits + c0);
+                if (c0 == 0) ok = all_lanes(ok);
                 tm_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 16; j += 2)
@@ -392,6 +398,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                 uint32_t sq[4][16];
 #pragma unroll
                 for (int qd = 0; qd < 4; ++qd) tm_ld16_issue(sq[qd], tS + 16 * qd);
+                ok = all_lanes(ok);
                 tm_ld_wait();
                 float mxr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                 if (full) {
@@ -449,6 +456,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                     uint32_t sa[32], sb[32];
                     tm_ld32_issue(sa, tS);
                     tm_ld32_issue(sb, tS + 32);
+                    ok = all_lanes(ok);
                     tm_ld_wait();
                     if (full) {
 #pragma unroll
@@ -514,7 +522,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
             mb_arrive(s32(&bars[B_PREADY + 2 * half + b]));
             corr_prev = corr;
         }
-        if (total > 0) fold(total - 1);
+        if (total > 0 && ok) fold(total - 1);
         // merge the two column halves of every row: half 1 hands its state over through shared memory
         float* xs = reinterpret_cast<float*>(base + OFF_K);         // [34][128] floats in the k stages, which are dead by now
         if (half == 1) {
@@ -820,6 +828,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 uint32_t sv[2][16], tv[2][16];      // two pieces: the first is stored while the second is worked on (64x128, N = 8: 518 -> 500 us)
 #pragma unroll
                 for (int i = 0; i < 2; ++i) { tm_ld16_issue(sv[i], tS + 16 * i); tm_ld16_issue(tv[i], tT + 16 * i); }
+                ok = all_lanes(ok);
                 tm_ld_wait();
                 // (two instantiations: blocks in which no row of the warp is masked skip the per-element range test)
                 auto elementwise = [&](auto unmasked) {
@@ -855,6 +864,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 uint32_t oa[32], ob[32];
                 tm_ld32_issue(oa, tm + TQ_ACC + grp * 64 + lanebits);
                 tm_ld32_issue(ob, tm + TQ_ACC + grp * 64 + 32 + lanebits);
+                ok = all_lanes(ok);
                 tm_ld_wait();
 #pragma unroll
                 for (int j = 0; j < C2; j += 2)
@@ -1140,6 +1150,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 uint32_t oa[32], ob[32];
                 tm_ld32_issue(oa, tm + TK_ACC + grp * 32 + lanebits);          // dV, this column half
                 tm_ld32_issue(ob, tm + TK_ACC + 64 + grp * 32 + lanebits);     // dK, this column half
+                ok = all_lanes(ok);
                 tm_ld_wait();
 #pragma unroll
                 for (int j = 0; j < C2; j += 2) {
@@ -1176,6 +1187,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                         nlv[4 * q4] = a.x; nlv[4 * q4 + 1] = a.y; nlv[4 * q4 + 2] = a.z; nlv[4 * q4 + 3] = a.w;
                         Dv[4 * q4] = d4.x; Dv[4 * q4 + 1] = d4.y; Dv[4 * q4 + 2] = d4.z; Dv[4 * q4 + 3] = d4.w;
                     }
+                    ok = all_lanes(ok);
                     tm_ld_wait();
                     // (two instantiations: blocks in which no row of the warp is masked skip the per-element range test)
                     auto elementwise = [&](auto unmasked) {
@@ -1393,17 +1405,21 @@ cudaError_t dense2_prepare_device() {
     return e;
 }
 
-// The give-up path of the bounded waits, exercised without disturbing any real kernel: one thread waits, with the
-// production wait routine but only `polls` polls, on an mbarrier that nothing ever arrives on, then records the failure
-// in the plan's status word exactly as the dense kernels do, and returns normally.
+// The give-up path of the bounded waits, exercised without disturbing any real kernel: the last lane of a warp waits, with the
+// production wait routine but only `polls` polls, on an mbarrier that nothing ever arrives on, the other lanes on one that is
+// complete.  Its first lane, whose own wait is over at once, must hear of it: it records the failure in the plan's status word as the
+// dense kernels do, and the kernel returns normally.
 __global__ void bounded_wait_probe_kernel(int* dev_status, int polls) {
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bars[2];
     if (threadIdx.x == 0) {
-        mb_init(s32(&bar), 1);
+        mb_init(s32(&bars[0]), 1);
+        mb_init(s32(&bars[1]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const bool ok = mb_wait_polls(s32(&bar), 0, polls);
-        if (!ok) atomicExch(dev_status, 1);
+        mb_arrive(s32(&bars[0]));
     }
+    __syncthreads();
+    const bool ok = all_lanes(mb_wait_polls(s32(&bars[threadIdx.x == 31]), 0, polls));
+    if (threadIdx.x == 0 && !ok) atomicExch(dev_status, 1);
 }
 
 cudaError_t launch_bounded_wait_probe(const DevPlan& p, int polls, cudaStream_t stream) {
