@@ -80,6 +80,11 @@ enum { B_KFULL = 0, B_KCONV = 2, B_KFREE = 4, B_VFULL = 6, B_VRAWFREE = 8, B_VCO
 // the stage, which waits for the stage's FREE barriers, which the GEMM issuers signal after having waited for the full CONV
 // phase; an issuer commits to a buffer's DONE / STFULL barrier again only for a block whose operands-ready phase needs the
 // element-wise threads to have seen the previous use of that buffer complete.
+// The statistics warp of the dk/dv kernel, the third party to its QCONV barriers, waits for a stage's FREE barrier like the producer: the
+// issuers commit to that after QCONV's phase and after both groups' READY, by which time the statistics have been read into registers.
+// The element-wise threads read them after STFULL.  A commit orders tensor-core work, not another warp's ordinary stores, so the
+// issuer of S, which has waited for QCONV, arrives on STFULL itself as well, after the commit that reports its MMAs (64x128 global,
+// N = 8: 887 us without, 888 with it; a wait of the element-wise threads for QCONV costs 75 more).
 
 // Lets a band kernel that was launched to follow this one (its programmatic dependent) take the SMs that the last blocks leave idle.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -1078,7 +1083,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             mb_init(s32(&bars[K_FREE + s]), 6);         // both first GEMMs and the four second-GEMM issuers
         }
         for (int g = 0; g < 2; ++g) {
-            mb_init(s32(&bars[K_STFULL + g]), 2);            // buffer g: both first GEMMs
+            mb_init(s32(&bars[K_STFULL + g]), 3);            // buffer g: both first GEMMs, the statistics
             mb_init(s32(&bars[K_READY + 2 * g]), 128);       // group g, buffer 0
             mb_init(s32(&bars[K_READY + 2 * g + 1]), 128);   // group g, buffer 1
             mb_init(s32(&bars[K_G2DONE + 2 * g]), 2);        // group g, buffer 0: its dV and dK issuers
@@ -1168,7 +1173,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 const uint32_t span = (uint32_t)(jh - jl);
                 const bool full = __all_sync(0xffffffffu, jl <= 0 && jh >= GC - 1);     // no masking anywhere in this warp
                 wk.advance();
-                PROF_WAIT(0, ok = mb_wait(s32(&bars[K_STFULL + b]), (it >> 1) & 1, ok) && ok);     // implies QCONV of this stage (the S issuer waited for it)
+                PROF_WAIT(0, ok = mb_wait(s32(&bars[K_STFULL + b]), (it >> 1) & 1, ok) && ok);     // and the statistics of this stage (see the barrier list)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const float* nlc = reinterpret_cast<const float*>(base + s * KST + 8 * TILE_K) + grp * GC;
                 const float* Dc = nlc + BNK;
@@ -1300,6 +1305,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
 #pragma unroll
                 for (int ks = 0; ks < C2 / 8; ++ks) mma_ts(tD, tA + ks * 8, db + 2 * ks, idS, 1);
                 mma_commit(s32(&bars[K_STFULL + b]));
+                if (!isT) mb_arrive(s32(&bars[K_STFULL + b]));      // passes on what QCONV has ordered: the statistics
                 mma_commit(s32(&bars[K_FREE + s]));
             }
         }
