@@ -80,8 +80,9 @@ enum { B_KFULL = 0, B_KCONV = 2, B_KFREE = 4, B_VFULL = 6, B_VRAWFREE = 8, B_VCO
 // the stage, which waits for the stage's FREE barriers, which the GEMM issuers signal after having waited for the full CONV
 // phase; an issuer commits to a buffer's DONE / STFULL barrier again only for a block whose operands-ready phase needs the
 // element-wise threads to have seen the previous use of that buffer complete.
-// The statistics warp of the dk/dv kernel, the third party to its QCONV barriers, waits for a stage's FREE barrier like the producer: the
-// issuers commit to that after QCONV's phase and after both groups' READY, by which time the statistics have been read into registers.
+// The statistics warp of the dk/dv kernel, the third party to its QCONV barriers, waits for a stage's FREE barrier like the producer.  Of
+// the six commits that it takes, the S issuer's follows QCONV's phase, and those of the second GEMMs follow both groups' READY, by which
+// time the statistics have been read into registers.
 // The element-wise threads read them after STFULL.  A commit orders tensor-core work, not another warp's ordinary stores, so the
 // issuer of S, which has waited for QCONV, arrives on STFULL itself as well, after the commit that reports its MMAs (64x128 global,
 // N = 8: 887 us without, 888 with it; a wait of the element-wise threads for QCONV costs 75 more).
@@ -91,8 +92,9 @@ __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontro
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // One lane of a whole warp, for the MMAs that one thread issues.  (With lane 0 picked by comparison the compiler does not know that
 // one lane is left, and each tcgen05.mma takes 55 cycles to issue and the first eight of a batch 580, against 16 and 85.  It pays where
-// many short MMAs are issued: a first-GEMM issuer of the dk/dv kernel was busy 1250 of 1880 cycles per block, now 490 of 1690.  In the
-// forward kernel, whose 128-column MMAs keep the tensor core busy for 66 cycles each, it changes nothing: 499 : 502 us on 64x128, N = 8.)
+// many short MMAs are issued: 64x128 global, N = 8, dk/dv 971 : 880 us, a first-GEMM issuer busy 1250 of 1880 cycles per block before, 490 of
+// 1630 now.  The forward kernel does without: with it in the S issuer, whose 128-column MMAs keep the tensor core busy for 66 cycles each,
+// it takes 469 us instead of 457; in the P V issuers alone it would take 453.)
 __device__ __forceinline__ bool elect_one() {
     uint32_t r;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
@@ -1026,9 +1028,11 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
 //   dV += P dY,  dK += scale * dS Q   (A operands P, dS from TMEM; B operands: q and dout blocks transposed by the converters).
 // Two groups of 128 threads do the element-wise work for one half of the block's columns each and write P over S^T, dS
 // over T^T and the two lo parts beside them; one warp fetches the partner points' statistics, two groups of converters prepare the q and
-// the dout blocks (with one group for both, and that latency in it, the converters were busy 1600 of the 1880 cycles that a block took;
-// 64x128 global, N = 8: 1010 -> 883 us, 128x256, cutoff 4 rings, N = 16, with the band kernel: 476 -> 457); four threads issue the second GEMMs (dV or dK, one column half each) into
-// their own accumulators, which collect FOLDK blocks in TMEM before the row's threads fold them into registers.  TMEM:
+// the dout blocks; four threads issue the second GEMMs (dV or dK, one column half each) into their own accumulators, which collect FOLDK
+// blocks in TMEM before the row's threads fold them into registers.  (One group of converters for both arrays, with the statistics'
+// latency in it, was busy 1600 of the 1880 cycles that a block took.  64x128 global, N = 8: 1010 us then, 880 with the second group, the
+// statistics warp and the elected issuers; without the second group alone 950, without the statistics warp alone 952, without the
+// elected issuers alone 971.)  TMEM:
 // 128 columns of fixed operands, two buffers of 128 (S^T, T^T, P_lo, dS_lo of 32 columns each) and 128 of accumulators.
 // With two buffers the first GEMMs of block j+1 run while the element-wise threads work on block j and the second
 // GEMMs on block j-1 (blocks of 64 points leave room for one buffer only, which serialised the three phases); TMA and
@@ -1038,7 +1042,7 @@ constexpr int BNK = 32;                          // partner points per block
 constexpr int TILE_K = BNK * 128;                // 4 KB
 constexpr int FOLDK = 8;
 constexpr int NSK = 5;                           // shared-memory stages
-// per stage: q raw, q lo, y raw, y lo, q^T hi, q^T lo, y^T hi, y^T lo, then log2 omega - lse*log2e and D of the 64 partner points
+// per stage: q raw, q lo, y raw, y lo, q^T hi, q^T lo, y^T hi, y^T lo, then log2 omega - lse*log2e and D of the 32 partner points
 constexpr int KST = 8 * TILE_K + 1024;
 constexpr size_t DKDV2_SMEM = NSK * KST + 1024;
 constexpr int TK_AK = 0, TK_AKL = 32, TK_AV = 64, TK_AVL = 96, TK_BUF = 128 /* + 128 b: S | T | P_lo | dS_lo, 32 columns each */, TK_ACC = 384 /* + 32 part */;
@@ -1272,6 +1276,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
         if (warp == 11) {
             // -------------------------------------------------------------- the partner points' statistics, up to NSK blocks ahead
             TileWalk wk(p.t_dense_lat, p.t_dense_m, e_begin, e_end, p.nlon_out, BNK, a_lo, a_hi, p.ps);
+            static_assert(BNK == 32, "one partner point per lane");
             for (int it = 0; it < total && ok; ++it, wk.advance()) {
                 const int s = it % NSK, u = it / NSK;
                 if (u > 0) ok = mb_wait(s32(&bars[K_FREE + s]), (u - 1) & 1, ok);
@@ -1437,11 +1442,13 @@ bool dense2_path_chosen(const DevPlan& p, int C, int N) {
     if (C != C2 || p.dense_ptr == nullptr || p.n_dense_rows == 0 || p.dense_all || !band_path_supported(p, C) || encode_fn2() == nullptr) return false;
     // One block per SM walks a tile's list, so the dense kernel takes at least the longest list's time, in which the band kernel fills
     // only the SMs that it leaves idle; with too little work per SM the band kernels alone, which share long streams between warps,
-    // are faster.  Measured (fwd / dq / dkdv us, with : without the dense kernels; work in longest lists per SM): 128x256, cutoff 4
-    // rings, N = 1 (0.1) 57/62/80 : 32/36/40, N = 4 (0.39) 97/113/150 : 88/108/123, N = 8 (0.8) 161/184/224 : 168/200/233, N = 16
-    // 307/353/439 : 329/389/456; 10 rings, N = 2 (0.47) 159/172/216 : 147/176/213; 256x512 -> 128x256 N = 4 (0.44) 196/212/272 :
-    // 208/246/280; 361x720 N = 1 (0.6) 237/253/321 : 254/298/352.
-    // The second bound is the fixed cost of another kernel: 32x64, N = 32 (0.9 lists of 3 blocks) 49/52/55 : 36/41/39.
+    // are faster.  Measured (fwd / dq / dkdv us, with : without the dense kernels; in brackets the work in longest lists per SM):
+    // 128x256, cutoff 4 rings, N = 1 (0.1) 44/40/54 : 38/41/47, N = 2 (0.2) 85/70/71 : 59/68/78, N = 4 (0.39) 101/106/126 : 103/119/137,
+    // N = 8 (0.8) 169/191/234 : 182/211/254, N = 16 316/365/454 : 344/404/492; 10 rings, N = 2 (0.47) 185/185/222 : 171/190/234;
+    // 256x512 -> 128x256 N = 2 (0.22) 183/136/148 : 121/139/160, N = 4 (0.44) 204/220/286 : 226/258/307; 361x720 N = 1 (0.6)
+    // 230/251/316 : 252/289/352.  (N = 4 of the first grid, on the line, would gain by 2 to 12 % now; the line was drawn at 97/113/150 :
+    // 88/108/123.)  The second bound is the fixed cost of another kernel: 32x64, N = 32 (0.9 lists of 3 blocks) 48/48/54 : 43/49/47.  It lies
+    // too low for lists that short: N = 128, past it, takes 140/154/177 : 108/127/150.
     const long long work = (long long)((p.nlon_out + M2 - 1) / M2) * N * p.dense_blocks;
     return work * 10 >= p.num_sms * 4LL * p.dense_longest && work >= p.num_sms * 6LL;
 }
@@ -1457,8 +1464,12 @@ bool dense2_global_chosen(const DevPlan& p, int C, int N, Pass pass) {
     // Both sides are a number of equal units of work of known duration (us).  Dense: each block walks all rings of the other grid in
     // units of `unit` columns, one block per SM at a time; rings that are no multiple of the unit leave it partly empty, and the
     // forward kernel masks then.  Band: 256 pairs per unit over the whole GPU.  Measured dense : band, fwd / dq / dkdv:
-    // 24x48 N = 4 73/38/57 : 21/23/23, 32x64 N = 16 339/170/277 : 149/165/196, 51x102 N = 4 263/224/402 : 242/287/342,
-    // 64x128 N = 1 131/132/255 : 154/182/230, N = 4 251/262/504 : 511/609/732, 90x180 N = 1 859/573/1047 : 502/597/739.
+    // 24x48 N = 4 64/39/57 : 29/29/29, 32x64 N = 16 285/170/264 : 162/176/217, 51x102 N = 4 223/223/375 : 268/299/377,
+    // 64x128 N = 1 119/131/230 : 174/187/264, N = 4 234/258/455 : 559/627/797, 80x160 N = 4 1626/1210/1737 : 1323/1481/1907,
+    // 90x180 N = 1 737/551/942 : 623/623/813, N = 2 1122/830/1412 : 1130/1227/1540.
+    // The durations are those of slower dense kernels: a unit takes 1.85, with masks 2.0 to 2.2, in dq 1.0 to 1.1, in dk/dv 0.87 to 0.94 of
+    // the present ones.  So the line is on the safe side: of the problems above the forward pass of 51x102 and of 90x180, N = 2, and dk/dv
+    // of 64x128, N = 1, 80x160 and 90x180, N = 2, stay on the band kernels although the dense ones are faster.
     const bool whole = p.nlon_in % M2 == 0 && p.nlon_out % M2 == 0;
     const int unit = pass == Pass::FORWARD ? 128 : pass == Pass::DQ ? 64 : 32;
     const double dense_unit = pass == Pass::FORWARD ? (whole ? 2.0 : 2.7) : pass == Pass::DQ ? 1.05 : 1.0;

@@ -14,7 +14,8 @@ constexpr int LT_MAXC = 128;
 constexpr int LT_WORDS = 64 * 129;      // shared tile: 64 channels x 128 points, or 128 channels x 32 points (pitch + 1)
 
 // Tiles of PTS points x C channels; PTS = 128 (each lane moves 16 bytes along the points) when C <= 64 and the planes are
-// 16-byte aligned (P % 4 == 0), else PTS = 32 with 4-byte accesses on the channels-first side.
+// 16-byte aligned (P % 4 == 0), else PTS = 32 with 4-byte accesses on the channels-first side.  To channels last, groups of 32 channels
+// of such planes take cf_to_cl_32_kernel below.
 // src: [slices][C][P] (channels first), dst: [slices][P][C] (channels last)
 template <int PTS>
 __global__ void __launch_bounds__(LT_THREADS) cf_to_cl_kernel(const float* __restrict__ src, float* __restrict__ dst, int C, long long P) {
