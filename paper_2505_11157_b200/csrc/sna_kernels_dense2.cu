@@ -92,9 +92,9 @@ __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontro
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // One lane of a whole warp, for the MMAs that one thread issues.  (With lane 0 picked by comparison the compiler does not know that
 // one lane is left, and each tcgen05.mma takes 55 cycles to issue and the first eight of a batch 580, against 16 and 85.  It pays where
-// many short MMAs are issued: 64x128 global, N = 8, dk/dv 971 : 880 us, a first-GEMM issuer busy 1250 of 1880 cycles per block before, 490 of
-// 1630 now.  The forward kernel does without: with it in the S issuer, whose 128-column MMAs keep the tensor core busy for 66 cycles each,
-// it takes 469 us instead of 457; in the P V issuers alone it would take 453.)
+// many short MMAs are issued: 64x128 global, N = 8, dk/dv 971 : 880 us, a first-GEMM issuer busy 1230 of 1880 cycles per block before, 490 of
+// 1630 now.  The forward kernel does without, at 457 us: with it in the P V issuers it would take 453, in the S issuer as well, whose
+// 128-column MMAs keep the tensor core busy for 66 cycles each, 469.)
 __device__ __forceinline__ bool elect_one() {
     uint32_t r;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
