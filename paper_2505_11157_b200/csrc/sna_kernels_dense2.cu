@@ -24,7 +24,7 @@
 // While the softmax threads work on block j, the tensor core computes S of block j+1 and P V of block j-1, TMA loads block
 // j+2 and the converters prepare block j+1.  Every accumulator has exactly one issuing thread and all sums are taken in a
 // fixed order, so results are reproducible bit for bit.  Every wait is bounded; a wait that runs out sets the plan's
-// device status word and the block leaves.
+// device status word and the block leaves, after another bounded wait for the copies and MMAs that it has under way.
 #include <cuda.h>
 
 #include "sna_kernels.cuh"
@@ -385,7 +385,8 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                             o[c0 + j], o[c0 + j + 1]);
             }
         };
-        for (int it = 0; it < total && ok; ++it) {
+        int it = 0;
+        for (; it < total && ok; ++it) {
             float corr = 1.f;
             const int b = it & 1, u = it >> 1;
             const float bias = p.log2_omega[wk.ring];
@@ -530,6 +531,8 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
             corr_prev = corr;
         }
         if (total > 0 && ok) fold(total - 1);
+        else if (it > 0) mb_wait_polls(s32(&bars[B_PVDONE + 2 * half + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2);      // P V under way
+        // (here for the P V issuers too: a wait at the end of theirs cost 1 %, 451 : 455 us on 64x128 global, N = 8)
         // merge the two column halves of every row: half 1 hands its state over through shared memory
         float* xs = reinterpret_cast<float*>(base + OFF_K);         // [34][128] floats in the k stages, which are dead by now
         if (half == 1) {
@@ -563,7 +566,8 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
             mb_expect(s32(&bars[B_QFULL]), TILE_B);
             tma_tile(sbase + OFF_Q, &map_q, w0, n * p.nlat_out + h, s32(&bars[B_QFULL]));
             TileWalk wk(p.dense_lat, p.dense_m, e_begin, e_end, p.nlon_in, BN2, a_lo, a_hi, 1);
-            for (int it = 0; it < total && ok; ++it, wk.advance()) {
+            int it = 0;
+            for (; it < total && ok; ++it, wk.advance()) {
                 const int s = it & 1, u = it >> 1;
                 const int hp = wk.ring;
                 const int c0 = wk.col();
@@ -571,10 +575,16 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                     ok = mb_wait(s32(&bars[B_KFREE + s]), (u - 1) & 1, ok);
                     ok = mb_wait(s32(&bars[B_VRAWFREE + s]), (u - 1) & 1, ok) && ok;
                 }
+                if (!ok) break;
                 mb_expect(s32(&bars[B_KFULL + s]), TILE_B);
                 tma_tile(sbase + OFF_K + s * 2 * TILE_B, &map_k, c0, n * p.nlat_in + hp, s32(&bars[B_KFULL + s]));
                 mb_expect(s32(&bars[B_VFULL + s]), TILE_B);
                 tma_tile(sbase + OFF_VRAW + s * TILE_B, &map_v, c0, n * p.nlat_in + hp, s32(&bars[B_VFULL + s]));
+            }
+            ok = mb_wait_polls(s32(&bars[B_QFULL]), 0, WAIT2) && ok;
+            for (int j = max(0, it - 2); j < it; ++j) {      // the copies under way
+                ok = mb_wait_polls(s32(&bars[B_KFULL + j % 2]), (j / 2) & 1, WAIT2) && ok;
+                ok = mb_wait_polls(s32(&bars[B_VFULL + j % 2]), (j / 2) & 1, WAIT2) && ok;
             }
         }
         // ------------------------------------------------------------------ S = Q K^T
@@ -583,7 +593,8 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
             // q_lo is written by the converter warps before their first k tile: covered by KCONV of block 0
             const uint32_t idS = idesc_tf32(BN2);
             const uint64_t dq = desc_k(sbase + OFF_Q), dql = desc_k(sbase + OFF_QLO);
-            for (int it = 0; it < total && ok; ++it) {
+            int it = 0;
+            for (; it < total && ok; ++it) {
                 const int s = it & 1, u = it >> 1;
                 ok = mb_wait(s32(&bars[B_KFULL + s]), u & 1, ok);
                 ok = mb_wait(s32(&bars[B_KCONV + s]), u & 1, ok) && ok;
@@ -603,6 +614,7 @@ forward_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q, cons
                 mma_commit(s32(&bars[B_SFULL + s]));
                 mma_commit(s32(&bars[B_KFREE + s]));
             }
+            if (it > 0) ok = mb_wait_polls(s32(&bars[B_SFULL + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2) && ok;      // the MMAs under way
         }
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -909,7 +921,8 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
         if (warp == 8 && lane == 0) {
             // -------------------------------------------------------------- TMA producer
             TileWalk wk(p.dense_lat, p.dense_m, e_begin, e_end, p.nlon_in, BNQ, a_lo, a_hi, 1);
-            for (int it = 0; it < total && ok; ++it, wk.advance()) {
+            int it = 0;
+            for (; it < total && ok; ++it, wk.advance()) {
                 const int s = it % NSQ, u = it / NSQ;
                 const int hp = wk.ring;
                 const int c0 = wk.col();
@@ -918,10 +931,15 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                     PROF_WAIT(1, ok = mb_wait(s32(&bars[Q_VFREE + s]), (u - 1) & 1, ok) && ok);
                     PROF_WAIT(2, ok = mb_wait(s32(&bars[Q_KTFREE + s]), (u - 1) & 1, ok) && ok);
                 }
+                if (!ok) break;
                 mb_expect(s32(&bars[Q_KFULL + s]), TILE_Q);
                 tma_tile(sbase + s * QST, &map_k, c0, n * p.nlat_in + hp, s32(&bars[Q_KFULL + s]));
                 mb_expect(s32(&bars[Q_VFULL + s]), TILE_Q);
                 tma_tile(sbase + s * QST + 2 * TILE_Q, &map_v, c0, n * p.nlat_in + hp, s32(&bars[Q_VFULL + s]));
+            }
+            for (int j = max(0, it - NSQ); j < it; ++j) {      // the copies under way
+                ok = mb_wait_polls(s32(&bars[Q_KFULL + j % NSQ]), (j / NSQ) & 1, WAIT2) && ok;
+                ok = mb_wait_polls(s32(&bars[Q_VFULL + j % NSQ]), (j / NSQ) & 1, WAIT2) && ok;
             }
         }
         if ((warp == 9 || warp == 10) && elect_one()) {
@@ -930,7 +948,8 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
             ok = mb_wait(s32(&bars[Q_AREADY]), 0, ok);
             const uint32_t idS = idesc_tf32(BNQ), idS16 = idesc_bf16(BNQ);
             const uint32_t tA = tm + (isT ? TQ_AY : TQ_AQ), tAl = tm + (isT ? TQ_AYL : TQ_AQL);
-            for (int it = 0; it < total && ok; ++it) {
+            int it = 0;
+            for (; it < total && ok; ++it) {
                 const int s = it % NSQ, us = it / NSQ, b = it & 1, u = it >> 1;
                 PROF_WAIT(0, ok = mb_wait(s32(&bars[(isT ? Q_VFULL : Q_KFULL) + s]), us & 1, ok));
                 PROF_WAIT(1, ok = mb_wait(s32(&bars[(isT ? Q_VCONV : Q_KCONV) + s]), us & 1, ok) && ok);
@@ -949,6 +968,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 mma_commit(s32(&bars[Q_STFULL + b]));
                 mma_commit(s32(&bars[(isT ? Q_VFREE : Q_KSFREE) + s]));
             }
+            if (it > 0) ok = mb_wait_polls(s32(&bars[Q_STFULL + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2) && ok;      // the MMAs under way
         }
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -957,7 +977,8 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
             const int part = warp - 12, grp = part >> 1;
             const uint32_t idO = idesc_tf32(C2);
             const uint32_t tO = tm + TQ_ACC + part * 32;
-            for (int it = 0; it < total && ok; ++it) {
+            int it = 0;
+            for (; it < total && ok; ++it) {
                 const int s = it % NSQ, us = it / NSQ, b = it & 1;
                 PROF_WAIT(0, ok = mb_wait(s32(&bars[Q_KCONV + s]), us & 1, ok));
                 PROF_WAIT(1, ok = mb_wait(s32(&bars[Q_DSREADY + 2 * grp + b]), (it >> 1) & 1, ok) && ok);
@@ -976,6 +997,7 @@ backward_dq_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_k, 
                 mma_commit(s32(&bars[Q_G2DONE + 2 * grp + b]));
                 mma_commit(s32(&bars[Q_KTFREE + s]));
             }
+            if (it > 0) ok = mb_wait_polls(s32(&bars[Q_G2DONE + 2 * grp + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2) && ok;      // the MMAs under way
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
@@ -1262,15 +1284,21 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
         if (warp == 8 && lane == 0) {
             // -------------------------------------------------------------- TMA producer: q and dout blocks of the partner rings
             TileWalk wk(p.t_dense_lat, p.t_dense_m, e_begin, e_end, p.nlon_out, BNK, a_lo, a_hi, p.ps);
-            for (int it = 0; it < total && ok; ++it, wk.advance()) {
+            int it = 0;
+            for (; it < total && ok; ++it, wk.advance()) {
                 const int s = it % NSK, u = it / NSK;
                 const int h = wk.ring;
                 const int w0 = wk.col();
                 if (u > 0) PROF_WAIT(0, ok = mb_wait(s32(&bars[K_FREE + s]), (u - 1) & 1, ok));
+                if (!ok) break;
                 mb_expect(s32(&bars[K_QFULL + s]), TILE_K);
                 tma_tile(sbase + s * KST, &map_q, w0, n * p.nlat_out + h, s32(&bars[K_QFULL + s]));
                 mb_expect(s32(&bars[K_YFULL + s]), TILE_K);
                 tma_tile(sbase + s * KST + 2 * TILE_K, &map_y, w0, n * p.nlat_out + h, s32(&bars[K_YFULL + s]));
+            }
+            for (int j = max(0, it - NSK); j < it; ++j) {      // the copies under way
+                ok = mb_wait_polls(s32(&bars[K_QFULL + j % NSK]), (j / NSK) & 1, WAIT2) && ok;
+                ok = mb_wait_polls(s32(&bars[K_YFULL + j % NSK]), (j / NSK) & 1, WAIT2) && ok;
             }
         }
         if (warp == 11) {
@@ -1293,7 +1321,8 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             ok = mb_wait(s32(&bars[K_AREADY]), 0, ok);
             const uint32_t idS = idesc_tf32(BNK), idS16 = idesc_bf16(BNK);
             const uint32_t tA = tm + (isT ? TK_AV : TK_AK), tAl = tm + (isT ? TK_AVL : TK_AKL);
-            for (int it = 0; it < total && ok; ++it) {
+            int it = 0;
+            for (; it < total && ok; ++it) {
                 const int s = it % NSK, us = it / NSK, b = it & 1, u = it >> 1;
                 PROF_WAIT(0, ok = mb_wait(s32(&bars[(isT ? K_YFULL : K_QFULL) + s]), us & 1, ok));
                 PROF_WAIT(1, ok = mb_wait(s32(&bars[(isT ? K_YCONV : K_QCONV) + s]), us & 1, ok) && ok);
@@ -1313,6 +1342,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 if (!isT) mb_arrive(s32(&bars[K_STFULL + b]));      // passes on what QCONV has ordered: the statistics
                 mma_commit(s32(&bars[K_FREE + s]));
             }
+            if (it > 0) ok = mb_wait_polls(s32(&bars[K_STFULL + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2) && ok;      // the MMAs under way
         }
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
@@ -1321,7 +1351,8 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
             const int part = warp - 12, kind = part >> 1, grp = part & 1;      // kind 0: dV = P dY, kind 1: dK = dS Q
             const uint32_t idO = idesc_tf32(C2);
             const uint32_t tO = tm + TK_ACC + part * 32;
-            for (int it = 0; it < total && ok; ++it) {
+            int it = 0;
+            for (; it < total && ok; ++it) {
                 const int s = it % NSK, us = it / NSK, b = it & 1;
                 const uint32_t tA = tm + TK_BUF + 128 * b + (kind ? TK_T : TK_S), tAl = tm + TK_BUF + 128 * b + (kind ? TK_DSLO : TK_PLO);
                 PROF_WAIT(0, ok = mb_wait(s32(&bars[(kind ? K_QCONV : K_YCONV) + s]), us & 1, ok));
@@ -1340,6 +1371,7 @@ backward_dkdv_dense2_kernel(DevPlan p, const __grid_constant__ CUtensorMap map_q
                 mma_commit(s32(&bars[K_G2DONE + 2 * grp + b]));
                 mma_commit(s32(&bars[K_FREE + s]));
             }
+            if (it > 0) ok = mb_wait_polls(s32(&bars[K_G2DONE + 2 * grp + ((it - 1) & 1)]), ((it - 1) >> 1) & 1, WAIT2) && ok;      // the MMAs under way
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
